@@ -94,6 +94,14 @@ __device__ __forceinline__ float2 czero() { return make_float2(0.f, 0.f); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// 16-byte asynchronous copies into shared memory (both addresses 16-byte aligned).
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 __device__ __forceinline__ float2 gather_obj(const float2* __restrict__ z, int n_rows, int n_cols,
                                              int gr, int gc) {
   if ((unsigned)gr < (unsigned)n_rows && (unsigned)gc < (unsigned)n_cols)
@@ -917,6 +925,39 @@ struct CTile {
   static constexpr int SLOTS = H * N2 / NT;    // column pass-B slots per thread
   static constexpr size_t smem_elems = (size_t)H * SR + (size_t)M * SC + (size_t)H * M;
   static_assert(H * M % NT == 0 && H * N2 % NT == 0 && NT <= 1024, "slab must split evenly");
+  static_assert(H % N1 == 0, "the outputs of one pass-B slot go to one CTA");
+};
+
+// Shared memory of the step kernel.  A slab holds H lines of M elements (stride
+// SR): my patch rows, or my storage columns, each line contiguous along the
+// direction it is transformed in.
+//
+// ONE = false (m <= 128): a row slab, a column slab (later the multigrid
+// buffers) and z_k on my rows.
+// ONE = true (m = 256): one slab, overwritten in place by the transposes, and
+// a second area that holds a_k on my storage columns during the transforms
+// and the multigrid buffers after them; z_k is read again from L2 where the
+// multigrid and the update need it.  199 KB per CTA with three slabs leave
+// one CTA of 16 warps per SM and at most 15 clusters of 8 on the device (120
+// SMs); 114 KB let two CTAs share an SM and hide each other's barriers.
+template <int M, int C>
+struct StepTile : CTile<M, C> {
+  using B = CTile<M, C>;
+  static constexpr bool ONE = M == 256;
+  static constexpr int S = B::SR;
+  // CTAs per SM the register budget leaves room for (as many as the shared memory does)
+  static constexpr int MIN_CTAS = ONE ? 2 : M == 128 ? C / 2 : 1;
+  static constexpr size_t slab = (size_t)B::H * S;
+  // multigrid buffers of every level at which each CTA keeps a row
+  static constexpr size_t mg_elems() {
+    size_t n = 0;
+    for (int w = M / 2; w >= C && w >= 2; w /= 2) n += (size_t)(2 * (w / C) + 2) * (w + 1);
+    return n;
+  }
+  static constexpr size_t amp_elems = (size_t)B::H * M / 2;  // floats, counted in float2
+  static constexpr size_t aux = mg_elems() > amp_elems ? mg_elems() : amp_elems;
+  static constexpr size_t smem_elems = ONE ? slab + aux : 2 * slab + (size_t)B::H * M;
+  static_assert(ONE || mg_elems() <= slab, "the multigrid buffers reuse the column slab");
 };
 
 // Row slab (after the row passes) -> column slabs of all C CTAs.
@@ -940,6 +981,62 @@ __device__ __forceinline__ void cluster_cols_to_rows(cg::cluster_group& cl, int 
     const int r = s / T::H, lc = s % T::H, d = r / T::H;
     float2* dst = d == rank ? rowbuf : cl.map_shared_rank(rowbuf, d);
     dst[(r % T::H) * T::SR + rank * T::H + lc] = colbuf[r * T::SC + lc];
+  }
+}
+
+// Row pass B on my row slab, its outputs stored straight into the column slabs
+// of all C CTAs (the transpose costs no pass of its own).  Lanes take
+// consecutive rows, which are consecutive elements of a column line, so each
+// store of a warp is one contiguous run.  With one slab per CTA the outputs wait in
+// registers until every CTA of the cluster has read its slab.  The caller's
+// cluster barrier makes the columns visible.
+template <int M, int C>
+__device__ __forceinline__ void row_pass_b_to_cols(cg::cluster_group& cl, int rank, const float2* rowbuf,
+                                                   float2* colbuf, int tid) {
+  using T = StepTile<M, C>;
+  float2 v[T::SLOTS][T::N1];
+  auto put = [&](int t) {
+    const int s = tid + t * T::NT, e0 = T::N1 * (s / T::H), line = s % T::H, d = e0 / T::H;
+    float2* dst = (d == rank ? colbuf : cl.map_shared_rank(colbuf, d)) + (e0 % T::H) * T::S + rank * T::H + line;
+#pragma unroll
+    for (int i = 0; i < T::N1; ++i) dst[i * T::S] = v[t][i];
+  };
+#pragma unroll
+  for (int t = 0; t < T::SLOTS; ++t) {
+    const int s = tid + t * T::NT;
+    const float2* p = rowbuf + (s % T::H) * T::S + T::N1 * (s / T::H);
+#pragma unroll
+    for (int i = 0; i < T::N1; ++i) v[t][i] = p[i];
+    Dft<T::N1, false>::run(v[t]);
+    if constexpr (!T::ONE) put(t);
+  }
+  if constexpr (T::ONE) {
+    cl.sync();
+#pragma unroll
+    for (int t = 0; t < T::SLOTS; ++t) put(t);
+  }
+}
+
+// Inverse column pass A on my column slab, its outputs (natural rows) stored
+// straight into the row slabs of all C CTAs; lanes take consecutive columns,
+// so each store of a warp is one contiguous run of a row.
+template <int M, int C>
+__device__ __forceinline__ void col_pass_a_inv_to_rows(cg::cluster_group& cl, int rank, const float2* colbuf,
+                                                       float2* rowbuf, int tid) {
+  using T = StepTile<M, C>;
+  const int j = tid / T::H, line = tid % T::H;
+  const float2* p = colbuf + line * T::S + j;
+  float2 v[T::N2];
+#pragma unroll
+  for (int k2 = 0; k2 < T::N2; ++k2) v[k2] = p[T::N1 * k2];
+#pragma unroll
+  for (int k2 = 1; k2 < T::N2; ++k2) v[k2] = cmulc(v[k2], stage_twiddle<M>(j, k2));
+  Dft<T::N2, true>::run(v);
+  if constexpr (T::ONE) cl.sync();
+#pragma unroll
+  for (int n2 = 0; n2 < T::N2; ++n2) {
+    const int d = T::N1 * n2 / T::H, lr = T::N1 * n2 % T::H + j;
+    (d == rank ? rowbuf : cl.map_shared_rank(rowbuf, d))[lr * T::S + rank * T::H + line] = v[n2];
   }
 }
 
@@ -978,16 +1075,19 @@ __device__ __forceinline__ void push_halo(cg::cluster_group& cl, int rank, T* y,
 // tensor-core DFT pair (a2-a4 done elsewhere); the kernel gathers z_k and runs
 // a5-a7 only.
 template <int M, int C, bool RIN = false>
-__global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) {
-  using TL = CTile<M, C>;
-  constexpr int NT = TL::NT, H = TL::H, SR = TL::SR, SC = TL::SC;
+__global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) k_stepc(const StepArgs a) {
+  using TL = StepTile<M, C>;
+  constexpr bool ONE = TL::ONE;
+  constexpr int NT = TL::NT, H = TL::H, SR = TL::S;
   constexpr int N1 = TL::N1, N2 = TL::N2, PER = TL::PER, SLOTS = TL::SLOTS;
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank();
   extern __shared__ __align__(16) float2 sm[];  // 16-byte aligned: the update pass reads pixel pairs
-  float2* rowbuf = sm;                     // H x SR: my patch rows
-  float2* colbuf = sm + H * SR;            // M x SC: my storage columns (all rows); multigrid buffers later
-  float2* zbuf = colbuf + M * SC;          // H x M: z_k on my rows (gathered once)
+  float2* rowbuf = sm;                                        // my patch rows
+  float2* colbuf = ONE ? sm : sm + TL::slab;                  // my storage columns (all rows)
+  float2* mgbuf = ONE ? sm + TL::slab : colbuf;               // multigrid buffers, after the transforms
+  float* ampbuf = reinterpret_cast<float*>(sm + TL::slab);    // ONE: a_k on my columns, [M][H], before them
+  float2* zbuf = sm + 2 * TL::slab;                           // !ONE: H x M, z_k on my rows (gathered once)
   __shared__ float xf[C];
   __shared__ double xd[C], xd2[C];
   __shared__ double redd[2];
@@ -1027,18 +1127,32 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
   const int row0 = rank * H;
 
   // amplitudes of my spectral slots: issued now, consumed after the row passes
-  float am_reg[SLOTS][N1];
+  float am_reg[ONE ? 1 : SLOTS][ONE ? 1 : N1];
   if constexpr (!RIN) {
     const float* amp = a.amp + (size_t)k * M * M + rank * H;
+    if constexpr (ONE) {
 #pragma unroll
-    for (int t = 0; t < SLOTS; ++t) {
-      const int s = tid + t * NT, k2 = s / H, lc = s % H;
+      for (int q = tid; q < M * H / 4; q += NT)
+        cp_async16(ampbuf + 4 * q, amp + (q / (H / 4)) * M + 4 * (q % (H / 4)));
+      cp_async_commit();
+    } else {
 #pragma unroll
-      for (int i = 0; i < N1; ++i) am_reg[t][i] = __ldg(amp + (i + N1 * k2) * M + lc);
+      for (int t = 0; t < SLOTS; ++t) {
+        const int s = tid + t * NT, k2 = s / H, lc = s % H;
+#pragma unroll
+        for (int i = 0; i < N1; ++i) am_reg[t][i] = __ldg(amp + (i + N1 * k2) * M + lc);
+      }
     }
   }
   pdl_trigger();
   pdl_wait();  // object, probe, max|Q|^2 and level arrays come from earlier kernels
+  // z_k at my local row lr, column c: the kept copy, or the object (0 outside)
+  auto z_at = [&](int lr, int c) -> float2 {
+    if constexpr (ONE)
+      return gather_obj(a.object, a.n_rows, a.n_cols, o_r + row0 + lr, o_c + c);
+    else
+      return zbuf[lr * M + c];
+  };
   const float MQ = __uint_as_float(*a.mq);
   cluster_arrive_relaxed();  // completed (wait) before the first distributed shared memory access
 
@@ -1056,7 +1170,7 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
     const int p = tid + t * NT;
     const int lr = p / M, c = p % M, r = row0 + lr;
     const float2 zk = gather_obj(a.object, a.n_rows, a.n_cols, o_r + r, o_c + c);
-    zbuf[p] = zk;
+    if constexpr (!ONE) zbuf[p] = zk;
     if constexpr (RIN)
       rowbuf[lr * SR + c] = a.r_in[(size_t)kb * M * M + r * M + c];
     else
@@ -1067,15 +1181,14 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
   warp_partial_max(mu_l, redf);
   __syncthreads();
   if constexpr (!RIN) {
-    // a2: row passes on my rows
+    // a2: row pass A on my rows
     gpass_a_fwd<M, H, SR, 1, NT>(rowbuf, tid);
-    __syncthreads();
-    gpass_b<M, H, SR, 1, NT, false>(rowbuf, tid);
+    if constexpr (ONE) cp_async_wait_all();  // a_k; the barriers below show it to the whole CTA
     __syncthreads();
   }
   cl.barrier_wait();  // all CTAs of the cluster resident
-  // transpose 1: my rows x all storage columns -> column slabs
-  if constexpr (!RIN) cluster_rows_to_cols<M, C>(cl, rank, rowbuf, colbuf, tid);
+  // row pass B, outputs to the column slabs
+  if constexpr (!RIN) row_pass_b_to_cols<M, C>(cl, rank, rowbuf, colbuf, tid);
   if (tid == 0) cluster_publish<C>(cl, rank, xf, partials_max<NT>(redf));
   cl.sync();
   float mu = xf[0];
@@ -1084,20 +1197,25 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
 
   if constexpr (!RIN) {
   // a2 (columns) + a3 + a4 (columns) on my storage columns
-  gpass_a_fwd<M, H, 1, SC, NT>(colbuf, tid);
+  gpass_a_fwd<M, H, SR, 1, NT>(colbuf, tid);
   __syncthreads();
   const float inv_m2 = 1.f / (float)(M * M);
   float acc = 0.f;
 #pragma unroll
   for (int t = 0; t < SLOTS; ++t) {
     const int s = tid + t * NT, k2 = s / H, lc = s % H;
+    float2* p = colbuf + lc * SR + N1 * k2;
     float2 v[N1];
 #pragma unroll
-    for (int i = 0; i < N1; ++i) v[i] = colbuf[(i + N1 * k2) * SC + lc];
+    for (int i = 0; i < N1; ++i) v[i] = p[i];
     Dft<N1, false>::run(v);
 #pragma unroll
     for (int i = 0; i < N1; ++i) {
-      const float am = am_reg[t][i];
+      float am;
+      if constexpr (ONE)
+        am = ampbuf[(i + N1 * k2) * H + lc];
+      else
+        am = am_reg[t][i];
       const float p2 = cabs2(v[i]);
       if (p2 > 0.f) {
         const float inv = rsqrtf(p2);
@@ -1111,15 +1229,13 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
     }
     Dft<N1, true>::run(v);
 #pragma unroll
-    for (int i = 0; i < N1; ++i) colbuf[(i + N1 * k2) * SC + lc] = v[i];
+    for (int i = 0; i < N1; ++i) p[i] = v[i];
   }
-  __syncthreads();
-  gpass_a_inv<M, H, 1, SC, NT>(colbuf, tid);
-  // per-warp misfit partials; the barrier also orders the pass before the transpose
+  // per-warp misfit partials; the barrier also orders the pass before the next one
   warp_partial_sum(acc, redf);
   __syncthreads();
-  // transpose 2: all rows x my columns -> row slabs
-  cluster_cols_to_rows<M, C>(cl, rank, colbuf, rowbuf, tid);
+  // inverse column pass A, outputs to the row slabs
+  col_pass_a_inv_to_rows<M, C>(cl, rank, colbuf, rowbuf, tid);
   if (tid == 0) cluster_publish<C>(cl, rank, xd, partials_sum<NT>(redf));
   cl.sync();
   // a4: inverse row passes -> R (natural order) on my rows
@@ -1144,7 +1260,7 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
       __syncthreads();
     }
   }
-  // a5: MAGPIE multigrid on row slabs; level-l buffers (l >= 1) reuse colbuf.
+  // a5: MAGPIE multigrid on row slabs; level-l buffers (l >= 1) in mgbuf.
   // Z_l keeps one halo row above and below my rows for the prolongation.
   float2* Zl[kMaxLevels];
   float2* Rl[kMaxLevels];
@@ -1152,9 +1268,9 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
     size_t off = 0;
     for (int l = 1; l < a.levels; ++l) {
       const int wl = M >> l, hl = wl / C, sl = wl + 1;
-      Zl[l] = colbuf + off + sl;
+      Zl[l] = mgbuf + off + sl;
       off += (size_t)(hl + 2) * sl;
-      Rl[l] = colbuf + off;
+      Rl[l] = mgbuf + off;
       off += (size_t)hl * sl;
     }
   }
@@ -1173,7 +1289,9 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
   const bool halo = a.prolong != 0;
   // With three levels (and slabs that split evenly over the threads) every
   // level array the coarse levels need is loaded into registers here, beside
-  // the loads of the first restriction, so the coarse phases wait on no load.
+  // the loads of the first restriction, so the coarse phases wait on no load
+  // (ONE: where they are used; the other CTA of the SM covers the wait and the
+  // registers are not there to hold them).
   constexpr int wc1 = M / 2, hc1 = wc1 / C, wc2 = M / 4, hc2 = wc2 / C;
   constexpr bool kL3 = hc2 >= 1 && hc2 * wc2 >= NT && (hc2 * wc2) % NT == 0 && (hc1 * wc1) % NT == 0;
   constexpr int Q12 = kL3 ? hc2 * wc2 / NT : 1, QUP = kL3 ? hc1 * wc1 / NT : 1;
@@ -1181,29 +1299,31 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
   float2 pf_wz1[Q12][2];     // W_z,1 at (2i + dy, 2j .. 2j + 1): (dx 0, dx 1) per dy
   float4 pf_wr1[Q12][2];     // W_R,1 at the same pixels
   float2 pf_g2[Q12], pf_q2[Q12], pf_g1[QUP], pf_q1[QUP];
+  auto load_l2 = [&](int t) {
+    const int p = tid + t * NT, i = p / wc2, j = p % wc2;
+#pragma unroll
+    for (int dy = 0; dy < 2; ++dy) {
+      const int r = rank * hc1 + 2 * i + dy, c = 2 * j;
+      const int wi = EMG_INB(r * wc1 + c + 1, wc1 * wc1, kBcLevel) ? r * wc1 + c : 0;
+      pf_wz1[t][dy] = __ldcg(reinterpret_cast<const float2*>(a.lv.Wz[1] + wi));
+      pf_wr1[t][dy] = __ldcg(reinterpret_cast<const float4*>(a.lv.WR[1] + wi));
+    }
+    const int li = EMG_INB((rank * hc2 + i) * wc2 + j, wc2 * wc2, kBcLevel) ? (rank * hc2 + i) * wc2 + j : 0;
+    pf_g2[t] = __ldcg(a.lv.G[2] + li);
+    pf_q2[t] = __ldcg(a.lv.Q[2] + li);
+  };
+  auto load_up = [&](int t) {
+    const int p = tid + t * NT, i = p / wc1, j = p % wc1;
+    const int li = EMG_INB((rank * hc1 + i) * wc1 + j, wc1 * wc1, kBcLevel) ? (rank * hc1 + i) * wc1 + j : 0;
+    pf_g1[t] = __ldcg(a.lv.G[1] + li);
+    pf_q1[t] = __ldcg(a.lv.Q[1] + li);
+  };
   if (a.levels > 1) {
-    if (l3) {
+    if (l3 && !ONE) {
 #pragma unroll
-      for (int t = 0; t < Q12; ++t) {
-        const int p = tid + t * NT, i = p / wc2, j = p % wc2;
+      for (int t = 0; t < Q12; ++t) load_l2(t);
 #pragma unroll
-        for (int dy = 0; dy < 2; ++dy) {
-          const int r = rank * hc1 + 2 * i + dy, c = 2 * j;
-          const int wi = EMG_INB(r * wc1 + c + 1, wc1 * wc1, kBcLevel) ? r * wc1 + c : 0;
-          pf_wz1[t][dy] = __ldcg(reinterpret_cast<const float2*>(a.lv.Wz[1] + wi));
-          pf_wr1[t][dy] = __ldcg(reinterpret_cast<const float4*>(a.lv.WR[1] + wi));
-        }
-        const int li = EMG_INB((rank * hc2 + i) * wc2 + j, wc2 * wc2, kBcLevel) ? (rank * hc2 + i) * wc2 + j : 0;
-        pf_g2[t] = __ldcg(a.lv.G[2] + li);
-        pf_q2[t] = __ldcg(a.lv.Q[2] + li);
-      }
-#pragma unroll
-      for (int t = 0; t < QUP; ++t) {
-        const int p = tid + t * NT, i = p / wc1, j = p % wc1;
-        const int li = EMG_INB((rank * hc1 + i) * wc1 + j, wc1 * wc1, kBcLevel) ? (rank * hc1 + i) * wc1 + j : 0;
-        pf_g1[t] = __ldcg(a.lv.G[1] + li);
-        pf_q1[t] = __ldcg(a.lv.Q[1] + li);
-      }
+      for (int t = 0; t < QUP; ++t) load_up(t);
     }
     {  // restrict level 0 -> 1: z_1 = I_h^H (W_z z_k), R_1 = I_h^H (W_R R)
       constexpr int wc = M / 2, hc = wc / C, sc = wc + 1;
@@ -1224,9 +1344,9 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
           // the weights of the pixel pair (c, c + 1) in one load each (c is even)
           const float2 wz = __ldcg(reinterpret_cast<const float2*>(Wz + r * M + c));
           const float4 wr = __ldcg(reinterpret_cast<const float4*>(WR + r * M + c));
-          zs = cadd(zs, cscale(zbuf[lr * M + c], wz.x));
+          zs = cadd(zs, cscale(z_at(lr, c), wz.x));
           rs = cfma(make_float2(wr.x, wr.y), rowbuf[lr * SR + c], rs);
-          zs = cadd(zs, cscale(zbuf[lr * M + c + 1], wz.y));
+          zs = cadd(zs, cscale(z_at(lr, c + 1), wz.y));
           rs = cfma(make_float2(wr.z, wr.w), rowbuf[lr * SR + c + 1], rs);
         }
         Z1w[i * sc + j] = cscale(zs, 0.25f);
@@ -1241,6 +1361,10 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
         const float2* __restrict__ const Zf = Zl[1];
         const float2* __restrict__ const Rf = Rl[1];
         float2* __restrict__ const Zc = Zl[2];
+        if constexpr (ONE) {
+#pragma unroll
+          for (int t = 0; t < Q12; ++t) load_l2(t);
+        }
 #pragma unroll
         for (int t = 0; t < Q12; ++t) {
           const int p = tid + t * NT, i = p / wc2, j = p % wc2;
@@ -1259,6 +1383,10 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
           Zc[i * sc + j] = cc;
           if (halo) push_halo<C>(cl, rank, Zc, sc, hc2, i, j, cc);
         }
+      }
+      if constexpr (ONE) {
+#pragma unroll
+        for (int t = 0; t < QUP; ++t) load_up(t);
       }
       if (halo) cl.sync();  // the pushed halo rows of level 2 are in place
       __syncthreads();
@@ -1357,7 +1485,9 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
   float acc_after = 0.f;
   // Groups of UG pixels: the probe and gain loads of a group are issued
   // together, and the loop body stays small enough for the instruction cache.
-  constexpr int UG0 = EMG_UPDATE_GROUP < PER ? EMG_UPDATE_GROUP : PER;
+  // (two CTAs per SM at m = 256 hide the load latency and leave 64 registers: groups of 4)
+  constexpr int UGM = ONE ? 4 : EMG_UPDATE_GROUP;
+  constexpr int UG0 = UGM < PER ? UGM : PER;
   constexpr int UG = PER % UG0 == 0 ? UG0 : 1;
   // The common case (multigrid, joint step, ordered combine, no verify) runs a
   // loop without the mode branches over pairs of adjacent pixels, with 16-byte
@@ -1384,7 +1514,13 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
         for (int u = 0; u < UGP; ++u) {
           const int p0 = 2 * (tid + (t0 + u) * NT);
           const int lr = p0 / M, c0 = p0 % M, r = row0 + lr;
-          const float4 zk2 = *reinterpret_cast<const float4*>(zbuf + p0);
+          float4 zk2;
+          if constexpr (ONE) {
+            const float2 za = z_at(lr, c0), zb = z_at(lr, c0 + 1);
+            zk2 = make_float4(za.x, za.y, zb.x, zb.y);
+          } else {
+            zk2 = *reinterpret_cast<const float4*>(zbuf + p0);
+          }
           // coarse-level correction at both pixels: the rows and the centre column are shared
           float2 pro[2];
           {
@@ -1427,7 +1563,7 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_stepc(const StepArgs a) 
     const int t = t0 + u;
     const int p = tid + t * NT;
     const int lr = p / M, c = p % M, r = row0 + lr;
-    const float2 zk = zbuf[p];
+    const float2 zk = z_at(lr, c);
     const float2 q = qv[u];
     const float2 R = rowbuf[lr * SR + c];
     const float2 pro = a.levels == 1 ? czero() : prolong_halo<float2>(Z1, M / 2 + 1, M / 2, lr, c, a.prolong);
@@ -2324,7 +2460,7 @@ bool prep_tiled_config(PrepArgs& a) {
 
 template <int M, int C>
 constexpr size_t stepc_smem_bytes() {
-  return CTile<M, C>::smem_elems * sizeof(float2);
+  return StepTile<M, C>::smem_elems * sizeof(float2);
 }
 
 // Clusters of the step kernel that can be resident at once (CTAs per SM from
@@ -2332,7 +2468,7 @@ constexpr size_t stepc_smem_bytes() {
 template <int M, int C>
 int stepc_resident_clusters() {
   int per_sm = 0, dev = 0, sms = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stepc<M, C>, CTile<M, C>::NT,
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stepc<M, C>, StepTile<M, C>::NT,
                                                     stepc_smem_bytes<M, C>()) != cudaSuccess ||
       cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
@@ -2469,6 +2605,11 @@ cudaError_t set_cluster_smem(Kernel k, size_t elems) {
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(elems * sizeof(float2)));
 }
 
+template <int M, int C, bool RIN = false>
+cudaError_t set_stepc_attrs() {
+  return set_cluster_smem(k_stepc<M, C, RIN>, StepTile<M, C>::smem_elems);
+}
+
 template <int M>
 cudaError_t set_grad_attrs() {
   constexpr int C = ClusterSize<M>::value;
@@ -2478,24 +2619,18 @@ cudaError_t set_grad_attrs() {
 // Dynamic shared-memory limits of the cluster kernels (once per device).
 cudaError_t set_cluster_attrs() {
   cudaError_t e;
-  if ((e = set_cluster_smem(k_stepc<16, 2>, CTile<16, 2>::smem_elems)) != cudaSuccess) return e;
-  if ((e = set_cluster_smem(k_stepc<32, 2>, CTile<32, 2>::smem_elems)) != cudaSuccess) return e;
-  if ((e = set_cluster_smem(k_stepc<64, 4>, CTile<64, 4>::smem_elems)) != cudaSuccess) return e;
-  if ((e = set_cluster_smem(k_stepc<128, 4>, CTile<128, 4>::smem_elems)) != cudaSuccess) return e;
-  if ((e = set_cluster_smem(k_stepc<128, 8>, CTile<128, 8>::smem_elems)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(k_stepc<64, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(CTile<64, 2>::smem_elems * sizeof(float2)))) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(k_stepc<128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(CTile<128, 2>::smem_elems * sizeof(float2)))) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(k_stepc<256, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(CTile<256, 8>::smem_elems * sizeof(float2)))) != cudaSuccess)
-    return e;
-  if ((e = set_cluster_smem(k_stepc<128, 2, true>, CTile<128, 2>::smem_elems)) != cudaSuccess) return e;
-  if ((e = set_cluster_smem(k_stepc<128, 4, true>, CTile<128, 4>::smem_elems)) != cudaSuccess) return e;
-  if ((e = set_cluster_smem(k_stepc<128, 8, true>, CTile<128, 8>::smem_elems)) != cudaSuccess) return e;
-  if ((e = set_cluster_smem(k_stepc<256, 8, true>, CTile<256, 8>::smem_elems)) != cudaSuccess) return e;
+  if ((e = set_stepc_attrs<16, 2>()) != cudaSuccess) return e;
+  if ((e = set_stepc_attrs<32, 2>()) != cudaSuccess) return e;
+  if ((e = set_stepc_attrs<64, 2>()) != cudaSuccess) return e;
+  if ((e = set_stepc_attrs<64, 4>()) != cudaSuccess) return e;
+  if ((e = set_stepc_attrs<128, 2>()) != cudaSuccess) return e;
+  if ((e = set_stepc_attrs<128, 4>()) != cudaSuccess) return e;
+  if ((e = set_stepc_attrs<128, 8>()) != cudaSuccess) return e;
+  if ((e = set_stepc_attrs<256, 8>()) != cudaSuccess) return e;
+  if ((e = set_stepc_attrs<128, 2, true>()) != cudaSuccess) return e;
+  if ((e = set_stepc_attrs<128, 4, true>()) != cudaSuccess) return e;
+  if ((e = set_stepc_attrs<128, 8, true>()) != cudaSuccess) return e;
+  if ((e = set_stepc_attrs<256, 8, true>()) != cudaSuccess) return e;
   if ((e = set_cluster_smem(k_fwdc<256, 8, 0>, CTile<256, 8>::smem_elems)) != cudaSuccess) return e;
   if ((e = set_cluster_smem(k_fwdc<256, 8, 1>, CTile<256, 8>::smem_elems)) != cudaSuccess) return e;
   if ((e = set_cluster_smem(k_fwdc<256, 8, 2>, CTile<256, 8>::smem_elems)) != cudaSuccess) return e;
@@ -2513,7 +2648,7 @@ cudaError_t set_cluster_attrs() {
 
 template <int M, int C>
 cudaError_t launch_stepc_t(int b, const StepArgs& a, cudaStream_t s) {
-  using TL = CTile<M, C>;
+  using TL = StepTile<M, C>;
   cudaError_t e = launch_cluster_pdl(k_stepc<M, C>, C, dim3(C * (b + a.prep_clusters)), dim3(TL::NT),
                                      TL::smem_elems * sizeof(float2), s, a);
   if (e != cudaSuccess) return e;
@@ -2522,7 +2657,7 @@ cudaError_t launch_stepc_t(int b, const StepArgs& a, cudaStream_t s) {
 
 template <int M, int C>
 cudaError_t launch_stepc_rin_t(int b, const StepArgs& a, cudaStream_t s) {
-  using TL = CTile<M, C>;
+  using TL = StepTile<M, C>;
   cudaError_t e = launch_cluster_pdl(k_stepc<M, C, true>, C, dim3(C * b), dim3(TL::NT),
                                      TL::smem_elems * sizeof(float2), s, a);
   if (e != cudaSuccess) return e;
@@ -2709,7 +2844,8 @@ bool step_supported(int m, int levels, int cluster) {
     const size_t wl = (size_t)m >> l, hl = wl / cluster;
     need += (2 * hl + 2) * (wl + 1);
   }
-  return need <= (size_t)m * (m / cluster + 1);
+  // the buffers reuse the column slab (m = 256: an area sized for every level count that passes the row rule)
+  return m == 256 || need <= (size_t)(m / cluster) * (m + 1);
 }
 
 cudaError_t launch_normalize_probe(const float* amp, int m, int n_pos, float2* probe,
