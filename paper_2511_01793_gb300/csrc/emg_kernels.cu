@@ -7,9 +7,9 @@
 //                  replacement (Def. 2.1), inverse FFT, MAGPIE object step,
 //                  ePIE probe step, geometric-mean joint step (Eq. geomean)
 //   k_apply        deterministic combine of the minibatch into object and probe
-//   k_misfit<M>    Phi_k = 1/2 ||Q . P_k z - R_k||^2 (Eq. exit_misfit), per position
-//   k_simulate<M>  d_k = |F(Q . P_k z)|^2 (Sec. 2.1 data model)
-//   k_fft2<M>      batched 2-D DFT of natural-order tiles
+//   k_forward<M>   Phi_k = 1/2 ||Q . P_k z - R_k||^2 (Eq. exit_misfit) per position,
+//                  d_k = |F(Q . P_k z)|^2 (Sec. 2.1 data model), batched 2-D DFT
+//                  of natural-order tiles
 #include <cooperative_groups.h>
 #include <math.h>
 #include <stdint.h>
@@ -131,24 +131,6 @@ __device__ __forceinline__ float2 geometric_mean_aligned(float2 x, float2 xp) {
   return y;
 }
 
-// y with y^2 = x * xp and Re(y conj(x)) >= 0 (Eq. geomean), branch-free.
-// With w = x xp = u + i v, s = (|u| + |w|)/2, t = sqrt(s), h = 1/(2t):
-// (t, v h) squares to w when u >= 0 (Kahan's half-angle form), and (v h, t)
-// squares to w when u < 0 (its real part is (v^2 - 4 s^2)/(4 s) = u); either
-// root is then negated if it points away from x.  Square roots come from rsqrtf.
-__device__ __forceinline__ float2 geometric_mean_aligned_fast(float2 x, float2 xp) {
-  const float2 w = cmul(x, xp);
-  const float n = fmaf(w.x, w.x, w.y * w.y);
-  const float mag = n * rsqrtf(n);
-  const float s = 0.5f * (fabsf(w.x) + mag);
-  const float rt = rsqrtf(s);
-  const float t = s * rt, vh = w.y * (0.5f * rt);
-  float2 y = w.x >= 0.f ? make_float2(t, vh) : make_float2(vh, t);
-  const float sgn = fmaf(y.x, x.x, y.y * x.y) < 0.f ? -1.f : 1.f;
-  y = n > 0.f ? make_float2(sgn * y.x, sgn * y.y) : czero();
-  return y;
-}
-
 // c + a b, c - a b and c + conj(a) b as chains of two fused multiply-adds per part.
 __device__ __forceinline__ float2 cfma(float2 a, float2 b, float2 c) {
   return make_float2(fmaf(a.x, b.x, fmaf(-a.y, b.y, c.x)), fmaf(a.x, b.y, fmaf(a.y, b.x, c.y)));
@@ -160,9 +142,11 @@ __device__ __forceinline__ float2 cfma_conj(float2 a, float2 b, float2 c) {
   return make_float2(fmaf(a.x, b.x, fmaf(a.y, b.y, c.x)), fmaf(a.x, b.y, fmaf(-a.y, b.x, c.y)));
 }
 
-// y with y^2 = x * xp and Re(y conj(x)) >= 0 (Eq. geomean), branch-free, in
-// the half-angle form of geometric_mean_aligned_fast with s' = 2 s, so that
-// t = sqrt(s) = s' r / sqrt(2) and v h = v r / sqrt(2) for r = 1 / sqrt(s').
+// y with y^2 = x * xp and Re(y conj(x)) >= 0 (Eq. geomean), branch-free.
+// With w = x xp = u + i v, s = (|u| + |w|)/2, t = sqrt(s), h = 1/(2t): (t, v h)
+// squares to w when u >= 0 (Kahan's half-angle form), and (v h, t) when u < 0
+// (its real part is (v^2 - 4 s^2)/(4 s) = u).  With s' = 2 s and r = 1 / sqrt(s'),
+// t = s' r / sqrt(2) and v h = v r / sqrt(2).
 // A floor of 1e-37 under both square roots gives y = 0 for w = 0 without a
 // branch; it changes no result for |w|^2 above about 1e-29.  The sign flip
 // is applied to the sign bit when Re(y conj(x)) < 0.
@@ -272,17 +256,40 @@ __device__ __forceinline__ double block_sum_f(float v, float* shf, double* shd) 
   return shd[0];
 }
 
+// FP64 block sum, broadcast: warp trees, then one warp's tree over the NT/32
+// warp sums.  (The FP64 pipe takes two results per SM and clock: every thread
+// adding all warp sums cost 8 us in a block of 1024.)
 template <int NT>
 __device__ __forceinline__ double block_sum(double v, double* sh) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
   __syncthreads();
-  double r = sh[0];
+  if (threadIdx.x < 32) {
+    double r = threadIdx.x < NT / 32 ? sh[threadIdx.x] : 0.0;
 #pragma unroll
-  for (int i = 1; i < NT / 32; ++i) r += sh[i];
+    for (int o = NT / 64; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    if (threadIdx.x == 0) sh[0] = r;
+  }
+  __syncthreads();
+  const double r = sh[0];
   __syncthreads();
   return r;
+}
+
+// Warp sum of FP32 values to FP64 accuracy without the FP64 pipe: each tree
+// level adds exactly (Knuth's TwoSum) and carries the rounding errors along.
+// Lane 0 gets the value.
+__device__ __forceinline__ double warp_sum_exact(float hi) {
+  float lo = 0.f;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float b = __shfl_xor_sync(0xffffffffu, hi, o), bl = __shfl_xor_sync(0xffffffffu, lo, o);
+    const float s = hi + b, t = s - hi;
+    lo += bl + ((hi - (s - t)) + (b - t));
+    hi = s;
+  }
+  return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
 }
 
 // ---------------------------------------------------------------------------
@@ -908,22 +915,14 @@ __device__ __forceinline__ void cluster_arrive_relaxed() {
 }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
 
-template <int M> struct ClusterSize;
-template <> struct ClusterSize<16> { static constexpr int value = 2; };
-template <> struct ClusterSize<32> { static constexpr int value = 2; };
-template <> struct ClusterSize<64> { static constexpr int value = 2; };
-template <> struct ClusterSize<128> { static constexpr int value = 2; };
-template <> struct ClusterSize<256> { static constexpr int value = 8; };
-
 template <int M, int C>
 struct CTile {
   static constexpr int H = M / C;              // rows of a row slab, columns of a column slab
-  static constexpr int SR = M + 1, SC = H + 1;  // odd strides: conflict-free lines
+  static constexpr int SR = M + 1;             // odd stride of a slab's lines: conflict-free
   static constexpr int N1 = FftPlan<M>::N1, N2 = FftPlan<M>::N2;
   static constexpr int NT = H * N1;            // one pass-A slot per thread
   static constexpr int PER = H * M / NT;       // slab pixels per thread
   static constexpr int SLOTS = H * N2 / NT;    // column pass-B slots per thread
-  static constexpr size_t smem_elems = (size_t)H * SR + (size_t)M * SC + (size_t)H * M;
   static_assert(H * M % NT == 0 && H * N2 % NT == 0 && NT <= 1024, "slab must split evenly");
   static_assert(H % N1 == 0, "the outputs of one pass-B slot go to one CTA");
 };
@@ -939,10 +938,14 @@ struct CTile {
 // and the multigrid buffers after them; z_k is read again from L2 where the
 // multigrid and the update need it.  199 KB per CTA with three slabs leave
 // one CTA of 16 warps per SM and at most 15 clusters of 8 on the device (120
-// SMs); 114 KB let two CTAs share an SM and hide each other's barriers.
+// SMs); 114 KB let two CTAs share an SM and hide each other's barriers.  An
+// epoch of 4096 positions with minibatches of 256: 8.51 -> 6.93 ms (with the
+// transposes taken into the passes, which alone gives 0.428 -> 0.404 ms for
+// 900 positions at m = 128 with minibatches of 64).
 template <int M, int C>
 struct StepTile : CTile<M, C> {
   using B = CTile<M, C>;
+  static constexpr int SIDE = M, CTAS = C;
   static constexpr bool ONE = M == 256;
   static constexpr int S = B::SR;
   // CTAs per SM the register budget leaves room for (as many as the shared memory does)
@@ -960,46 +963,64 @@ struct StepTile : CTile<M, C> {
   static_assert(ONE || mg_elems() <= slab, "the multigrid buffers reuse the column slab");
 };
 
-// Row slab (after the row passes) -> column slabs of all C CTAs.
-template <int M, int C>
-__device__ __forceinline__ void cluster_rows_to_cols(cg::cluster_group& cl, int rank, const float2* rowbuf,
-                                                     float2* colbuf, int tid) {
-  using T = CTile<M, C>;
-  for (int s = tid; s < T::H * M; s += T::NT) {
-    const int lr = s / M, e = s % M, d = e / T::H;
-    float2* dst = d == rank ? colbuf : cl.map_shared_rank(colbuf, d);
-    dst[(rank * T::H + lr) * T::SC + (e % T::H)] = rowbuf[lr * T::SR + e];
-  }
+// Forward and gradient kernels: whole launches of many positions, so the
+// shared memory is one slab (transposed in place) and as many CTAs share an SM
+// as 64 registers per thread allow.
+template <int M> struct WaveCluster { static constexpr int value = M == 256 ? 8 : M == 128 ? 2 : 1; };
+template <int M>
+struct WaveTile : CTile<M, WaveCluster<M>::value> {
+  using B = CTile<M, WaveCluster<M>::value>;
+  static constexpr int SIDE = M, CTAS = WaveCluster<M>::value;
+  static constexpr bool ONE = true;
+  static constexpr int S = B::SR;
+  static constexpr size_t slab = (size_t)B::H * S;
+  static constexpr int MIN_CTAS = 1024 / B::NT;
+  static_assert(B::H % B::N2 == 0, "the natural columns of one pass-B output index go to one CTA");
+};
+
+// Barrier of all CTAs of the cluster that also publishes shared-memory writes.
+template <int C>
+__device__ __forceinline__ void tile_sync(cg::cluster_group& cl) {
+  if constexpr (C == 1)
+    __syncthreads();
+  else
+    cl.sync();
 }
 
-// Column slab -> row slabs of all C CTAs.
-template <int M, int C>
-__device__ __forceinline__ void cluster_cols_to_rows(cg::cluster_group& cl, int rank, const float2* colbuf,
-                                                     float2* rowbuf, int tid) {
-  using T = CTile<M, C>;
-  for (int s = tid; s < M * T::H; s += T::NT) {
-    const int r = s / T::H, lc = s % T::H, d = r / T::H;
-    float2* dst = d == rank ? rowbuf : cl.map_shared_rank(rowbuf, d);
-    dst[(r % T::H) * T::SR + rank * T::H + lc] = colbuf[r * T::SC + lc];
-  }
+// `buf` of CTA d of the cluster.
+template <int C, typename V>
+__device__ __forceinline__ V* tile_rank(cg::cluster_group& cl, int rank, V* buf, int d) {
+  if constexpr (C == 1)
+    return buf;
+  else
+    return d == rank ? buf : cl.map_shared_rank(buf, d);
 }
 
 // Row pass B on my row slab, its outputs stored straight into the column slabs
-// of all C CTAs (the transpose costs no pass of its own).  Lanes take
+// of all CTAs (the transpose costs no pass of its own).  Lanes take
 // consecutive rows, which are consecutive elements of a column line, so each
-// store of a warp is one contiguous run.  With one slab per CTA the outputs wait in
-// registers until every CTA of the cluster has read its slab.  The caller's
-// cluster barrier makes the columns visible.
-template <int M, int C>
+// store of a warp is one contiguous run.  NAT = false: the slab of CTA d holds
+// storage columns [d H, (d + 1) H); NAT = true: natural columns of that range.
+// With one slab per CTA the outputs wait in registers until every CTA of the
+// cluster has read its slab.  The caller's barrier makes the columns visible.
+template <class T, bool NAT = false>
 __device__ __forceinline__ void row_pass_b_to_cols(cg::cluster_group& cl, int rank, const float2* rowbuf,
                                                    float2* colbuf, int tid) {
-  using T = StepTile<M, C>;
   float2 v[T::SLOTS][T::N1];
   auto put = [&](int t) {
-    const int s = tid + t * T::NT, e0 = T::N1 * (s / T::H), line = s % T::H, d = e0 / T::H;
-    float2* dst = (d == rank ? colbuf : cl.map_shared_rank(colbuf, d)) + (e0 % T::H) * T::S + rank * T::H + line;
+    const int s = tid + t * T::NT, k2 = s / T::H, at = rank * T::H + s % T::H;
+    if constexpr (NAT) {
 #pragma unroll
-    for (int i = 0; i < T::N1; ++i) dst[i * T::S] = v[t][i];
+      for (int i = 0; i < T::N1; ++i) {
+        const int d = T::N2 * i / T::H;  // k2 < N2 and N2 divides H
+        tile_rank<T::CTAS>(cl, rank, colbuf, d)[(T::N2 * i % T::H + k2) * T::S + at] = v[t][i];
+      }
+    } else {
+      const int e0 = T::N1 * k2;
+      float2* dst = tile_rank<T::CTAS>(cl, rank, colbuf, e0 / T::H) + (e0 % T::H) * T::S + at;
+#pragma unroll
+      for (int i = 0; i < T::N1; ++i) dst[i * T::S] = v[t][i];
+    }
   };
 #pragma unroll
   for (int t = 0; t < T::SLOTS; ++t) {
@@ -1011,32 +1032,31 @@ __device__ __forceinline__ void row_pass_b_to_cols(cg::cluster_group& cl, int ra
     if constexpr (!T::ONE) put(t);
   }
   if constexpr (T::ONE) {
-    cl.sync();
+    tile_sync<T::CTAS>(cl);
 #pragma unroll
     for (int t = 0; t < T::SLOTS; ++t) put(t);
   }
 }
 
 // Inverse column pass A on my column slab, its outputs (natural rows) stored
-// straight into the row slabs of all C CTAs; lanes take consecutive columns,
+// straight into the row slabs of all CTAs; lanes take consecutive columns,
 // so each store of a warp is one contiguous run of a row.
-template <int M, int C>
+template <class T>
 __device__ __forceinline__ void col_pass_a_inv_to_rows(cg::cluster_group& cl, int rank, const float2* colbuf,
                                                        float2* rowbuf, int tid) {
-  using T = StepTile<M, C>;
   const int j = tid / T::H, line = tid % T::H;
   const float2* p = colbuf + line * T::S + j;
   float2 v[T::N2];
 #pragma unroll
   for (int k2 = 0; k2 < T::N2; ++k2) v[k2] = p[T::N1 * k2];
 #pragma unroll
-  for (int k2 = 1; k2 < T::N2; ++k2) v[k2] = cmulc(v[k2], stage_twiddle<M>(j, k2));
+  for (int k2 = 1; k2 < T::N2; ++k2) v[k2] = cmulc(v[k2], stage_twiddle<T::SIDE>(j, k2));
   Dft<T::N2, true>::run(v);
-  if constexpr (T::ONE) cl.sync();
+  if constexpr (T::ONE) tile_sync<T::CTAS>(cl);
 #pragma unroll
   for (int n2 = 0; n2 < T::N2; ++n2) {
     const int d = T::N1 * n2 / T::H, lr = T::N1 * n2 % T::H + j;
-    (d == rank ? rowbuf : cl.map_shared_rank(rowbuf, d))[lr * T::S + rank * T::H + line] = v[n2];
+    tile_rank<T::CTAS>(cl, rank, rowbuf, d)[lr * T::S + rank * T::H + line] = v[n2];
   }
 }
 
@@ -1079,7 +1099,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   using TL = StepTile<M, C>;
   constexpr bool ONE = TL::ONE;
   constexpr int NT = TL::NT, H = TL::H, SR = TL::S;
-  constexpr int N1 = TL::N1, N2 = TL::N2, PER = TL::PER, SLOTS = TL::SLOTS;
+  constexpr int N1 = TL::N1, PER = TL::PER, SLOTS = TL::SLOTS;
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank();
   extern __shared__ __align__(16) float2 sm[];  // 16-byte aligned: the update pass reads pixel pairs
@@ -1188,7 +1208,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   }
   cl.barrier_wait();  // all CTAs of the cluster resident
   // row pass B, outputs to the column slabs
-  if constexpr (!RIN) row_pass_b_to_cols<M, C>(cl, rank, rowbuf, colbuf, tid);
+  if constexpr (!RIN) row_pass_b_to_cols<TL>(cl, rank, rowbuf, colbuf, tid);
   if (tid == 0) cluster_publish<C>(cl, rank, xf, partials_max<NT>(redf));
   cl.sync();
   float mu = xf[0];
@@ -1235,7 +1255,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   warp_partial_sum(acc, redf);
   __syncthreads();
   // inverse column pass A, outputs to the row slabs
-  col_pass_a_inv_to_rows<M, C>(cl, rank, colbuf, rowbuf, tid);
+  col_pass_a_inv_to_rows<TL>(cl, rank, colbuf, rowbuf, tid);
   if (tid == 0) cluster_publish<C>(cl, rank, xd, partials_sum<NT>(redf));
   cl.sync();
   // a4: inverse row passes -> R (natural order) on my rows
@@ -1618,66 +1638,92 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
 }
 
 // ---------------------------------------------------------------------------
-// Forward transform of one tile per cluster (any m): modes
-//   0 misfit partial (1/2 m^2) sum (|F psi| - a_k)^2 per position,
-//   1 intensity |F psi|^2 in natural order,
-//   2 F x of a natural-order tile.
-template <int M, int C, int MODE>
-__global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_fwdc(const FwdArgs a) {
-  using TL = CTile<M, C>;
-  constexpr int NT = TL::NT, H = TL::H, SR = TL::SR, SC = TL::SC, N1 = TL::N1, N2 = TL::N2;
+// Forward transform of one tile per cluster: modes
+//   0 misfit partial (1/2 m^2) sum (|F psi| - a_k)^2 per position (Parseval
+//     form of Eq. exit_misfit),
+//   1 intensity |F psi|^2 in natural order (data model of Sec. 2.1),
+//   2 F x of a natural-order tile, 3 F^-1 x = conj(F conj(x / m^2)).
+// Bound by instruction issue and shared-memory latency, so the tile takes the
+// smallest cluster whose slab leaves 32 warps per SM.  The outputs of modes
+// 1-3 leave column pass B from registers: the slabs hold natural columns, so a
+// warp writes whole 128-byte runs of a natural row.
+template <int M, int MODE>
+__global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_forward(const FwdArgs a) {
+  using TL = WaveTile<M>;
+  constexpr int NT = TL::NT, H = TL::H, S = TL::S, N1 = TL::N1, N2 = TL::N2, C = TL::CTAS, PER = TL::PER;
   cg::cluster_group cl = cg::this_cluster();
-  const int rank = (int)cl.block_rank();
+  const int rank = C == 1 ? 0 : (int)cl.block_rank();
   extern __shared__ float2 sm[];
-  float2* rowbuf = sm;
-  float2* colbuf = sm + H * SR;
   __shared__ double xd[C];
-  __shared__ double redd[2];
-  __shared__ float redf[NT / 32];
+  __shared__ double redd[(NT + 31) / 32];
   const int tid = threadIdx.x;
   const int t = blockIdx.x / C;
   const int row0 = rank * H;
-  cluster_arrive_relaxed();
-  if (MODE == 2) {
-    const float2* x = a.in + (size_t)t * M * M;
-    for (int p = tid; p < H * M; p += NT) rowbuf[(p / M) * SR + p % M] = x[row0 * M + p];
+  const float inv_m2 = 1.f / (float)(M * M);
+  if constexpr (MODE >= 2) {
+    const float2* x = a.in + (size_t)t * M * M + row0 * M;
+#pragma unroll (PER < 8 ? PER : 8)
+    for (int u = 0; u < PER; ++u) {
+      const int p = tid + u * NT;
+      const float2 v = x[p];
+      sm[(p / M) * S + p % M] = MODE == 3 ? make_float2(v.x * inv_m2, -v.y * inv_m2) : v;
+    }
   } else {
     const int o_r = a.pos[2 * t], o_c = a.pos[2 * t + 1];
-    for (int p = tid; p < H * M; p += NT) {
-      const int lr = p / M, c = p % M, r = row0 + lr;
-      rowbuf[lr * SR + c] = cmul(a.probe[r * M + c], gather_obj(a.object, a.n_rows, a.n_cols, o_r + r, o_c + c));
+#pragma unroll (PER < 8 ? PER : 8)
+    for (int u = 0; u < PER; ++u) {
+      const int p = tid + u * NT, lr = p / M, c = p % M, r = row0 + lr;
+      sm[lr * S + c] = cmul(a.probe[r * M + c], gather_obj(a.object, a.n_rows, a.n_cols, o_r + r, o_c + c));
     }
   }
   __syncthreads();
-  gpass_a_fwd<M, H, SR, 1, NT>(rowbuf, tid);
+  gpass_a_fwd<M, H, S, 1, NT>(sm, tid);
   __syncthreads();
-  gpass_b<M, H, SR, 1, NT, false>(rowbuf, tid);
-  __syncthreads();
-  cl.barrier_wait();
-  cluster_rows_to_cols<M, C>(cl, rank, rowbuf, colbuf, tid);
-  cl.sync();
-  gpass_a_fwd<M, H, 1, SC, NT>(colbuf, tid);
-  __syncthreads();
-  gpass_b<M, H, 1, SC, NT, false>(colbuf, tid);
+  row_pass_b_to_cols<TL, MODE != 0>(cl, rank, sm, sm, tid);
+  tile_sync<C>(cl);
+  gpass_a_fwd<M, H, S, 1, NT>(sm, tid);
   __syncthreads();
   float acc = 0.f;
-  for (int p = tid; p < M * H; p += NT) {
-    const int er = p / H, lc = p % H, ec = rank * H + lc;
-    const float2 v = colbuf[er * SC + lc];
-    const size_t nat = (size_t)storage_to_freq<M>(er) * M + storage_to_freq<M>(ec);
-    if (MODE == 0) {
-      const float dm = sqrtf(cabs2(v)) - a.amp[(size_t)t * M * M + er * M + ec];
-      acc = fmaf(dm, dm, acc);
-    } else if (MODE == 1) {
-      a.out_intensity[(size_t)t * M * M + nat] = cabs2(v);
-    } else {
-      a.out[(size_t)t * M * M + nat] = v;
+#pragma unroll
+  for (int q = 0; q < TL::SLOTS; ++q) {
+    const int s = tid + q * NT, k2 = s / H, lc = s % H;
+    const float2* p = sm + lc * S + N1 * k2;
+    float am[MODE == 0 ? N1 : 1];
+    if constexpr (MODE == 0) {
+#pragma unroll
+      for (int i = 0; i < N1; ++i) am[i] = __ldg(a.amp + (size_t)t * M * M + (i + N1 * k2) * M + row0 + lc);
+    }
+    float2 v[N1];
+#pragma unroll
+    for (int i = 0; i < N1; ++i) v[i] = p[i];
+    Dft<N1, false>::run(v);
+#pragma unroll
+    for (int i = 0; i < N1; ++i) {
+      const size_t nat = (size_t)t * M * M + (k2 + N2 * i) * M + row0 + lc;
+      if constexpr (MODE == 0) {
+        const float dm = sqrtf(cabs2(v[i])) - am[i];
+        acc = fmaf(dm, dm, acc);
+      } else if constexpr (MODE == 1) {
+        a.out_intensity[nat] = cabs2(v[i]);
+      } else {
+        a.out[nat] = MODE == 3 ? cconj(v[i]) : v[i];
+      }
     }
   }
-  if (MODE == 0) {
-    const double part = block_sum_f<NT>(acc, redf, redd);
-    if (tid == 0) cluster_publish<C>(cl, rank, xd, part);
-    cl.sync();
+  if constexpr (MODE == 0) {
+    const double w = warp_sum_exact(acc);
+    if ((tid & 31) == 0) redd[tid >> 5] = w;
+    __syncthreads();
+    double part = 0.0;
+    if (tid == 0)
+      for (int i = 0; i < NT / 32; ++i) part += redd[i];
+    if constexpr (C > 1) {
+      // only rank 0 needs the parts; no CTA touches another's memory after this barrier
+      if (tid == 0) *tile_rank<C>(cl, rank, &xd[rank], 0) = part;
+      cl.sync();
+    } else if (tid == 0) {
+      xd[0] = part;
+    }
     if (rank == 0 && tid == 0) {
       double tot = 0.0;
 #pragma unroll
@@ -1687,106 +1733,61 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_fwdc(const FwdArgs a) {
   }
 }
 
-// Inverse 2-D DFT (with 1/m^2) of natural-order tiles, one tile per cluster.
-template <int M, int C>
-__global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_ifftc(const FwdArgs a) {
-  using TL = CTile<M, C>;
-  constexpr int NT = TL::NT, H = TL::H, SR = TL::SR, SC = TL::SC;
-  cg::cluster_group cl = cg::this_cluster();
-  const int rank = (int)cl.block_rank();
-  extern __shared__ float2 sm[];
-  float2* rowbuf = sm;
-  float2* colbuf = sm + H * SR;
-  const int tid = threadIdx.x;
-  const int t = blockIdx.x / C;
-  const float2* x = a.in + (size_t)t * M * M;
-  const float sc = 1.f / (float)(M * M);
-  cluster_arrive_relaxed();
-  for (int p = tid; p < M * H; p += NT) {
-    const int er = p / H, lc = p % H, ec = rank * H + lc;
-    colbuf[er * SC + lc] = cscale(x[(size_t)storage_to_freq<M>(er) * M + storage_to_freq<M>(ec)], sc);
-  }
-  __syncthreads();
-  gpass_b<M, H, 1, SC, NT, true>(colbuf, tid);
-  __syncthreads();
-  gpass_a_inv<M, H, 1, SC, NT>(colbuf, tid);
-  __syncthreads();
-  cl.barrier_wait();
-  cluster_cols_to_rows<M, C>(cl, rank, colbuf, rowbuf, tid);
-  cl.sync();
-  gpass_b<M, H, SR, 1, NT, true>(rowbuf, tid);
-  __syncthreads();
-  gpass_a_inv<M, H, SR, 1, NT>(rowbuf, tid);
-  __syncthreads();
-  float2* y = a.out + (size_t)t * M * M + rank * H * M;
-  for (int p = tid; p < H * M; p += NT) y[p] = rowbuf[(p / M) * SR + p % M];
-}
-
 // ---------------------------------------------------------------------------
 // Wirtinger gradient of the exit-wave misfit per position (Sec. 2.1), with the
 // revised exit wave recomputed: forward FFT, modulus replacement, inverse FFT,
 // then gz = conj(Q) (psi - R), gq = conj(z_k) (psi - R) on the patch.
-template <int M, int C>
-__global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_gradc(const GradArgs a) {
-  using TL = CTile<M, C>;
-  constexpr int NT = TL::NT, H = TL::H, SR = TL::SR, SC = TL::SC, N1 = TL::N1, N2 = TL::N2, SLOTS = TL::SLOTS;
+// One slab per CTA, a_k by cp.async beside it, z_k read again from L2 at the
+// end: 32 warps per SM (as for the forward kernels and the step at m = 256).
+template <int M>
+__global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_gradc(const GradArgs a) {
+  using TL = WaveTile<M>;
+  constexpr int NT = TL::NT, H = TL::H, S = TL::S, N1 = TL::N1, C = TL::CTAS, SLOTS = TL::SLOTS, PER = TL::PER;
   cg::cluster_group cl = cg::this_cluster();
-  const int rank = (int)cl.block_rank();
-  extern __shared__ float2 sm[];
-  float2* rowbuf = sm;
-  float2* colbuf = sm + H * SR;
-  float2* zbuf = colbuf + M * SC;
+  const int rank = C == 1 ? 0 : (int)cl.block_rank();
+  extern __shared__ __align__(16) float2 sm[];
+  float* ampbuf = reinterpret_cast<float*>(sm + TL::slab);  // a_k on my storage columns, [M][H]
   __shared__ double xd[C];
-  __shared__ float redf[NT / 32];
+  __shared__ float redf[(NT + 31) / 32];
   const int tid = threadIdx.x;
   const int kb = blockIdx.x / C;
   const int k = a.first + kb;
   const int o_r = a.pos[2 * k], o_c = a.pos[2 * k + 1];
   const int row0 = rank * H;
-  constexpr int PER = TL::PER;
-  // amplitudes of my spectral slots: issued now, consumed after the row passes
-  float am_reg[SLOTS][N1];
   {
-    const float* amp = a.amp + (size_t)k * M * M + rank * H;
+    const float* amp = a.amp + (size_t)k * M * M + row0;
 #pragma unroll
-    for (int t = 0; t < SLOTS; ++t) {
-      const int s = tid + t * NT, k2 = s / H, lc = s % H;
-#pragma unroll
-      for (int i = 0; i < N1; ++i) am_reg[t][i] = __ldg(amp + (i + N1 * k2) * M + lc);
-    }
+    for (int q = tid; q < M * H / 4; q += NT)
+      cp_async16(ampbuf + 4 * q, amp + (q / (H / 4)) * M + 4 * (q % (H / 4)));
+    cp_async_commit();
   }
-  cluster_arrive_relaxed();
-  // gather: the loads of 8 pixels of a thread in flight together
-#pragma unroll 8
+  constexpr int UL = PER < 8 ? PER : 8;
+#pragma unroll (UL)
   for (int t = 0; t < PER; ++t) {
-    const int p = tid + t * NT;
-    const int lr = p / M, c = p % M, r = row0 + lr;
-    const float2 zk = gather_obj(a.object, a.n_rows, a.n_cols, o_r + r, o_c + c);
-    zbuf[p] = zk;
-    rowbuf[lr * SR + c] = cmul(a.probe[r * M + c], zk);
+    const int p = tid + t * NT, lr = p / M, c = p % M, r = row0 + lr;
+    sm[lr * S + c] = cmul(a.probe[r * M + c], gather_obj(a.object, a.n_rows, a.n_cols, o_r + r, o_c + c));
   }
   __syncthreads();
-  gpass_a_fwd<M, H, SR, 1, NT>(rowbuf, tid);
+  gpass_a_fwd<M, H, S, 1, NT>(sm, tid);
+  cp_async_wait_all();  // a_k; the barriers below show it to the whole CTA
   __syncthreads();
-  gpass_b<M, H, SR, 1, NT, false>(rowbuf, tid);
-  __syncthreads();
-  cl.barrier_wait();
-  cluster_rows_to_cols<M, C>(cl, rank, rowbuf, colbuf, tid);
-  cl.sync();
-  gpass_a_fwd<M, H, 1, SC, NT>(colbuf, tid);
+  row_pass_b_to_cols<TL>(cl, rank, sm, sm, tid);
+  tile_sync<C>(cl);
+  gpass_a_fwd<M, H, S, 1, NT>(sm, tid);
   __syncthreads();
   const float inv_m2 = 1.f / (float)(M * M);
   float acc = 0.f;
 #pragma unroll
   for (int t = 0; t < SLOTS; ++t) {
     const int s = tid + t * NT, k2 = s / H, lc = s % H;
+    float2* p = sm + lc * S + N1 * k2;
     float2 v[N1];
 #pragma unroll
-    for (int i = 0; i < N1; ++i) v[i] = colbuf[(i + N1 * k2) * SC + lc];
+    for (int i = 0; i < N1; ++i) v[i] = p[i];
     Dft<N1, false>::run(v);
 #pragma unroll
     for (int i = 0; i < N1; ++i) {
-      const float am = am_reg[t][i];
+      const float am = ampbuf[(i + N1 * k2) * H + lc];
       const float p2 = cabs2(v[i]);
       if (p2 > 0.f) {
         const float inv = rsqrtf(p2);
@@ -1800,41 +1801,38 @@ __global__ void __launch_bounds__(CTile<M, C>::NT, 1) k_gradc(const GradArgs a) 
     }
     Dft<N1, true>::run(v);
 #pragma unroll
-    for (int i = 0; i < N1; ++i) colbuf[(i + N1 * k2) * SC + lc] = v[i];
+    for (int i = 0; i < N1; ++i) p[i] = v[i];
   }
-  __syncthreads();
-  gpass_a_inv<M, H, 1, SC, NT>(colbuf, tid);
-  // per-warp misfit partials; the barrier also orders the pass before the transpose
+  // per-warp misfit partials; the barrier also orders the pass before the next one
   warp_partial_sum(acc, redf);
   __syncthreads();
-  cluster_cols_to_rows<M, C>(cl, rank, colbuf, rowbuf, tid);
-  if (tid == 0) cluster_publish<C>(cl, rank, xd, partials_sum<NT>(redf));
-  cl.sync();
-  gpass_b<M, H, SR, 1, NT, true>(rowbuf, tid);
+  // rank 0 collects the parts (every CTA has started: the row pass waited for them all)
+  if (tid == 0) *tile_rank<C>(cl, rank, &xd[rank], 0) = partials_sum<NT>(redf);
+  col_pass_a_inv_to_rows<TL>(cl, rank, sm, sm, tid);
+  tile_sync<C>(cl);
+  gpass_b<M, H, S, 1, NT, true>(sm, tid);
   __syncthreads();
-  gpass_a_inv<M, H, SR, 1, NT>(rowbuf, tid);
+  gpass_a_inv<M, H, S, 1, NT>(sm, tid);
   __syncthreads();
   float2* gz = a.gz + (size_t)kb * M * M;
   float2* gq = a.gq + (size_t)kb * M * M;
-  // patch gradients; the probe loads of 8 pixels of a thread are issued together
-  constexpr int UG = PER < 8 ? PER : 8;
+  // patch gradients; the loads of UG pixels of a thread are issued together
+  constexpr int UG = PER < 4 ? PER : 4;
 #pragma unroll 1
   for (int t0 = 0; t0 < PER; t0 += UG) {
-    float2 qv[UG];
+    float2 qv[UG], zv[UG];
 #pragma unroll
     for (int u = 0; u < UG; ++u) {
-      const int p = tid + (t0 + u) * NT;
-      qv[u] = __ldg(a.probe + (row0 + p / M) * M + p % M);
+      const int p = tid + (t0 + u) * NT, r = row0 + p / M, c = p % M;
+      qv[u] = __ldg(a.probe + r * M + c);
+      zv[u] = gather_obj(a.object, a.n_rows, a.n_cols, o_r + r, o_c + c);
     }
 #pragma unroll
     for (int u = 0; u < UG; ++u) {
-      const int p = tid + (t0 + u) * NT;
-      const int lr = p / M, c = p % M, r = row0 + lr;
-      const float2 zk = zbuf[p];
-      const float2 q = qv[u];
-      const float2 e = csub(cmul(q, zk), rowbuf[lr * SR + c]);
-      gz[r * M + c] = cconjmul(q, e);
-      gq[r * M + c] = cconjmul(zk, e);
+      const int p = tid + (t0 + u) * NT, lr = p / M, c = p % M, r = row0 + lr;
+      const float2 e = csub(cmul(qv[u], zv[u]), sm[lr * S + c]);
+      gz[r * M + c] = cconjmul(qv[u], e);
+      gq[r * M + c] = cconjmul(zv[u], e);
     }
   }
   if (rank == 0 && tid == 0) {
@@ -2142,47 +2140,8 @@ __global__ void __launch_bounds__(kApplyThreads, EMG_APPLY_MIN_BLOCKS) k_apply(c
 }
 
 // ---------------------------------------------------------------------------
-// Phi_k = (1/2 M^2) sum (|F psi| - a_k)^2 per position (Parseval form of Eq. exit_misfit).
-template <int M>
-__global__ void __launch_bounds__(StepThreads<M>::value)
-    k_misfit(const float2* __restrict__ object, const float2* __restrict__ probe,
-             const int32_t* __restrict__ pos, const float* __restrict__ amp, int n_rows, int n_cols,
-             double* __restrict__ partial) {
-  constexpr int NT = StepThreads<M>::value;
-  constexpr int S = M + 1;
-  constexpr int N1 = FftPlan<M>::N1, N2 = FftPlan<M>::N2;
-  extern __shared__ float2 sm[];
-  __shared__ double redd[NT / 32];
-  const int tid = threadIdx.x;
-  const int k = blockIdx.x;
-  const int o_r = pos[2 * k], o_c = pos[2 * k + 1];
-  float2* buf = sm;
-  for (int p = tid; p < M * M; p += NT) {
-    const int r = p / M, c = p % M;
-    buf[r * S + c] = cmul(probe[p], gather_obj(object, n_rows, n_cols, o_r + r, o_c + c));
-  }
-  __syncthreads();
-  fft2_fwd_until_col_b<M, NT>(buf, tid);
-  const float* ak = amp + (size_t)k * M * M;
-  float acc = 0.f;
-  for (int s = tid; s < M * N2; s += NT) {
-    const int k2 = s / M, c = s % M;
-    float2 v[N1];
-#pragma unroll
-    for (int i = 0; i < N1; ++i) v[i] = buf[(i + N1 * k2) * S + c];
-    Dft<N1, false>::run(v);
-#pragma unroll
-    for (int i = 0; i < N1; ++i) {
-      const float dm = sqrtf(cabs2(v[i])) - ak[(i + N1 * k2) * M + c];
-      acc = fmaf(dm, dm, acc);
-    }
-  }
-  const double tot = block_sum<NT>((double)acc, redd);
-  if (tid == 0) partial[k] = tot * (0.5 / (double)(M * M));
-}
-
 // Deterministic single-block sum: out = scale * sum x[0..n).
-constexpr int kSumThreads = 1024;
+constexpr int kSumThreads = 256;  // 1024 threads: 13.8 us for 1444 values, most of it the FP64 trees
 __global__ void __launch_bounds__(kSumThreads) k_sum(const double* __restrict__ x, int n,
                                                      double scale, double* __restrict__ out) {
   __shared__ double redd[kSumThreads / 32];
@@ -2190,69 +2149,6 @@ __global__ void __launch_bounds__(kSumThreads) k_sum(const double* __restrict__ 
   for (int i = threadIdx.x; i < n; i += kSumThreads) s += x[i];
   s = block_sum<kSumThreads>(s, redd);
   if (threadIdx.x == 0) *out = s * scale;
-}
-
-// ---------------------------------------------------------------------------
-// Data model of Sec. 2.1: d_k = |F(Q . P_k z)|^2 in natural order.
-template <int M>
-__global__ void __launch_bounds__(StepThreads<M>::value)
-    k_simulate(const float2* __restrict__ object, const float2* __restrict__ probe,
-               const int32_t* __restrict__ pos, int n_rows, int n_cols, float* __restrict__ out) {
-  constexpr int NT = StepThreads<M>::value;
-  constexpr int S = M + 1;
-  extern __shared__ float2 sm[];
-  const int tid = threadIdx.x;
-  const int k = blockIdx.x;
-  const int o_r = pos[2 * k], o_c = pos[2 * k + 1];
-  float2* buf = sm;
-  for (int p = tid; p < M * M; p += NT) {
-    const int r = p / M, c = p % M;
-    buf[r * S + c] = cmul(probe[p], gather_obj(object, n_rows, n_cols, o_r + r, o_c + c));
-  }
-  __syncthreads();
-  fft2_fwd_until_col_b<M, NT>(buf, tid);
-  pass_b<M, true, NT, false>(buf, tid);
-  __syncthreads();
-  float* dk = out + (size_t)k * M * M;
-  for (int p = tid; p < M * M; p += NT) {
-    const int er = p / M, ec = p % M;
-    dk[storage_to_freq<M>(er) * M + storage_to_freq<M>(ec)] = cabs2(buf[er * S + ec]);
-  }
-}
-
-// Batched 2-D DFT of natural-order tiles.
-template <int M>
-__global__ void __launch_bounds__(StepThreads<M>::value)
-    k_fft2(const float2* in, float2* out, int inverse) {
-  constexpr int NT = StepThreads<M>::value;
-  constexpr int S = M + 1;
-  extern __shared__ float2 sm[];
-  const int tid = threadIdx.x;
-  const float2* x = in + (size_t)blockIdx.x * M * M;
-  float2* y = out + (size_t)blockIdx.x * M * M;
-  float2* buf = sm;
-  if (!inverse) {
-    for (int p = tid; p < M * M; p += NT) buf[(p / M) * S + p % M] = x[p];
-    __syncthreads();
-    fft2_fwd_until_col_b<M, NT>(buf, tid);
-    pass_b<M, true, NT, false>(buf, tid);
-    __syncthreads();
-    for (int p = tid; p < M * M; p += NT) {
-      const int er = p / M, ec = p % M;
-      y[storage_to_freq<M>(er) * M + storage_to_freq<M>(ec)] = buf[er * S + ec];
-    }
-  } else {
-    const float s = 1.f / (float)(M * M);
-    for (int p = tid; p < M * M; p += NT) {
-      const int er = p / M, ec = p % M;
-      buf[er * S + ec] = cscale(x[storage_to_freq<M>(er) * M + storage_to_freq<M>(ec)], s);
-    }
-    __syncthreads();
-    pass_b<M, true, NT, true>(buf, tid);
-    __syncthreads();
-    fft2_inv_after_col_b<M, NT>(buf, tid);
-    for (int p = tid; p < M * M; p += NT) y[p] = buf[(p / M) * S + p % M];
-  }
 }
 
 // dp_avg probe scaling (Sec. 4.1): partial sums of a^2 = max(d, 0).
@@ -2270,19 +2166,20 @@ __global__ void __launch_bounds__(kNormThreads) k_sum_sq(const float* __restrict
   if (threadIdx.x == 0) partial[blockIdx.x] = s;
 }
 
-__global__ void __launch_bounds__(kSumThreads) k_scale_probe(const double* __restrict__ partial,
+constexpr int kScaleThreads = 1024;
+__global__ void __launch_bounds__(kScaleThreads) k_scale_probe(const double* __restrict__ partial,
                                                              int n_partial, int m, int n_pos,
                                                              float2* __restrict__ probe) {
-  __shared__ double redd[kSumThreads / 32];
+  __shared__ double redd[kScaleThreads / 32];
   double s = 0.0;
-  for (int i = threadIdx.x; i < n_partial; i += kSumThreads) s += partial[i];
-  const double sum_d = block_sum<kSumThreads>(s, redd);
+  for (int i = threadIdx.x; i < n_partial; i += kScaleThreads) s += partial[i];
+  const double sum_d = block_sum<kScaleThreads>(s, redd);
   double q2 = 0.0;
-  for (int p = threadIdx.x; p < m * m; p += kSumThreads) q2 += (double)cabs2(probe[p]);
-  const double norm2 = block_sum<kSumThreads>(q2, redd);
+  for (int p = threadIdx.x; p < m * m; p += kScaleThreads) q2 += (double)cabs2(probe[p]);
+  const double norm2 = block_sum<kScaleThreads>(q2, redd);
   const double dp_avg = sqrt(sum_d / (double)n_pos) / (double)m;
   const float scale = norm2 > 0.0 ? (float)(dp_avg / sqrt(norm2)) : 0.f;
-  for (int p = threadIdx.x; p < m * m; p += kSumThreads) probe[p] = cscale(probe[p], scale);
+  for (int p = threadIdx.x; p < m * m; p += kScaleThreads) probe[p] = cscale(probe[p], scale);
 }
 
 template <int M>
@@ -2298,48 +2195,13 @@ cudaError_t launch_step_t(int b, const StepArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <int M>
-cudaError_t launch_misfit_t(const float2* object, const float2* probe, const int32_t* pos,
-                            const float* amp, int n_rows, int n_cols, int n_pos, double* partial,
-                            cudaStream_t s) {
-  const size_t bytes = level_floats2<M>(0) * sizeof(float2);
-  k_misfit<M><<<n_pos, StepThreads<M>::value, bytes, s>>>(object, probe, pos, amp, n_rows, n_cols,
-                                                          partial);
-  return cudaGetLastError();
-}
-
-template <int M>
-cudaError_t launch_simulate_t(const float2* object, const float2* probe, const int32_t* pos,
-                              int n_rows, int n_cols, int n_pos, float* out, cudaStream_t s) {
-  const size_t bytes = level_floats2<M>(0) * sizeof(float2);
-  k_simulate<M><<<n_pos, StepThreads<M>::value, bytes, s>>>(object, probe, pos, n_rows, n_cols, out);
-  return cudaGetLastError();
-}
-
-template <int M>
-cudaError_t launch_fft2_t(const float2* in, float2* out, int count, int inverse, cudaStream_t s) {
-  const size_t bytes = level_floats2<M>(0) * sizeof(float2);
-  k_fft2<M><<<count, StepThreads<M>::value, bytes, s>>>(in, out, inverse);
-  return cudaGetLastError();
-}
-
-template <int M>
-cudaError_t set_aux_smem() {
-  const int bytes = (int)(level_floats2<M>(0) * sizeof(float2));
-  cudaError_t e = cudaFuncSetAttribute(k_misfit<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_simulate<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_fft2<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  return e;
-}
-
 #define EMG_DISPATCH_M(m, CALL)        \
   switch (m) {                         \
     case 16: { constexpr int M = 16; return CALL; }   \
     case 32: { constexpr int M = 32; return CALL; }   \
     case 64: { constexpr int M = 64; return CALL; }   \
     case 128: { constexpr int M = 128; return CALL; } \
+    case 256: { constexpr int M = 256; return CALL; } \
     default: return cudaErrorInvalidValue;            \
   }
 
@@ -2392,10 +2254,6 @@ cudaError_t upload_twiddles() {
   if ((e = set_step_smem<64>()) != cudaSuccess) return e;
   if ((e = set_step_smem<128>()) != cudaSuccess) return e;
   if ((e = set_cluster_attrs()) != cudaSuccess) return e;
-  if ((e = set_aux_smem<16>()) != cudaSuccess) return e;
-  if ((e = set_aux_smem<32>()) != cudaSuccess) return e;
-  if ((e = set_aux_smem<64>()) != cudaSuccess) return e;
-  if ((e = set_aux_smem<128>()) != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_prep_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPrepTileSmemMax);
@@ -2574,30 +2432,34 @@ cudaError_t launch_cluster_plain(Kernel kernel, int cluster, dim3 grid, dim3 blo
 }
 
 template <int M, int MODE>
-cudaError_t launch_fwdc_t(int count, const FwdArgs& a, cudaStream_t s) {
-  constexpr int C = ClusterSize<M>::value;
-  using TL = CTile<M, C>;
-  cudaError_t e = launch_cluster_plain(k_fwdc<M, C, MODE>, C, dim3(C * count), dim3(TL::NT),
-                                       TL::smem_elems * sizeof(float2), s, a);
-  return e != cudaSuccess ? e : cudaGetLastError();
+cudaError_t launch_forward_t(int count, const FwdArgs& a, cudaStream_t s) {
+  using TL = WaveTile<M>;
+  constexpr size_t bytes = TL::slab * sizeof(float2);
+  if constexpr (TL::CTAS == 1) {
+    k_forward<M, MODE><<<count, TL::NT, bytes, s>>>(a);
+  } else {
+    cudaError_t e = launch_cluster_plain(k_forward<M, MODE>, TL::CTAS, dim3(TL::CTAS * count), dim3(TL::NT), bytes, s, a);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaGetLastError();
 }
 
 template <int M>
-cudaError_t launch_ifftc_t(int count, const FwdArgs& a, cudaStream_t s) {
-  constexpr int C = ClusterSize<M>::value;
-  using TL = CTile<M, C>;
-  cudaError_t e = launch_cluster_plain(k_ifftc<M, C>, C, dim3(C * count), dim3(TL::NT),
-                                       TL::smem_elems * sizeof(float2), s, a);
-  return e != cudaSuccess ? e : cudaGetLastError();
+constexpr size_t gradc_smem_elems() {
+  return WaveTile<M>::slab + (size_t)WaveTile<M>::H * M / 2;
 }
 
 template <int M>
 cudaError_t launch_gradc_t(int b, const GradArgs& a, cudaStream_t s) {
-  constexpr int C = ClusterSize<M>::value;
-  using TL = CTile<M, C>;
-  cudaError_t e = launch_cluster_plain(k_gradc<M, C>, C, dim3(C * b), dim3(TL::NT),
-                                       TL::smem_elems * sizeof(float2), s, a);
-  return e != cudaSuccess ? e : cudaGetLastError();
+  using TL = WaveTile<M>;
+  constexpr size_t bytes = gradc_smem_elems<M>() * sizeof(float2);
+  if constexpr (TL::CTAS == 1) {
+    k_gradc<M><<<b, TL::NT, bytes, s>>>(a);
+  } else {
+    cudaError_t e = launch_cluster_plain(k_gradc<M>, TL::CTAS, dim3(TL::CTAS * b), dim3(TL::NT), bytes, s, a);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaGetLastError();
 }
 
 template <typename Kernel>
@@ -2611,9 +2473,17 @@ cudaError_t set_stepc_attrs() {
 }
 
 template <int M>
+cudaError_t set_forward_attrs() {
+  cudaError_t e;
+  if ((e = set_cluster_smem(k_forward<M, 0>, WaveTile<M>::slab)) != cudaSuccess) return e;
+  if ((e = set_cluster_smem(k_forward<M, 1>, WaveTile<M>::slab)) != cudaSuccess) return e;
+  if ((e = set_cluster_smem(k_forward<M, 2>, WaveTile<M>::slab)) != cudaSuccess) return e;
+  return set_cluster_smem(k_forward<M, 3>, WaveTile<M>::slab);
+}
+
+template <int M>
 cudaError_t set_grad_attrs() {
-  constexpr int C = ClusterSize<M>::value;
-  return set_cluster_smem(k_gradc<M, C>, CTile<M, C>::smem_elems);
+  return set_cluster_smem(k_gradc<M>, gradc_smem_elems<M>());
 }
 
 // Dynamic shared-memory limits of the cluster kernels (once per device).
@@ -2631,10 +2501,11 @@ cudaError_t set_cluster_attrs() {
   if ((e = set_stepc_attrs<128, 4, true>()) != cudaSuccess) return e;
   if ((e = set_stepc_attrs<128, 8, true>()) != cudaSuccess) return e;
   if ((e = set_stepc_attrs<256, 8, true>()) != cudaSuccess) return e;
-  if ((e = set_cluster_smem(k_fwdc<256, 8, 0>, CTile<256, 8>::smem_elems)) != cudaSuccess) return e;
-  if ((e = set_cluster_smem(k_fwdc<256, 8, 1>, CTile<256, 8>::smem_elems)) != cudaSuccess) return e;
-  if ((e = set_cluster_smem(k_fwdc<256, 8, 2>, CTile<256, 8>::smem_elems)) != cudaSuccess) return e;
-  if ((e = set_cluster_smem(k_ifftc<256, 8>, CTile<256, 8>::smem_elems)) != cudaSuccess) return e;
+  if ((e = set_forward_attrs<16>()) != cudaSuccess) return e;
+  if ((e = set_forward_attrs<32>()) != cudaSuccess) return e;
+  if ((e = set_forward_attrs<64>()) != cudaSuccess) return e;
+  if ((e = set_forward_attrs<128>()) != cudaSuccess) return e;
+  if ((e = set_forward_attrs<256>()) != cudaSuccess) return e;
   if ((e = set_grad_attrs<16>()) != cudaSuccess) return e;
   if ((e = set_grad_attrs<32>()) != cudaSuccess) return e;
   if ((e = set_grad_attrs<64>()) != cudaSuccess) return e;
@@ -2734,18 +2605,15 @@ cudaError_t launch_apply(const ApplyArgs& a, cudaStream_t s) {
 cudaError_t launch_misfit(int m, const float2* object, const float2* probe, const int32_t* pos,
                           const float* amp, int n_rows, int n_cols, int n_pos, double* partial,
                           cudaStream_t s) {
-  if (m == 256) {
-    FwdArgs f{};
-    f.object = object;
-    f.probe = probe;
-    f.pos = pos;
-    f.amp = amp;
-    f.n_rows = n_rows;
-    f.n_cols = n_cols;
-    f.partial = partial;
-    return launch_fwdc_t<256, 0>(n_pos, f, s);
-  }
-  EMG_DISPATCH_M(m, (launch_misfit_t<M>(object, probe, pos, amp, n_rows, n_cols, n_pos, partial, s)));
+  FwdArgs f{};
+  f.object = object;
+  f.probe = probe;
+  f.pos = pos;
+  f.amp = amp;
+  f.n_rows = n_rows;
+  f.n_cols = n_cols;
+  f.partial = partial;
+  EMG_DISPATCH_M(m, (launch_forward_t<M, 0>(n_pos, f, s)));
 }
 
 cudaError_t launch_sum(const double* x, int n, double scale, double* out, cudaStream_t s) {
@@ -2755,47 +2623,52 @@ cudaError_t launch_sum(const double* x, int n, double scale, double* out, cudaSt
 
 cudaError_t launch_simulate(int m, const float2* object, const float2* probe, const int32_t* pos,
                             int n_rows, int n_cols, int n_pos, float* out, cudaStream_t s) {
-  if (m == 256) {
-    FwdArgs f{};
-    f.object = object;
-    f.probe = probe;
-    f.pos = pos;
-    f.n_rows = n_rows;
-    f.n_cols = n_cols;
-    f.out_intensity = out;
-    return launch_fwdc_t<256, 1>(n_pos, f, s);
-  }
-  EMG_DISPATCH_M(m, (launch_simulate_t<M>(object, probe, pos, n_rows, n_cols, n_pos, out, s)));
+  FwdArgs f{};
+  f.object = object;
+  f.probe = probe;
+  f.pos = pos;
+  f.n_rows = n_rows;
+  f.n_cols = n_cols;
+  f.out_intensity = out;
+  EMG_DISPATCH_M(m, (launch_forward_t<M, 1>(n_pos, f, s)));
 }
 
 cudaError_t launch_fft2(int m, const float2* in, float2* out, int count, int inverse,
                         cudaStream_t s) {
-  if (m == 256) {
-    FwdArgs f{};
-    f.in = in;
-    f.out = out;
-    return inverse ? launch_ifftc_t<256>(count, f, s) : launch_fwdc_t<256, 2>(count, f, s);
-  }
-  EMG_DISPATCH_M(m, (launch_fft2_t<M>(in, out, count, inverse, s)));
+  FwdArgs f{};
+  f.in = in;
+  f.out = out;
+  if (inverse) EMG_DISPATCH_M(m, (launch_forward_t<M, 3>(count, f, s)));
+  EMG_DISPATCH_M(m, (launch_forward_t<M, 2>(count, f, s)));
 }
 
 template <int M>
 int gradient_wave_t() {
-  constexpr int C = ClusterSize<M>::value;
-  using TL = CTile<M, C>;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(C * 4096);
-  cfg.blockDim = dim3(TL::NT);
-  cfg.dynamicSmemBytes = TL::smem_elems * sizeof(float2);
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = C;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  using TL = WaveTile<M>;
+  constexpr size_t bytes = gradc_smem_elems<M>() * sizeof(float2);
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, k_gradc<M, C>, &cfg) != cudaSuccess) {
+  cudaError_t e;
+  if constexpr (TL::CTAS == 1) {
+    int dev = 0, sms = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gradc<M>, TL::NT, bytes);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    n *= sms;
+  } else {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(TL::CTAS * 4096);
+    cfg.blockDim = dim3(TL::NT);
+    cfg.dynamicSmemBytes = bytes;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = TL::CTAS;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    e = cudaOccupancyMaxActiveClusters(&n, k_gradc<M>, &cfg);
+  }
+  if (e != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -2856,7 +2729,7 @@ cudaError_t launch_normalize_probe(const float* amp, int m, int n_pos, float2* p
   k_sum_sq<<<blocks, kNormThreads, 0, s>>>(amp, n, scratch);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_scale_probe<<<1, kSumThreads, 0, s>>>(scratch, blocks, m, n_pos, probe);
+  k_scale_probe<<<1, kScaleThreads, 0, s>>>(scratch, blocks, m, n_pos, probe);
   return cudaGetLastError();
 }
 
