@@ -915,6 +915,16 @@ emg_status set_intensity_impl(emg_ctx* c, const float* intensity) {
   return EMG_OK;
 }
 
+// Sum of d_phi[0..n) (FP64), synchronising.
+emg_status read_misfit_sum(emg_ctx* c, int n, double* out) {
+  cudaError_t e = emg::launch_sum(c->d_phi, n, 1.0, c->d_scalar, c->stream);
+  if (e != cudaSuccess) return cuda_fail(c, e, "k_sum launch");
+  EMG_CUDA(c, cudaMemcpyAsync(c->h_scalar, c->d_scalar, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  EMG_CUDA(c, cudaStreamSynchronize(c->stream));
+  *out = c->h_scalar[0];
+  return EMG_OK;
+}
+
 // Phi of the bound state (FP64 sum), synchronising.
 emg_status misfit_now(emg_ctx* c, double* out) {
   cudaError_t e = emg::launch_misfit(c->m, c->object, c->probe, c->d_pos, c->d_amp, c->n_rows, c->n_cols,
@@ -1401,6 +1411,14 @@ emg_status emg_misfit_gradient(emg_ctx* c, const float* object, const float* pro
   if (!object || !probe) return fail(c, EMG_EINVAL, "object or probe is NULL");
   DeviceGuard g(c->device);
   const int N = c->n_pos;
+  if (!grad_object && !grad_probe) {
+    // the misfit alone: the forward transforms, without the inverse ones and the patch gradients
+    cudaError_t e = emg::launch_misfit(c->m, (const float2*)object, (const float2*)probe, c->d_pos, c->d_amp, c->n_rows,
+                                       c->n_cols, N, c->d_phi, c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "k_forward launch");
+    c->launches[kKindOther] += 1;
+    return misfit ? read_misfit_sum(c, N, misfit) : EMG_OK;
+  }
   if (c->grad_chunk == 0) {
     // By default a multiple of the position clusters that can be resident at
     // once, about 128 positions per launch; the chunking fixes the order of the sums.
@@ -1419,12 +1437,11 @@ emg_status emg_misfit_gradient(emg_ctx* c, const float* object, const float* pro
     c->grad_chunk = chunk;
   }
   const int B = c->grad_chunk;
-  const bool sums = grad_object || grad_probe;
-  // With the sums asked for and more than one chunk, the sums of chunk i run on
+  // With more than one chunk, the sums of chunk i run on
   // the side stream while chunk i + 1's patches are computed into the other
   // buffer pair; the sums stay in chunk order on the side stream, so the
   // result is the same bitwise.  Without a second pair the chunks run in turn.
-  bool overlap = sums && N > B;
+  bool overlap = N > B;
   if (overlap && !c->d_gz2) {
     const size_t bytes = (size_t)B * c->m * c->m * sizeof(float2);
     if (cudaMalloc(&c->d_gz2, bytes) != cudaSuccess || cudaMalloc(&c->d_gq2, bytes) != cudaSuccess) {
@@ -1461,44 +1478,35 @@ emg_status emg_misfit_gradient(emg_ctx* c, const float* object, const float* pro
     cudaError_t e = emg::launch_gradient(c->m, b, ga, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "k_gradc launch");
     c->launches[kKindOther] += 1;
-    if (sums) {
-      const cudaStream_t rs = overlap ? c->side : c->stream;
-      if (overlap) {
-        EMG_CUDA(c, cudaEventRecord(c->ev_grad[0], c->stream));
-        EMG_CUDA(c, cudaStreamWaitEvent(c->side, c->ev_grad[0], 0));
-      }
-      emg::GradReduceArgs ra{};
-      ra.pos = c->d_pos;
-      ra.first = first;
-      ra.b = b;
-      ra.n_rows = c->n_rows;
-      ra.n_cols = c->n_cols;
-      ra.m = c->m;
-      ra.accumulate = first > 0;
-      ra.gz = gz;
-      ra.gq = gq;
-      ra.grad_object = (float2*)grad_object;
-      ra.grad_probe = (float2*)grad_probe;
-      ra.tiles_x = (c->n_cols + emg::kApplyTile - 1) / emg::kApplyTile;
-      ra.tiles_y = (c->n_rows + emg::kApplyTile - 1) / emg::kApplyTile;
-      e = emg::launch_grad_reduce(ra, rs);
-      if (e != cudaSuccess) return cuda_fail(c, e, "k_grad_reduce launch");
-      c->launches[kKindOther] += 1;
-      if (overlap) EMG_CUDA(c, cudaEventRecord(c->ev_grad[1 + pair], c->side));
+    const cudaStream_t rs = overlap ? c->side : c->stream;
+    if (overlap) {
+      EMG_CUDA(c, cudaEventRecord(c->ev_grad[0], c->stream));
+      EMG_CUDA(c, cudaStreamWaitEvent(c->side, c->ev_grad[0], 0));
     }
+    emg::GradReduceArgs ra{};
+    ra.pos = c->d_pos;
+    ra.first = first;
+    ra.b = b;
+    ra.n_rows = c->n_rows;
+    ra.n_cols = c->n_cols;
+    ra.m = c->m;
+    ra.accumulate = first > 0;
+    ra.gz = gz;
+    ra.gq = gq;
+    ra.grad_object = (float2*)grad_object;
+    ra.grad_probe = (float2*)grad_probe;
+    ra.tiles_x = (c->n_cols + emg::kApplyTile - 1) / emg::kApplyTile;
+    ra.tiles_y = (c->n_rows + emg::kApplyTile - 1) / emg::kApplyTile;
+    e = emg::launch_grad_reduce(ra, rs);
+    if (e != cudaSuccess) return cuda_fail(c, e, "k_grad_reduce launch");
+    c->launches[kKindOther] += 1;
+    if (overlap) EMG_CUDA(c, cudaEventRecord(c->ev_grad[1 + pair], c->side));
   }
   if (overlap) {  // the caller's stream sees every sum
     EMG_CUDA(c, cudaEventRecord(c->ev_grad[0], c->side));
     EMG_CUDA(c, cudaStreamWaitEvent(c->stream, c->ev_grad[0], 0));
   }
-  if (misfit) {
-    cudaError_t e = emg::launch_sum(c->d_phi, N, 1.0, c->d_scalar, c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "k_sum launch");
-    EMG_CUDA(c, cudaMemcpyAsync(c->h_scalar, c->d_scalar, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    EMG_CUDA(c, cudaStreamSynchronize(c->stream));
-    *misfit = c->h_scalar[0];
-  }
-  return EMG_OK;
+  return misfit ? read_misfit_sum(c, N, misfit) : EMG_OK;
 }
 
 emg_status emg_set_gradient_chunk(emg_ctx* c, int32_t positions) {
