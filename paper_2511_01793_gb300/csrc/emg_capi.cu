@@ -1920,6 +1920,7 @@ void emg_destroy(emg_ctx* c) {
     if (c->stream) cudaStreamSynchronize(c->stream);
     else cudaDeviceSynchronize();
     free_all(c);
+    emg::scratch_trim(c->device);
   }
   delete c;
 }

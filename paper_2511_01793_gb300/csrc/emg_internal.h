@@ -113,7 +113,7 @@ struct ApplyArgs {
   float* s_den;
 };
 
-// Forward-only cluster kernels (m up to 256): misfit partials, simulated
+// Forward-only kernels: misfit partials, simulated
 // intensities, forward / inverse 2-D DFT of natural-order tiles.
 struct FwdArgs {
   const float2* object;
@@ -236,5 +236,8 @@ cudaError_t launch_tc_amp(const float* d, float* amp_t, int m, int n_pos, cudaSt
 // One bounded mbarrier wait that nothing satisfies; sets *err when it gives up.
 cudaError_t launch_wait_selftest(int* err, cudaStream_t s);
 int step_smem_limit();
+
+// Gives back what the scratch pool of the quality reductions keeps on `dev` (see emg_metrics.cu).
+void scratch_trim(int dev);
 
 }  // namespace emg

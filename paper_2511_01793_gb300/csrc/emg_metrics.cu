@@ -16,14 +16,17 @@
 // the scanned field, Sec. 4.1).
 //
 // Every sum is taken in FP64.  Each kernel uses a fixed grid and a fixed
-// reduction tree, and the partial sums are added in block order, so results
+// reduction tree, and the partial sums are added in a fixed order, so results
 // are bitwise repeatable.  The illumination of a pixel is summed over the
 // positions in index order, as a sequential loop would.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "../../include/emagpie.h"
+#include "emg_internal.h"
 
 namespace emg {
 namespace {
@@ -32,21 +35,66 @@ constexpr int kMetThreads = 256;
 constexpr int kMetBlocks = 304;  // 2 per SM on 152 SMs; fixed, so the sums are repeatable
 constexpr int kPosChunk = 512;   // positions staged in shared memory at a time
 
-struct D2 {
-  double x, y;
-};
+// Scratch of one call, from a stream-ordered pool of this library (one per
+// device): cudaMalloc and cudaFree cost more than the reductions themselves
+// (about 200 us of a call's 2.7 ms went into them and their synchronisation).
+// The driver orders reuse between streams and threads; the pool keeps at most
+// kScratchKeep bytes between calls and gives them back when a context is destroyed.
+constexpr size_t kScratchKeep = (size_t)64 << 20;
+std::mutex g_scratch_mu;
+cudaMemPool_t g_scratch_pool[256] = {nullptr};
 
-__device__ __forceinline__ double block_sum_d(double v, double* sh) {
-  const int tid = threadIdx.x;
-  sh[tid] = v;
-  __syncthreads();
-  for (int s = kMetThreads / 2; s > 0; s >>= 1) {
-    if (tid < s) sh[tid] += sh[tid + s];
-    __syncthreads();
+cudaError_t scratch_alloc(double** p, size_t words, cudaStream_t s) {
+  *p = nullptr;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess && (dev < 0 || dev >= 256)) e = cudaErrorInvalidDevice;
+  cudaMemPool_t pool = nullptr;
+  if (e == cudaSuccess) {
+    std::lock_guard<std::mutex> lk(g_scratch_mu);
+    if (!g_scratch_pool[dev]) {
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      cudaMemPool_t made = nullptr;
+      unsigned long long keep = kScratchKeep;
+      e = cudaMemPoolCreate(&made, &props);
+      if (e == cudaSuccess) {
+        e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e == cudaSuccess)
+          g_scratch_pool[dev] = made;
+        else
+          cudaMemPoolDestroy(made);
+      }
+    }
+    pool = g_scratch_pool[dev];
   }
-  const double r = sh[0];
+  if (e == cudaSuccess) e = cudaMallocFromPoolAsync((void**)p, words * sizeof(double), pool, s);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
+// The block's sums of N quantities into out[0..N): shuffle trees, then the
+// warps' values in warp order (one barrier for all of them).
+template <int N>
+__device__ __forceinline__ void block_sums(const double (&v)[N], double* out) {
+  __shared__ double sh[N][kMetThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    double s = v[j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) sh[j][warp] = s;
+  }
   __syncthreads();
-  return r;
+  if (threadIdx.x < N) {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < kMetThreads / 32; ++w) s += sh[threadIdx.x][w];
+    out[threadIdx.x] = s;
+  }
 }
 
 // Partial sums over the region: |z|^2, conj(z) z_ref (re, im), |z_ref|^2, count.
@@ -54,7 +102,6 @@ __global__ void __launch_bounds__(kMetThreads) k_align_pass1(const float2* __res
                                                              const float2* __restrict__ zr,
                                                              const uint8_t* __restrict__ region, size_t n,
                                                              double* __restrict__ part) {
-  __shared__ double sh[kMetThreads];
   double zz = 0.0, cr = 0.0, ci = 0.0, rr = 0.0, cnt = 0.0;
   for (size_t i = (size_t)blockIdx.x * kMetThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kMetThreads) {
     if (region && !region[i]) continue;
@@ -66,22 +113,34 @@ __global__ void __launch_bounds__(kMetThreads) k_align_pass1(const float2* __res
     rr += bx * bx + by * by;
     cnt += 1.0;
   }
-  double* out = part + (size_t)blockIdx.x * 5;
   const double v[5] = {zz, cr, ci, rr, cnt};
-#pragma unroll
-  for (int j = 0; j < 5; ++j) {
-    const double s = block_sum_d(v[j], sh);
-    if (threadIdx.x == 0) out[j] = s;
-  }
+  block_sums(v, part + (size_t)blockIdx.x * 5);
 }
 
-// Sums the per-block partials in block order; with `finish` = 0 it also forms
-// c = <z, z_ref> / <z, z> into res[0..1] (res[2] = ||z_ref||^2, res[3] = count).
-__global__ void k_align_final1(const double* __restrict__ part, int blocks, double* __restrict__ res) {
+// Sum of the kMetBlocks partials of one quantity (stride `words`) by one warp:
+// a fixed number per lane in block order, then a shuffle tree.  (One thread
+// that walked all partials took 90 us: a chain of dependent FP64 adds on loads.)
+__device__ __forceinline__ double warp_sum_partials(const double* part, int words) {
+  double s = 0.0;
+#pragma unroll
+  for (int i = 0; i < (kMetBlocks + 31) / 32; ++i) {
+    const int b = i * 32 + (threadIdx.x & 31);
+    if (b < kMetBlocks) s += part[(size_t)b * words];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// c = <z, z_ref> / <z, z> into res[0..1]; res[2] = ||z_ref||^2, res[3] = count.
+// One warp per summed quantity.
+__global__ void __launch_bounds__(160) k_align_final1(const double* __restrict__ part, double* __restrict__ res) {
+  __shared__ double s[5];
+  const int w = threadIdx.x >> 5;
+  const double v = warp_sum_partials(part + w, 5);
+  if ((threadIdx.x & 31) == 0) s[w] = v;
+  __syncthreads();
   if (threadIdx.x != 0) return;
-  double s[5] = {0, 0, 0, 0, 0};
-  for (int b = 0; b < blocks; ++b)
-    for (int j = 0; j < 5; ++j) s[j] += part[(size_t)b * 5 + j];
   res[0] = s[0] > 0.0 ? s[1] / s[0] : 0.0;
   res[1] = s[0] > 0.0 ? s[2] / s[0] : 0.0;
   res[2] = s[3];
@@ -97,7 +156,6 @@ __global__ void __launch_bounds__(kMetThreads) k_align_pass2(const float2* __res
                                                              const float2* __restrict__ qr, size_t nq,
                                                              const double* __restrict__ res,
                                                              double* __restrict__ part) {
-  __shared__ double sh[kMetThreads];
   const double c_x = res[0], c_y = res[1];
   double e_obj = 0.0, e_ph = 0.0, e_q = 0.0, q_rr = 0.0;
   const size_t stride = (size_t)gridDim.x * kMetThreads;
@@ -121,88 +179,132 @@ __global__ void __launch_bounds__(kMetThreads) k_align_pass2(const float2* __res
     e_q += dx * dx + dy * dy;
     q_rr += (double)b.x * b.x + (double)b.y * b.y;
   }
-  double* out = part + (size_t)blockIdx.x * 4;
   const double v[4] = {e_obj, e_ph, e_q, q_rr};
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const double s = block_sum_d(v[j], sh);
-    if (threadIdx.x == 0) out[j] = s;
-  }
+  block_sums(v, part + (size_t)blockIdx.x * 4);
 }
 
-__global__ void k_align_final2(const double* __restrict__ part, int blocks, double* __restrict__ res) {
+__global__ void __launch_bounds__(128) k_align_final2(const double* __restrict__ part, double* __restrict__ res) {
+  __shared__ double s[4];
+  const int w = threadIdx.x >> 5;
+  const double v = warp_sum_partials(part + w, 4);
+  if ((threadIdx.x & 31) == 0) s[w] = v;
+  __syncthreads();
   if (threadIdx.x != 0) return;
-  double s[4] = {0, 0, 0, 0};
-  for (int b = 0; b < blocks; ++b)
-    for (int j = 0; j < 4; ++j) s[j] += part[(size_t)b * 4 + j];
   const double rr = res[2], cnt = res[3];
   res[4] = rr > 0.0 ? sqrt(s[0] / rr) : 0.0;
   res[5] = s[3] > 0.0 ? sqrt(s[2] / s[3]) : 0.0;
   res[6] = cnt > 0.0 ? sqrt(s[1] / cnt) : 0.0;
 }
 
-// Summed illumination of each object pixel, positions in index order, and
-// the largest value per block.
-__global__ void __launch_bounds__(kMetThreads) k_illumination(const float2* __restrict__ qr, int m,
+// |Q_ref|^2 in FP64 (both products are exact); also clears the maximum.
+__global__ void __launch_bounds__(kMetThreads) k_probe_intensity(const float2* __restrict__ qr, size_t n,
+                                                                 double* __restrict__ p2,
+                                                                 unsigned long long* __restrict__ max_bits) {
+  const size_t first = (size_t)blockIdx.x * kMetThreads + threadIdx.x;
+  if (first == 0) *max_bits = 0ull;
+  for (size_t i = first; i < n; i += (size_t)gridDim.x * kMetThreads)
+    p2[i] = (double)qr[i].x * qr[i].x + (double)qr[i].y * qr[i].y;
+}
+
+// Summed illumination of each object pixel, positions in index order, and the
+// largest value (as bits: no value is negative).  One block per tile of 8 x 32
+// pixels: the positions whose patch overlaps the tile are first gathered, in
+// order, into a list, so a pixel walks only those instead of every position;
+// |Q|^2 comes from a table, which leaves one FP64 add per covered pixel and
+// position (the FP64 pipe is the bound: 23 us for 14.7 M of them).  512^2 pixels,
+// 900 positions, m = 128: 2210 us with every position tested at every pixel.
+constexpr int kIllumRows = 8, kIllumCols = 32, kIllumWarps = kMetThreads / 32;
+__global__ void __launch_bounds__(kMetThreads) k_illumination(const double* __restrict__ p2, int m,
                                                               const int32_t* __restrict__ pos, int n_pos,
-                                                              int n_rows, int n_cols, double* __restrict__ illum,
-                                                              double* __restrict__ part_max) {
-  __shared__ int2 sp[kPosChunk];
-  __shared__ double sh[kMetThreads];
-  const size_t n = (size_t)n_rows * n_cols;
-  double mx = 0.0;
-  // every block walks the same number of rounds, so the barriers stay uniform
-  const size_t stride = (size_t)gridDim.x * kMetThreads;
-  const size_t rounds = (n + stride - 1) / stride;
-  for (size_t rd = 0; rd < rounds; ++rd) {
-    const size_t i = rd * stride + (size_t)blockIdx.x * kMetThreads + threadIdx.x;
-    const bool live = i < n;
-    const int r = live ? (int)(i / n_cols) : 0, c = live ? (int)(i % n_cols) : 0;
-    double s = 0.0;
-    for (int k0 = 0; k0 < n_pos; k0 += kPosChunk) {
-      const int cnt = min(kPosChunk, n_pos - k0);
-      __syncthreads();
-      for (int j = threadIdx.x; j < cnt; j += kMetThreads) sp[j] = make_int2(pos[2 * (k0 + j)], pos[2 * (k0 + j) + 1]);
-      __syncthreads();
-      if (live) {
-        for (int j = 0; j < cnt; ++j) {
-          const int lr = r - sp[j].x, lc = c - sp[j].y;
-          if ((unsigned)lr < (unsigned)m && (unsigned)lc < (unsigned)m) {
-            const float2 q = qr[lr * m + lc];
-            s += (double)q.x * q.x + (double)q.y * q.y;
+                                                              int n_rows, int n_cols, int tiles_x,
+                                                              double* __restrict__ illum,
+                                                              unsigned long long* __restrict__ max_bits) {
+  __shared__ int2 list[kPosChunk];
+  __shared__ int count[kIllumWarps];
+  __shared__ double warp_max[kIllumWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int r0 = (int)(blockIdx.x / tiles_x) * kIllumRows, c0 = (int)(blockIdx.x % tiles_x) * kIllumCols;
+  const int r = r0 + warp, c = c0 + lane;
+  const bool live = r < n_rows && c < n_cols;
+  double s = 0.0;
+  constexpr int PW = kPosChunk / kIllumWarps, ROUNDS = PW / 32;  // positions of a chunk per warp
+  for (int k0 = 0; k0 < n_pos; k0 += kPosChunk) {
+    // ordered compaction: warp w takes the w-th run of the chunk's positions
+    int2 p[ROUNDS];
+    unsigned mask[ROUNDS];
+    int mine = 0;
+#pragma unroll
+    for (int i = 0; i < ROUNDS; ++i) {
+      const int k = k0 + warp * PW + i * 32 + lane;
+      bool hit = false;
+      if (k < n_pos) {
+        p[i] = make_int2(pos[2 * k], pos[2 * k + 1]);
+        hit = p[i].x < r0 + kIllumRows && (long long)p[i].x + m > r0 && p[i].y < c0 + kIllumCols &&
+              (long long)p[i].y + m > c0;
+      }
+      mask[i] = __ballot_sync(0xffffffffu, hit);
+      mine += __popc(mask[i]);
+    }
+    __syncthreads();  // the previous chunk's list has been walked
+    if (lane == 0) count[warp] = mine;
+    __syncthreads();
+    int at = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < kIllumWarps; ++w) {
+      if (w < warp) at += count[w];
+      total += count[w];
+    }
+#pragma unroll
+    for (int i = 0; i < ROUNDS; ++i) {
+      if (mask[i] >> lane & 1u) list[at + __popc(mask[i] & ((1u << lane) - 1u))] = p[i];
+      at += __popc(mask[i]);
+    }
+    __syncthreads();
+    if (live) {
+      // the loads of eight positions in flight, the sums in order; 0 where the patch does not reach
+      for (int j0 = 0; j0 < total; j0 += 8) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          v[u] = 0.0;
+          if (j0 + u < total) {
+            const int lr = r - list[j0 + u].x, lc = c - list[j0 + u].y;
+            if ((unsigned)lr < (unsigned)m && (unsigned)lc < (unsigned)m) v[u] = p2[(size_t)lr * m + lc];
           }
         }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s += v[u];
       }
     }
-    if (live) {
-      illum[i] = s;
-      mx = fmax(mx, s);
-    }
   }
-  sh[threadIdx.x] = mx;
+  if (live) illum[(size_t)r * n_cols + c] = s;
+  double mx = live ? fmax(s, 0.0) : 0.0;  // fmax: a NaN never becomes the maximum
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) warp_max[warp] = mx;
   __syncthreads();
-  for (int s = kMetThreads / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + s]);
-    __syncthreads();
+  if (tid == 0) {
+#pragma unroll
+    for (int w = 0; w < kIllumWarps; ++w) mx = fmax(mx, warp_max[w]);
+    atomicMax(max_bits, (unsigned long long)__double_as_longlong(mx));
   }
-  if (threadIdx.x == 0) part_max[blockIdx.x] = sh[0];
 }
 
 __global__ void __launch_bounds__(kMetThreads) k_region_mask(const double* __restrict__ illum, size_t n,
-                                                             const double* __restrict__ part_max, int blocks,
+                                                             const unsigned long long* __restrict__ max_bits,
                                                              double frac, uint8_t* __restrict__ region) {
-  __shared__ double thr;
-  if (threadIdx.x == 0) {
-    double mx = 0.0;
-    for (int b = 0; b < blocks; ++b) mx = fmax(mx, part_max[b]);
-    thr = frac * mx;
-  }
-  __syncthreads();
+  const double thr = frac * __longlong_as_double((long long)*max_bits);
   for (size_t i = (size_t)blockIdx.x * kMetThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kMetThreads)
     region[i] = illum[i] >= thr ? 1 : 0;
 }
 
 }  // namespace
+
+void scratch_trim(int dev) {
+  std::lock_guard<std::mutex> lk(g_scratch_mu);
+  if (dev >= 0 && dev < 256 && g_scratch_pool[dev]) cudaMemPoolTrimTo(g_scratch_pool[dev], 0);
+}
+
 }  // namespace emg
 
 extern "C" emg_status emg_aligned_errors(const float* object, const float* object_ref, int32_t n_rows,
@@ -214,11 +316,7 @@ extern "C" emg_status emg_aligned_errors(const float* object, const float* objec
   const cudaStream_t s = (cudaStream_t)stream;
   const size_t n = (size_t)n_rows * n_cols, nq = (size_t)m * m;
   double* scratch = nullptr;  // 5 + 4 partials per block, then 7 results
-  const size_t words = (size_t)kMetBlocks * 9 + 8;
-  if (cudaMalloc(&scratch, words * sizeof(double)) != cudaSuccess) {
-    cudaGetLastError();
-    return EMG_ENOMEM;
-  }
+  if (scratch_alloc(&scratch, (size_t)kMetBlocks * 9 + 8, s) != cudaSuccess) return EMG_ENOMEM;
   double* p1 = scratch;
   double* p2 = scratch + (size_t)kMetBlocks * 5;
   double* res = scratch + (size_t)kMetBlocks * 9;
@@ -226,7 +324,7 @@ extern "C" emg_status emg_aligned_errors(const float* object, const float* objec
   cudaError_t e = cudaSuccess;
   k_align_pass1<<<kMetBlocks, kMetThreads, 0, s>>>((const float2*)object, (const float2*)object_ref, region, n, p1);
   if ((e = cudaGetLastError()) == cudaSuccess) {
-    k_align_final1<<<1, 32, 0, s>>>(p1, kMetBlocks, res);
+    k_align_final1<<<1, 160, 0, s>>>(p1, res);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
@@ -235,13 +333,13 @@ extern "C" emg_status emg_aligned_errors(const float* object, const float* objec
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
-    k_align_final2<<<1, 32, 0, s>>>(p2, kMetBlocks, res);
+    k_align_final2<<<1, 128, 0, s>>>(p2, res);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(host, res, sizeof(host), cudaMemcpyDeviceToHost, s);
+  const cudaError_t ef = cudaFreeAsync(scratch, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(scratch);
-  if (e != cudaSuccess) return EMG_ECUDA;
+  if (e != cudaSuccess || ef != cudaSuccess) return EMG_ECUDA;
   out[0] = host[0];  // c (re, im)
   out[1] = host[1];
   out[2] = host[4];  // object relative error
@@ -258,20 +356,21 @@ extern "C" emg_status emg_illuminated_region(const float* probe_ref, int32_t m, 
       !isfinite(frac))
     return EMG_EINVAL;
   const cudaStream_t s = (cudaStream_t)stream;
-  const size_t n = (size_t)n_rows * n_cols;
-  double* scratch = nullptr;
-  if (cudaMalloc(&scratch, (n + kMetBlocks) * sizeof(double)) != cudaSuccess) {
-    cudaGetLastError();
-    return EMG_ENOMEM;
-  }
-  k_illumination<<<kMetBlocks, kMetThreads, 0, s>>>((const float2*)probe_ref, m, pos, n_pos, n_rows, n_cols,
-                                                    scratch, scratch + n);
+  const size_t n = (size_t)n_rows * n_cols, nq = (size_t)m * m;
+  const size_t tiles_x = (n_cols + kIllumCols - 1) / kIllumCols, tiles_y = (n_rows + kIllumRows - 1) / kIllumRows;
+  double* scratch = nullptr;  // illumination, |Q_ref|^2, the maximum
+  if (scratch_alloc(&scratch, n + nq + 1, s) != cudaSuccess) return EMG_ENOMEM;
+  double* p2 = scratch + n;
+  unsigned long long* max_bits = (unsigned long long*)(p2 + nq);
+  k_probe_intensity<<<kMetBlocks, kMetThreads, 0, s>>>((const float2*)probe_ref, nq, p2, max_bits);
+  k_illumination<<<(unsigned)(tiles_x * tiles_y), kMetThreads, 0, s>>>(p2, m, pos, n_pos, n_rows, n_cols, (int)tiles_x,
+                                                                      scratch, max_bits);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) {
-    k_region_mask<<<kMetBlocks, kMetThreads, 0, s>>>(scratch, n, scratch + n, kMetBlocks, frac, region);
+    k_region_mask<<<kMetBlocks, kMetThreads, 0, s>>>(scratch, n, max_bits, frac, region);
     e = cudaGetLastError();
   }
+  const cudaError_t ef = cudaFreeAsync(scratch, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(scratch);
-  return e == cudaSuccess ? EMG_OK : EMG_ECUDA;
+  return e == cudaSuccess && ef == cudaSuccess ? EMG_OK : EMG_ECUDA;
 }
