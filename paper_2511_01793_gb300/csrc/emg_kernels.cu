@@ -1266,8 +1266,9 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   }  // !RIN
 
   if constexpr (!RIN) {
-    if (a.prep_clusters > 0 && a.levels > 1) {
-      // the level arrays of this minibatch come from the prep clusters of this launch
+    if (a.prep_clusters > 0) {
+      // the level arrays of this minibatch (with one level the gain G_0 alone) come
+      // from the prep clusters of this launch
       if (tid == 0) {
         const unsigned long long t0 = globaltimer_ns();
         while (ld_acquire_u32(a.sync + 1) < a.prep_target) {

@@ -315,6 +315,23 @@ def test_fused_probe_prep_equals_the_separate_kernel(lib, torch, m, levels, prol
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
 
 
+@pytest.mark.parametrize("m,cl", [(32, 2), (64, 2), (64, 4), (128, 4), (128, 8)])
+def test_fused_probe_prep_with_one_level_waits_for_the_gain(lib, torch, m, cl):
+    """One multigrid level reads G_0 of the probe prep too: with the prep inside the step launch
+    the positions wait for it, so the states equal those of the separate kernel bitwise."""
+    case = Case(n=2 * m + 40, m=m, side=5, seed=105 + m)
+    p = oracle_params(minibatch=3, levels=1)
+    out = []
+    for fuse in (1, 0):
+        c = make_context(lib, case, p, seed=3)
+        lib.emg_set_cluster(c.ctx, cl)
+        lib.emg_set_prep_fusion(c.ctx, fuse)
+        lib.emg_run_epochs(c.ctx, 4)
+        out.append(state(c))
+        c.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
 def test_host_buffer_call_reports_a_wait_that_gave_up_and_recovers(lib, torch):
     """The host-buffer entry point queues its downloads and waits once; a bounded
     wait that gave up in the step kernel (made to run out) still makes it return
