@@ -71,6 +71,7 @@ struct emg_ctx {
   // launches that follow a max|Q|^2 seed; the host keeps their expected values.
   unsigned* d_sync = nullptr;
   unsigned ticket_base = 0, prep_done_base = 0;
+  bool seeded = false;            // the seed is the last kernel enqueued: the next one waits for its end
   int resident_cluster = -1, resident_clusters = 0;  // step clusters resident at once, for `cluster`
   int fuse_prep = 1;              // probe prep inside the step launch where it fits (emg_set_prep_fusion)
   unsigned prep_wait_extra = 0;   // test hook: added to the prep count a launch waits for
@@ -425,14 +426,22 @@ void permutation(uint64_t seed, int64_t epoch, int32_t n, int32_t* out) {
   }
 }
 
-// Seeds max|Q|^2 of the bound probe into slot 0 before a call's first minibatch.
-emg_status seed_probe_max(emg_ctx* c, cudaStream_t s) {
-  EMG_CUDA(c, cudaMemsetAsync(c->d_mq, 0, 2 * sizeof(unsigned), s));
-  EMG_CUDA(c, cudaMemsetAsync(c->d_sync, 0, 2 * sizeof(unsigned), s));
+// Seeds max|Q|^2 of the bound probe into slot 0 and clears the counters before
+// a call's first minibatch; with `idx` also puts its b indices into d_orders.
+emg_status seed_probe_max(emg_ctx* c, cudaStream_t s, const int32_t* idx = nullptr, int b = 0) {
+  if (idx) {
+    emg_status st = ensure_orders(c, (size_t)c->n_pos);
+    if (st != EMG_OK) return st;
+    if (!emg::seed_takes_idx(b)) {
+      if ((st = upload_orders(c, idx, (size_t)b, s)) != EMG_OK) return st;
+      idx = nullptr;
+    }
+  }
   c->ticket_base = c->prep_done_base = 0;
+  c->seeded = true;
   LaunchMark mk(c, kKindOther);
-  cudaError_t e = emg::launch_probe_max(c->probe, c->m, c->d_mq, s);
-  if (e != cudaSuccess) return cuda_fail(c, e, "k_probe_max launch");
+  cudaError_t e = emg::launch_seed(c->probe, c->m, c->d_mq, c->d_sync, c->d_orders, idx, b, s);
+  if (e != cudaSuccess) return cuda_fail(c, e, "k_seed launch");
   return EMG_OK;
 }
 
@@ -462,6 +471,8 @@ emg_status enqueue_minibatch(emg_ctx* c, const int32_t* d_idx, int b, double* d_
   float2* qt_all = sh ? sh->qt : c->d_qt;
   float* mu_all = sh ? sh->mu : c->d_mu;
   if (do_step) {
+  const bool overlap = !c->seeded;
+  c->seeded = false;
   PrepArgs pa = c->prep;
   pa.probe = c->probe;  // the probe bound right now (emg_reconstruct_host swaps it)
   pa.mq_read = c->d_mq + (seq & 1);
@@ -491,7 +502,7 @@ emg_status enqueue_minibatch(emg_ctx* c, const int32_t* d_idx, int b, double* d_
   if (fused_tiles == 0) {
     {
       LaunchMark mk(c, kKindPrep);
-      e = emg::launch_prep(pa, strm);
+      e = emg::launch_prep(pa, overlap, strm);
     }
     if (e != cudaSuccess) return cuda_fail(c, e, "k_prep launch");
   }
@@ -562,7 +573,7 @@ emg_status enqueue_minibatch(emg_ctx* c, const int32_t* d_idx, int b, double* d_
     }
   } else {
     LaunchMark mk(c, kKindStep);
-    e = emg::launch_step(c->m, nb, sa, strm);
+    e = emg::launch_step(c->m, nb, sa, overlap || fused_tiles == 0, strm);
   }
   if (e != cudaSuccess) return cuda_fail(c, e, "k_step launch");
   }  // do_step
@@ -1104,9 +1115,7 @@ emg_status emg_step_minibatch(emg_ctx* c, const int32_t* idx, int32_t b, double*
   for (int i = 0; i < b; ++i)
     if (idx[i] < 0 || idx[i] >= c->n_pos) return fail(c, EMG_EINVAL, "idx entry out of range");
   DeviceGuard g(c->device);
-  if ((st = ensure_orders(c, (size_t)c->n_pos)) != EMG_OK) return st;
-  if ((st = upload_orders(c, idx, (size_t)b, c->stream)) != EMG_OK) return st;
-  if ((st = seed_probe_max(c, c->stream)) != EMG_OK) return st;
+  if ((st = seed_probe_max(c, c->stream, idx, b)) != EMG_OK) return st;
   if ((st = enqueue_minibatch(c, c->d_orders, b, c->d_phi, 0, c->stream)) != EMG_OK) return st;
   c->last_b = b;
   if (sampled_misfit) {
@@ -1142,9 +1151,7 @@ emg_status emg_shard_step(emg_ctx* c, const int32_t* idx, int32_t b, int32_t slo
   if (slot_begin < 0 || slot_end < slot_begin || slot_end > b)
     return fail(c, EMG_EINVAL, "need 0 <= slot_begin <= slot_end <= b");
   DeviceGuard g(c->device);
-  if ((st = ensure_orders(c, (size_t)c->n_pos)) != EMG_OK) return st;
-  if ((st = upload_orders(c, idx, (size_t)b, c->stream)) != EMG_OK) return st;
-  if ((st = seed_probe_max(c, c->stream)) != EMG_OK) return st;
+  if ((st = seed_probe_max(c, c->stream, idx, b)) != EMG_OK) return st;
   ShardPart sh{slot_begin, slot_end, (float2*)zt, (float2*)qt, mu, true, false};
   return enqueue_minibatch(c, c->d_orders, b, c->d_phi, 0, c->stream, &sh);
 }

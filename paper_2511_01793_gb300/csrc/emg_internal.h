@@ -183,16 +183,22 @@ cudaError_t upload_twiddles();
 cudaError_t launch_amp_prep(const float* d, float* amp, int m, int n_pos, cudaStream_t s);
 // a_k of positions idx[0..b) (device indices) from d, which may be mapped host memory.
 cudaError_t launch_amp_gather(const float* d, const int32_t* idx, int b, float* amp, int m, cudaStream_t s);
-cudaError_t launch_prep(const PrepArgs& a, cudaStream_t s);
+// `overlap`: the kernel may start while its predecessor drains.  Not for the first kernel after
+// launch_seed, which writes what the kernels read before they wait (tickets, position indices).
+cudaError_t launch_prep(const PrepArgs& a, bool overlap, cudaStream_t s);
 // Fused probe prep for the cluster step kernel: sets a.tile / a.halo for it
 // and returns its tile count, or 0 when it does not fit beside the step.
 int fused_prep_tiles(PrepArgs& a, int m, int cluster);
 // Step-kernel clusters that can be resident on the device at once (0 if unknown).
 int step_resident_clusters(int m, int cluster);
-cudaError_t launch_probe_max(const float2* probe, int m, unsigned* slot, cudaStream_t s);
+// Before a call's first minibatch: max|Q|^2 into mq[0], mq[1] = 0, sync[0..1] = 0 (sync may be
+// NULL) and, with `idx` (host, b <= 2048, see seed_takes_idx), the b indices into `order`.
+cudaError_t launch_seed(const float2* probe, int m, unsigned* mq, unsigned* sync, int32_t* order, const int32_t* idx,
+                        int b, cudaStream_t s);
+bool seed_takes_idx(int b);
 // Fills tile/halo of a and returns true when the tiled prep fits in shared memory.
 bool prep_tiled_config(PrepArgs& a);
-cudaError_t launch_step(int m, int b, const StepArgs& a, cudaStream_t s);
+cudaError_t launch_step(int m, int b, const StepArgs& a, bool overlap, cudaStream_t s);
 // The step with R_k and the misfit partials given (a.r_in, a.r_partial): m = 128 (cluster 2, 4), 256 (8).
 cudaError_t launch_step_rin(int m, int b, const StepArgs& a, cudaStream_t s);
 cudaError_t launch_apply(const ApplyArgs& a, cudaStream_t s);

@@ -13,6 +13,7 @@
 #include <cooperative_groups.h>
 #include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "emg_fft.cuh"
 #include "emg_internal.h"
@@ -500,11 +501,47 @@ __device__ __forceinline__ void warp_atomic_max(unsigned* slot, float v) {
   if ((threadIdx.x & 31) == 0) atomicMax(slot, __float_as_uint(v));
 }
 
-__global__ void __launch_bounds__(256) k_probe_max(const float2* __restrict__ probe, int n,
-                                                   unsigned* __restrict__ slot) {
+// What precedes a call's first minibatch, in one launch: max|Q|^2 of the probe
+// into mq[0], mq[1] and the ticket counters cleared, and (NI > 0) the
+// minibatch's position indices, which travel in the launch parameters (the
+// runtime copies them when the launch is enqueued, so the caller may overwrite
+// its host array, pinned or not, once the call returns).  One cluster, so that
+// the maximum needs no memory cleared beforehand.
+constexpr int kSeedThreads = 512, kSeedCtas = 8, kSeedMaxIdx = 2048;
+template <int NI>
+struct SeedIdx {
+  int32_t v[NI > 0 ? NI : 1];
+};
+template <int NI>
+__global__ void __launch_bounds__(kSeedThreads) k_seed(const float2* __restrict__ probe, int n, unsigned* __restrict__ mq,
+                                                       unsigned* __restrict__ sync, int32_t* __restrict__ order, int b,
+                                                       const SeedIdx<NI> idx) {
+  __shared__ float redf[kSeedThreads / 32];
+  __shared__ float part[kSeedCtas];
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const int rank = (int)cl.block_rank(), ctas = (int)cl.num_blocks(), tid = threadIdx.x;
+  pdl_wait();  // the probe and the counters belong to the previous kernel until it has ended
   float mx = 0.f;
-  for (int p = blockIdx.x * 256 + threadIdx.x; p < n; p += gridDim.x * 256) mx = fmaxf(mx, cabs2(probe[p]));
-  warp_atomic_max(slot, mx);
+#pragma unroll 8
+  for (int p = rank * kSeedThreads + tid; p < n; p += ctas * kSeedThreads) mx = fmaxf(mx, cabs2(probe[p]));
+  warp_partial_max(mx, redf);
+  __syncthreads();
+  if (ctas > 1) {
+    if (tid == 0) *cl.map_shared_rank(&part[rank], 0) = partials_max<kSeedThreads>(redf);
+    cl.sync();
+  } else if (tid == 0) {
+    part[0] = partials_max<kSeedThreads>(redf);
+  }
+  if (rank != 0) return;
+  if (tid == 0) {
+    float m = part[0];
+    for (int d = 1; d < ctas; ++d) m = fmaxf(m, part[d]);
+    mq[0] = __float_as_uint(m);
+    mq[1] = 0u;
+    if (sync) sync[0] = sync[1] = 0u;
+  }
+  if constexpr (NI > 0)
+    for (int i = tid; i < b; i += kSeedThreads) order[i] = idx.v[i];
 }
 
 // Tiled probe-only prep: one CTA per tile x tile block of level-0 pixels.
@@ -2373,23 +2410,19 @@ int fused_prep_tiles(PrepArgs& a, int m, int cluster) {
   return (m / tile) * (m / tile);
 }
 
-cudaError_t launch_prep(const PrepArgs& a, cudaStream_t s) {
+cudaError_t launch_prep(const PrepArgs& a, bool overlap, cudaStream_t s) {
   PrepArgs t = a;
   if (a.mq_read && prep_tiled_config(t)) {
     const int tiles = (t.m / t.tile) * (t.m / t.tile);
-    cudaError_t e = launch_pdl(k_prep_tile, dim3(tiles), dim3(kPrepTileThreads), prep_tile_smem(t), s, t);
-    if (e != cudaSuccess) return e;
+    if (overlap) {
+      cudaError_t e = launch_pdl(k_prep_tile, dim3(tiles), dim3(kPrepTileThreads), prep_tile_smem(t), s, t);
+      if (e != cudaSuccess) return e;
+    } else {
+      k_prep_tile<<<tiles, kPrepTileThreads, prep_tile_smem(t), s>>>(t);
+    }
   } else {
     k_prep<<<1, kPrepThreads, 0, s>>>(a);
   }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_probe_max(const float2* probe, int m, unsigned* slot, cudaStream_t s) {
-  const int n = m * m;
-  int blocks = (n + 255) / 256;
-  if (blocks > 64) blocks = 64;
-  k_probe_max<<<blocks, 256, 0, s>>>(probe, n, slot);
   return cudaGetLastError();
 }
 
@@ -2430,6 +2463,26 @@ cudaError_t launch_cluster_plain(Kernel kernel, int cluster, dim3 grid, dim3 blo
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <int NI>
+cudaError_t launch_seed_t(const float2* probe, int m, unsigned* mq, unsigned* sync, int32_t* order, const int32_t* idx,
+                          int b, cudaStream_t s) {
+  SeedIdx<NI> pv;
+  if (NI > 0) memcpy(pv.v, idx, (size_t)b * sizeof(int32_t));
+  const int ctas = m <= 64 ? 1 : kSeedCtas;  // 4096 pixels are 8 loads a thread for one CTA
+  const cudaError_t e = launch_cluster_pdl(k_seed<NI>, ctas, dim3(ctas), dim3(kSeedThreads), 0, s, probe, m * m, mq, sync,
+                                           order, b, pv);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+bool seed_takes_idx(int b) { return b <= kSeedMaxIdx; }
+
+cudaError_t launch_seed(const float2* probe, int m, unsigned* mq, unsigned* sync, int32_t* order, const int32_t* idx, int b,
+                        cudaStream_t s) {
+  if (!idx) return launch_seed_t<0>(probe, m, mq, sync, nullptr, nullptr, 0, s);
+  if (b <= 64) return launch_seed_t<64>(probe, m, mq, sync, order, idx, b, s);
+  return launch_seed_t<kSeedMaxIdx>(probe, m, mq, sync, order, idx, b, s);
 }
 
 template <int M, int MODE>
@@ -2519,10 +2572,12 @@ cudaError_t set_cluster_attrs() {
 }
 
 template <int M, int C>
-cudaError_t launch_stepc_t(int b, const StepArgs& a, cudaStream_t s) {
+cudaError_t launch_stepc_t(int b, const StepArgs& a, bool overlap, cudaStream_t s) {
   using TL = StepTile<M, C>;
-  cudaError_t e = launch_cluster_pdl(k_stepc<M, C>, C, dim3(C * (b + a.prep_clusters)), dim3(TL::NT),
-                                     TL::smem_elems * sizeof(float2), s, a);
+  const dim3 grid(C * (b + a.prep_clusters)), block(TL::NT);
+  constexpr size_t bytes = TL::smem_elems * sizeof(float2);
+  cudaError_t e = overlap ? launch_cluster_pdl(k_stepc<M, C>, C, grid, block, bytes, s, a)
+                          : launch_cluster_plain(k_stepc<M, C>, C, grid, block, bytes, s, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -2546,18 +2601,18 @@ cudaError_t launch_step_rin(int m, int b, const StepArgs& a, cudaStream_t s) {
   }
 }
 
-cudaError_t launch_step(int m, int b, const StepArgs& a, cudaStream_t s) {
+cudaError_t launch_step(int m, int b, const StepArgs& a, bool overlap, cudaStream_t s) {
   switch (m * 16 + a.cluster) {
     case 16 * 16 + 1: return launch_step_t<16>(b, a, s);
-    case 16 * 16 + 2: return launch_stepc_t<16, 2>(b, a, s);
+    case 16 * 16 + 2: return launch_stepc_t<16, 2>(b, a, overlap, s);
     case 32 * 16 + 1: return launch_step_t<32>(b, a, s);
-    case 32 * 16 + 2: return launch_stepc_t<32, 2>(b, a, s);
-    case 64 * 16 + 2: return launch_stepc_t<64, 2>(b, a, s);
-    case 64 * 16 + 4: return launch_stepc_t<64, 4>(b, a, s);
-    case 128 * 16 + 2: return launch_stepc_t<128, 2>(b, a, s);
-    case 128 * 16 + 4: return launch_stepc_t<128, 4>(b, a, s);
-    case 128 * 16 + 8: return launch_stepc_t<128, 8>(b, a, s);
-    case 256 * 16 + 8: return launch_stepc_t<256, 8>(b, a, s);
+    case 32 * 16 + 2: return launch_stepc_t<32, 2>(b, a, overlap, s);
+    case 64 * 16 + 2: return launch_stepc_t<64, 2>(b, a, overlap, s);
+    case 64 * 16 + 4: return launch_stepc_t<64, 4>(b, a, overlap, s);
+    case 128 * 16 + 2: return launch_stepc_t<128, 2>(b, a, overlap, s);
+    case 128 * 16 + 4: return launch_stepc_t<128, 4>(b, a, overlap, s);
+    case 128 * 16 + 8: return launch_stepc_t<128, 8>(b, a, overlap, s);
+    case 256 * 16 + 8: return launch_stepc_t<256, 8>(b, a, overlap, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -2823,17 +2878,8 @@ cudaError_t noalloc_setup(int dev, unsigned char** base) {
   return cudaSuccess;
 }
 
-// The minibatch's position indices travel inside the launch parameters, which
-// the runtime copies when the launch is enqueued: the caller may overwrite its
-// host array as soon as the call returns, pinned or not.
-constexpr int kNoAllocMaxIdx = 2048;
-struct NoAllocIdx {
-  int32_t v[kNoAllocMaxIdx];
-};
-
-__global__ void k_noalloc_idx(const NoAllocIdx p, int b, int32_t* __restrict__ out) {
-  for (int i = threadIdx.x; i < b; i += blockDim.x) out[i] = p.v[i];
-}
+// The minibatch's position indices travel inside the seed kernel's launch parameters.
+constexpr int kNoAllocMaxIdx = kSeedMaxIdx;
 
 template <int M>
 cudaError_t launch_step_natural(int b, const StepArgs& a, cudaStream_t s) {
@@ -2873,16 +2919,8 @@ extern "C" emg_status emg_step_minibatch_noalloc(float* object, int32_t n_rows, 
   if (cudaGetDevice(&dev) != cudaSuccess || noalloc_setup(dev, &base) != cudaSuccess) return EMG_ECUDA;
   const cudaStream_t s = (cudaStream_t)stream;
   int32_t* d_idx = (int32_t*)(base + L.idx);
-  {
-    NoAllocIdx pv;
-    memcpy(pv.v, idx, (size_t)b * sizeof(int32_t));
-    k_noalloc_idx<<<1, 256, 0, s>>>(pv, b, d_idx);
-    if (cudaGetLastError() != cudaSuccess) return EMG_ECUDA;
-  }
-
   unsigned* d_mq = (unsigned*)(base + L.mq);
-  if (cudaMemsetAsync(d_mq, 0, 2 * sizeof(unsigned), s) != cudaSuccess) return EMG_ECUDA;
-  if (launch_probe_max((const float2*)probe, m, d_mq, s) != cudaSuccess) return EMG_ECUDA;
+  if (launch_seed((const float2*)probe, m, d_mq, nullptr, d_idx, idx, b, s) != cudaSuccess) return EMG_ECUDA;
 
   PrepArgs pa{};
   StepArgs sa{};
@@ -2948,7 +2986,7 @@ extern "C" emg_status emg_step_minibatch_noalloc(float* object, int32_t n_rows, 
   aa.tiles_x = apply_tiles_x(n_cols);
   aa.tiles_y = apply_tiles_y(n_rows);
 
-  cudaError_t e = launch_prep(pa, s);
+  cudaError_t e = launch_prep(pa, false, s);
   if (e == cudaSuccess) {
     switch (m) {
       case 16: e = launch_step_natural<16>(b, sa, s); break;

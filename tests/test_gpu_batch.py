@@ -332,6 +332,33 @@ def test_fused_probe_prep_with_one_level_waits_for_the_gain(lib, torch, m, cl):
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
 
 
+@pytest.mark.parametrize("b", [1, 64, 65, 2048, 2049])
+def test_minibatch_indices_reach_the_step_by_every_route(lib, torch, b):
+    """Indices of up to 64, up to 2048 and more positions travel differently (two sizes of launch
+    parameters, a staged copy): each gives bitwise the epoch whose one minibatch has that order."""
+    m, N = 16, 2304
+    rng = np.random.default_rng(b)
+    pos = rng.integers(-4, 60, size=(N, 2)).astype(np.int32)
+    d = rng.uniform(0.0, 4.0, size=(N, m, m)).astype(np.float32)
+    z0 = (rng.standard_normal((64, 70)) + 1j * rng.standard_normal((64, 70))).astype(np.complex64)
+    q0 = (rng.standard_normal((m, m)) + 1j * rng.standard_normal((m, m))).astype(np.complex64)
+    idx = rng.permutation(N)[:b].astype(np.int32)
+    out = []
+    for n in (N, b):
+        sub = np.arange(N) if n == N else idx
+        params = lib.emg_default_params(alpha=0.05, minibatch=b, levels=2)
+        c = lib.Context(pos[sub], d[sub], 64, 70, params, obj=torch.from_numpy(z0), probe=torch.from_numpy(q0))
+        if n == N:
+            host = idx.copy()
+            lib.emg_step_minibatch(c.ctx, host)
+            host[:] = -1  # the caller's array is free once the call returns
+        else:
+            lib.emg_run_epochs(c.ctx, 1, order=np.arange(b, dtype=np.int32)[None])
+        out.append(state(c))
+        c.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
 def test_host_buffer_call_reports_a_wait_that_gave_up_and_recovers(lib, torch):
     """The host-buffer entry point queues its downloads and waits once; a bounded
     wait that gave up in the step kernel (made to run out) still makes it return
