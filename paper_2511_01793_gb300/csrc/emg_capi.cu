@@ -490,7 +490,7 @@ emg_status enqueue_minibatch(emg_ctx* c, const int32_t* d_idx, int b, double* d_
   // launch fits in one wave of resident clusters: there it overlaps the gather
   // and transforms.  Otherwise it is its own kernel before the step.
   PrepArgs pf = pa;
-  int fused_tiles = (c->fuse_prep && !c->tc && c->cluster >= 2) ? emg::fused_prep_tiles(pf, c->m, c->cluster) : 0;
+  int fused_tiles = (c->fuse_prep && !c->tc && c->cluster >= 1) ? emg::fused_prep_tiles(pf, c->m, c->cluster) : 0;
   if (fused_tiles > 0) {
     const int prep_clusters = (fused_tiles + c->cluster - 1) / c->cluster;
     if (c->resident_cluster != c->cluster) {

@@ -3,9 +3,10 @@
 //   k_amp_prep     a_k = sqrt(max(d_k, 0)) reordered into the FFT storage order
 //   k_prep         per-minibatch probe-only arrays: max|Q|^2, gains G_l, MAGPIE
 //                  weights W_z, W_R and restricted probes Q_l (Sec. 3.2)
-//   k_step<M>      one CTA per scan position: gather, exit wave, 2-D FFT, modulus
-//                  replacement (Def. 2.1), inverse FFT, MAGPIE object step,
+//   k_stepc<M, C>  one cluster of C CTAs per scan position: gather, exit wave, 2-D FFT,
+//                  modulus replacement (Def. 2.1), inverse FFT, MAGPIE object step,
 //                  ePIE probe step, geometric-mean joint step (Eq. geomean)
+//   k_step<M>      the same in one CTA, for the allocation-free entry point
 //   k_apply        deterministic combine of the minibatch into object and probe
 //   k_forward<M>   Phi_k = 1/2 ||Q . P_k z - R_k||^2 (Eq. exit_misfit) per position,
 //                  d_k = |F(Q . P_k z)|^2 (Sec. 2.1 data model), batched 2-D DFT
@@ -726,10 +727,10 @@ __host__ __device__ inline size_t step_smem_elems(int levels) {
   return n;
 }
 
-// NATURAL_AMP = true is the variant used by the allocation-free entry point:
-// a.amp then holds the caller's intensities d_k in natural order and the
-// amplitude sqrt(max(d, 0)) is formed on the fly.
-template <int M, bool NATURAL_AMP = false>
+// The step of the allocation-free entry point: a.amp holds the caller's
+// intensities d_k in natural order and the amplitude sqrt(max(d, 0)) is formed
+// on the fly; ordered combine, no verify mode.
+template <int M>
 __global__ void __launch_bounds__(StepThreads<M>::value) k_step(const StepArgs a) {
   constexpr int NT = StepThreads<M>::value;
   constexpr int S = M + 1;
@@ -770,9 +771,7 @@ __global__ void __launch_bounds__(StepThreads<M>::value) k_step(const StepArgs a
     Dft<N1, false>::run(v);
 #pragma unroll
     for (int i = 0; i < N1; ++i) {
-      const float am = NATURAL_AMP
-                           ? sqrtf(fmaxf(amp[storage_to_freq<M>(i + N1 * k2) * M + storage_to_freq<M>(c)], 0.f))
-                           : amp[(i + N1 * k2) * M + c];
+      const float am = sqrtf(fmaxf(amp[storage_to_freq<M>(i + N1 * k2) * M + storage_to_freq<M>(c)], 0.f));
       const float p2 = cabs2(v[i]);
       if (p2 > 0.f) {
         const float inv = rsqrtf(p2);
@@ -879,10 +878,8 @@ __global__ void __launch_bounds__(StepThreads<M>::value) k_step(const StepArgs a
   // a5 (finest level) + a6 + a7: z+, Q+, geometric-mean joint step
   const float inv_mu = mu > 0.f ? 1.f / mu : 0.f;
   const float2* G0 = a.lv.G[0];
-  const float MQ = a.s_num ? __uint_as_float(*a.mq) : 0.f;  // combine weight of the atomic scatter
   float2* zt = a.zt + (size_t)kb * M * M;
   float2* qt = a.qt + (size_t)kb * M * M;
-  float acc_after = 0.f;
   for (int p = tid; p < M * M; p += NT) {
     const int r = p / M, c = p % M;
     const float2 zk = gather_obj(a.object, a.n_rows, a.n_cols, o_r + r, o_c + c);
@@ -907,20 +904,14 @@ __global__ void __launch_bounds__(StepThreads<M>::value) k_step(const StepArgs a
       zn = zplus;
       qn = qplus;
     }
-    if (a.s_num)
-      scatter_atomic(a.s_num, a.s_den, a.combine, a.n_rows, a.n_cols, o_r + r, o_c + c, zn, zk,
-                     fmaf(a.w_eps, MQ, cabs2(q)));
-    else if (slot_ok)
+    if (slot_ok) {
       zt[p] = zn;
-    if (slot_ok) qt[p] = qn;
-    if (a.verify) acc_after += cabs2(csub(cmul(qn, zn), R));
+      qt[p] = qn;
+    }
   }
-  double phi_after = 0.0;
-  if (a.verify) phi_after = 0.5 * block_sum<NT>((double)acc_after, redd);
   if (tid == 0) {
     a.mu[kb] = mu;
     a.phi[kb] = phi;
-    if (a.verify) a.phi_after[kb] = phi_after;
   }
 }
 
@@ -986,7 +977,7 @@ struct StepTile : CTile<M, C> {
   static constexpr bool ONE = M == 256;
   static constexpr int S = B::SR;
   // CTAs per SM the register budget leaves room for (as many as the shared memory does)
-  static constexpr int MIN_CTAS = ONE ? 2 : M == 128 ? C / 2 : 1;
+  static constexpr int MIN_CTAS = ONE ? 2 : M == 128 ? C / 2 : M == 64 ? 3 * C / 2 : 1;
   static constexpr size_t slab = (size_t)B::H * S;
   // multigrid buffers of every level at which each CTA keeps a row
   static constexpr size_t mg_elems() {
@@ -1101,7 +1092,7 @@ __device__ __forceinline__ void col_pass_a_inv_to_rows(cg::cluster_group& cl, in
 template <int C, typename V>
 __device__ __forceinline__ void cluster_publish(cg::cluster_group& cl, int rank, V* arr, V v) {
 #pragma unroll
-  for (int d = 0; d < C; ++d) *(d == rank ? &arr[rank] : cl.map_shared_rank(&arr[rank], d)) = v;
+  for (int d = 0; d < C; ++d) *tile_rank<C>(cl, rank, &arr[rank], d) = v;
 }
 
 // (I_H^h y)(lr, c) for a coarse row slab stored with one halo row above and
@@ -1124,8 +1115,13 @@ __device__ __forceinline__ T prolong_halo(const T* y, int sl, int wc, int lr, in
 // the rows visible before they are read.
 template <int C, typename T>
 __device__ __forceinline__ void push_halo(cg::cluster_group& cl, int rank, T* y, int sl, int hl, int i, int j, T v) {
-  if (i == 0) *(rank > 0 ? cl.map_shared_rank(y, rank - 1) + hl * sl + j : y - sl + j) = v;
-  if (i == hl - 1) *(rank < C - 1 ? cl.map_shared_rank(y, rank + 1) - sl + j : y + hl * sl + j) = v;
+  if constexpr (C == 1) {
+    if (i == 0) y[j - sl] = v;
+    if (i == hl - 1) y[hl * sl + j] = v;
+  } else {
+    if (i == 0) *(rank > 0 ? cl.map_shared_rank(y, rank - 1) + hl * sl + j : y - sl + j) = v;
+    if (i == hl - 1) *(rank < C - 1 ? cl.map_shared_rank(y, rank + 1) - sl + j : y + hl * sl + j) = v;
+  }
 }
 
 // RIN = true: the revised exit waves R_k and the misfit partials come from the
@@ -1138,7 +1134,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   constexpr int NT = TL::NT, H = TL::H, SR = TL::S;
   constexpr int N1 = TL::N1, PER = TL::PER, SLOTS = TL::SLOTS;
   cg::cluster_group cl = cg::this_cluster();
-  const int rank = (int)cl.block_rank();
+  const int rank = C == 1 ? 0 : (int)cl.block_rank();
   extern __shared__ __align__(16) float2 sm[];  // 16-byte aligned: the update pass reads pixel pairs
   float2* rowbuf = sm;                                        // my patch rows
   float2* colbuf = ONE ? sm : sm + TL::slab;                  // my storage columns (all rows)
@@ -1157,8 +1153,8 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
       // role by ticket, taken before this launch lets the next one start: a
       // cluster only ever waits for clusters that started before it
       if (rank == 0 && tid == 0) ticket_sh = (int)(atomicAdd(a.sync, 1u) - a.ticket_base);
-      cl.sync();  // every CTA of the cluster is running; rank 0's ticket is visible
-      const int t = *cl.map_shared_rank(&ticket_sh, 0);
+      tile_sync<C>(cl);  // every CTA of the cluster is running; rank 0's ticket is visible
+      const int t = *tile_rank<C>(cl, rank, &ticket_sh, 0);
       if (t < a.prep_clusters) {
         pdl_trigger();
         pdl_wait();  // the probe and max|Q|^2 come from the previous combine
@@ -1171,7 +1167,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
             atomicAdd(a.sync + 1, 1u);
           }
         }
-        cl.sync();  // no CTA leaves while a peer may still read rank 0's ticket
+        if constexpr (C > 1) cl.sync();  // no CTA leaves while a peer may still read rank 0's ticket
         return;
       }
       kb = t - a.prep_clusters;
@@ -1211,7 +1207,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
       return zbuf[lr * M + c];
   };
   const float MQ = __uint_as_float(*a.mq);
-  cluster_arrive_relaxed();  // completed (wait) before the first distributed shared memory access
+  if constexpr (C > 1) cluster_arrive_relaxed();  // completed (wait) before the first distributed shared memory access
 
   // a1: gather my rows, psi = Q z_k, partial mu_k
   float mu_l = 0.f;
@@ -1243,11 +1239,11 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
     if constexpr (ONE) cp_async_wait_all();  // a_k; the barriers below show it to the whole CTA
     __syncthreads();
   }
-  cl.barrier_wait();  // all CTAs of the cluster resident
+  if constexpr (C > 1) cl.barrier_wait();  // all CTAs of the cluster resident
   // row pass B, outputs to the column slabs
   if constexpr (!RIN) row_pass_b_to_cols<TL>(cl, rank, rowbuf, colbuf, tid);
   if (tid == 0) cluster_publish<C>(cl, rank, xf, partials_max<NT>(redf));
-  cl.sync();
+  tile_sync<C>(cl);
   float mu = xf[0];
 #pragma unroll
   for (int d = 1; d < C; ++d) mu = fmaxf(mu, xf[d]);
@@ -1294,7 +1290,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   // inverse column pass A, outputs to the row slabs
   col_pass_a_inv_to_rows<TL>(cl, rank, colbuf, rowbuf, tid);
   if (tid == 0) cluster_publish<C>(cl, rank, xd, partials_sum<NT>(redf));
-  cl.sync();
+  tile_sync<C>(cl);
   // a4: inverse row passes -> R (natural order) on my rows
   gpass_b<M, H, SR, 1, NT, true>(rowbuf, tid);
   __syncthreads();
@@ -1304,8 +1300,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
 
   if constexpr (!RIN) {
     if (a.prep_clusters > 0) {
-      // the level arrays of this minibatch (with one level the gain G_0 alone) come
-      // from the prep clusters of this launch
+      // the level arrays of this minibatch come from the prep clusters of this launch
       if (tid == 0) {
         const unsigned long long t0 = globaltimer_ns();
         while (ld_acquire_u32(a.sync + 1) < a.prep_target) {
@@ -1337,8 +1332,12 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   auto fill_halo = [&](int l) {
     const int wl = M >> l, hl = wl / C, sl = wl + 1;
     float2* Z = Zl[l];
-    const float2* Zup = rank > 0 ? cl.map_shared_rank(Zl[l], rank - 1) : Z;
-    const float2* Zdn = rank < C - 1 ? cl.map_shared_rank(Zl[l], rank + 1) : Z;
+    const float2* Zup = Z;
+    const float2* Zdn = Z;
+    if constexpr (C > 1) {
+      if (rank > 0) Zup = cl.map_shared_rank(Zl[l], rank - 1);
+      if (rank < C - 1) Zdn = cl.map_shared_rank(Zl[l], rank + 1);
+    }
     for (int j = tid; j < wl; j += NT) {
       Z[-sl + j] = rank > 0 ? Zup[(hl - 1) * sl + j] : Z[j];
       Z[hl * sl + j] = rank < C - 1 ? Zdn[j] : Z[(hl - 1) * sl + j];
@@ -1354,6 +1353,9 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   constexpr bool kL3 = hc2 >= 1 && hc2 * wc2 >= NT && (hc2 * wc2) % NT == 0 && (hc1 * wc1) % NT == 0;
   constexpr int Q12 = kL3 ? hc2 * wc2 / NT : 1, QUP = kL3 ? hc1 * wc1 / NT : 1;
   const bool l3 = kL3 && a.levels == 3;
+  // With two levels the coarse step follows the restriction at the same pixel
+  // at once (it needs nothing from other threads), and its halo rows are pushed.
+  const bool l2 = a.levels == 2;
   float2 pf_wz1[Q12][2];     // W_z,1 at (2i + dy, 2j .. 2j + 1): (dx 0, dx 1) per dy
   float4 pf_wr1[Q12][2];     // W_R,1 at the same pixels
   float2 pf_g2[Q12], pf_q2[Q12], pf_g1[QUP], pf_q1[QUP];
@@ -1396,6 +1398,12 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
         const int p = tid + t * NT;
         const int i = p / wc, j = p % wc;
         float2 zs = czero(), rs = czero();
+        float2 g1 = czero(), q1 = czero();
+        if (l2) {
+          const int li = EMG_INB((rank * hc + i) * wc + j, wc * wc, kBcLevel) ? (rank * hc + i) * wc + j : 0;
+          g1 = __ldcg(a.lv.G[1] + li);
+          q1 = __ldcg(a.lv.Q[1] + li);
+        }
 #pragma unroll
         for (int dy = 0; dy < 2; ++dy) {
           const int lr = 2 * i + dy, r = row0 + lr, c = 2 * j;
@@ -1407,12 +1415,21 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
           zs = cadd(zs, cscale(z_at(lr, c + 1), wz.y));
           rs = cfma(make_float2(wr.z, wr.w), rowbuf[lr * SR + c + 1], rs);
         }
-        Z1w[i * sc + j] = cscale(zs, 0.25f);
-        R1w[i * sc + j] = cscale(rs, 0.25f);
+        const float2 z1 = cscale(zs, 0.25f), r1 = cscale(rs, 0.25f);
+        if (l2) {
+          // coarsest level 1: correction c = G (R - Q z)
+          const float2 cc = cmul(g1, cfnma(q1, z1, r1));
+          Z1w[i * sc + j] = cc;
+          if (halo) push_halo<C>(cl, rank, Z1w, sc, hc, i, j, cc);
+        } else {
+          Z1w[i * sc + j] = z1;
+          R1w[i * sc + j] = r1;
+        }
       }
     }
-    __syncthreads();
-    if (l3) {
+    if (!l2) __syncthreads();
+    if (l2) {
+    } else if (l3) {
       {  // restrict 1 -> 2 from the prefetched weights, and at once the coarsest step
          // on the same level-2 pixel (it needs nothing from other threads)
         constexpr int sf = wc1 + 1, sc = wc2 + 1;
@@ -1446,7 +1463,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
 #pragma unroll
         for (int t = 0; t < QUP; ++t) load_up(t);
       }
-      if (halo) cl.sync();  // the pushed halo rows of level 2 are in place
+      if (halo) tile_sync<C>(cl);  // the pushed halo rows of level 2 are in place
       __syncthreads();
       {  // back up to level 1
         constexpr int sl = wc1 + 1, sc = wc2 + 1;
@@ -1506,7 +1523,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
     // back up: c_l = I_H^h c_{l+1} + G_l (R_l - Q_l (z_l + I_H^h c_{l+1}))
     for (int l = a.levels - 2; l >= 1; --l) {
       if (halo) {
-        cl.sync();
+        tile_sync<C>(cl);
         fill_halo(l + 1);
       }
       __syncthreads();
@@ -1527,8 +1544,8 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
     }
     }  // generic levels
     if (halo) {
-      cl.sync();
-      if (!l3) fill_halo(1);  // three levels: the halo rows were pushed
+      tile_sync<C>(cl);
+      if (!l3 && !l2) fill_halo(1);  // two and three levels: the halo rows were pushed
     }
     __syncthreads();
   }
@@ -1650,13 +1667,13 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
     if (tid == 0) cluster_publish<C>(cl, rank, xd2, part);
   }
   // With halo rows read from the neighbours (bilinear prolongation, other
-  // than three levels) a neighbour may still read my coarse rows: no CTA leaves
+  // than two or three levels) a neighbour may still read my coarse rows: no CTA leaves
   // before all arrive.  The verify mode also publishes xd2, which needs the
   // release / acquire pair.  Otherwise no CTA touches another's shared memory
   // after the last cluster barrier, and each may leave when done.
   if (a.verify) {
-    cl.sync();
-  } else if (halo && !l3 && a.levels > 1) {
+    tile_sync<C>(cl);
+  } else if (C > 1 && halo && !l3 && !l2 && a.levels > 1) {
     cluster_arrive_relaxed();
     cluster_wait();
   }
@@ -2220,19 +2237,6 @@ __global__ void __launch_bounds__(kScaleThreads) k_scale_probe(const double* __r
   for (int p = threadIdx.x; p < m * m; p += kScaleThreads) probe[p] = cscale(probe[p], scale);
 }
 
-template <int M>
-cudaError_t set_step_smem() {
-  return cudaFuncSetAttribute(k_step<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              step_smem_limit());
-}
-
-template <int M>
-cudaError_t launch_step_t(int b, const StepArgs& a, cudaStream_t s) {
-  const size_t bytes = step_smem_elems<M>(a.levels) * sizeof(float2);
-  k_step<M><<<b, StepThreads<M>::value, bytes, s>>>(a);
-  return cudaGetLastError();
-}
-
 #define EMG_DISPATCH_M(m, CALL)        \
   switch (m) {                         \
     case 16: { constexpr int M = 16; return CALL; }   \
@@ -2287,10 +2291,6 @@ cudaError_t upload_twiddles() {
   }
   cudaError_t e = cudaMemcpyToSymbol(c_twiddle, h, sizeof(h));
   if (e != cudaSuccess) return e;
-  if ((e = set_step_smem<16>()) != cudaSuccess) return e;
-  if ((e = set_step_smem<32>()) != cudaSuccess) return e;
-  if ((e = set_step_smem<64>()) != cudaSuccess) return e;
-  if ((e = set_step_smem<128>()) != cudaSuccess) return e;
   if ((e = set_cluster_attrs()) != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
   if (e != cudaSuccess) return e;
@@ -2376,6 +2376,8 @@ int stepc_resident_clusters() {
 
 int step_resident_clusters(int m, int cluster) {
   switch (m * 16 + cluster) {
+    case 16 * 16 + 1: return stepc_resident_clusters<16, 1>();
+    case 32 * 16 + 1: return stepc_resident_clusters<32, 1>();
     case 16 * 16 + 2: return stepc_resident_clusters<16, 2>();
     case 32 * 16 + 2: return stepc_resident_clusters<32, 2>();
     case 64 * 16 + 2: return stepc_resident_clusters<64, 2>();
@@ -2391,6 +2393,8 @@ int step_resident_clusters(int m, int cluster) {
 int fused_prep_tiles(PrepArgs& a, int m, int cluster) {
   size_t smem = 0;
   switch (m * 16 + cluster) {
+    case 16 * 16 + 1: smem = stepc_smem_bytes<16, 1>(); break;
+    case 32 * 16 + 1: smem = stepc_smem_bytes<32, 1>(); break;
     case 16 * 16 + 2: smem = stepc_smem_bytes<16, 2>(); break;
     case 32 * 16 + 2: smem = stepc_smem_bytes<32, 2>(); break;
     case 64 * 16 + 2: smem = stepc_smem_bytes<64, 2>(); break;
@@ -2543,6 +2547,8 @@ cudaError_t set_grad_attrs() {
 // Dynamic shared-memory limits of the cluster kernels (once per device).
 cudaError_t set_cluster_attrs() {
   cudaError_t e;
+  if ((e = set_stepc_attrs<16, 1>()) != cudaSuccess) return e;
+  if ((e = set_stepc_attrs<32, 1>()) != cudaSuccess) return e;
   if ((e = set_stepc_attrs<16, 2>()) != cudaSuccess) return e;
   if ((e = set_stepc_attrs<32, 2>()) != cudaSuccess) return e;
   if ((e = set_stepc_attrs<64, 2>()) != cudaSuccess) return e;
@@ -2603,9 +2609,9 @@ cudaError_t launch_step_rin(int m, int b, const StepArgs& a, cudaStream_t s) {
 
 cudaError_t launch_step(int m, int b, const StepArgs& a, bool overlap, cudaStream_t s) {
   switch (m * 16 + a.cluster) {
-    case 16 * 16 + 1: return launch_step_t<16>(b, a, s);
+    case 16 * 16 + 1: return launch_stepc_t<16, 1>(b, a, overlap, s);
     case 16 * 16 + 2: return launch_stepc_t<16, 2>(b, a, overlap, s);
-    case 32 * 16 + 1: return launch_step_t<32>(b, a, s);
+    case 32 * 16 + 1: return launch_stepc_t<32, 1>(b, a, overlap, s);
     case 32 * 16 + 2: return launch_stepc_t<32, 2>(b, a, overlap, s);
     case 64 * 16 + 2: return launch_stepc_t<64, 2>(b, a, overlap, s);
     case 64 * 16 + 4: return launch_stepc_t<64, 4>(b, a, overlap, s);
@@ -2766,7 +2772,6 @@ bool step_supported(int m, int levels, int cluster) {
   const bool built = (cluster == 1 && m <= 32) || (cluster == 2 && m <= 128) || (cluster == 4 && (m == 64 || m == 128)) ||
                      (cluster == 8 && m >= 128);
   if (!built) return false;
-  if (cluster == 1) return step_smem_bytes(m, levels) <= (size_t)step_smem_limit();
   if ((m >> (levels - 1)) < cluster) return false;  // every CTA needs a row at the coarsest level
   size_t need = 0;
   for (int l = 1; l < levels; ++l) {
@@ -2865,10 +2870,10 @@ cudaError_t noalloc_setup(int dev, unsigned char** base) {
   cudaError_t e = upload_twiddles();
   if (e != cudaSuccess) return e;
   const int lim = step_smem_limit();
-  if ((e = cudaFuncSetAttribute(k_step<16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) ||
-      (e = cudaFuncSetAttribute(k_step<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) ||
-      (e = cudaFuncSetAttribute(k_step<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) ||
-      (e = cudaFuncSetAttribute(k_step<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)))
+  if ((e = cudaFuncSetAttribute(k_step<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) ||
+      (e = cudaFuncSetAttribute(k_step<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) ||
+      (e = cudaFuncSetAttribute(k_step<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) ||
+      (e = cudaFuncSetAttribute(k_step<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)))
     return e;
   void* p = nullptr;
   e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
@@ -2884,7 +2889,7 @@ constexpr int kNoAllocMaxIdx = kSeedMaxIdx;
 template <int M>
 cudaError_t launch_step_natural(int b, const StepArgs& a, cudaStream_t s) {
   const size_t bytes = step_smem_elems<M>(a.levels) * sizeof(float2);
-  k_step<M, true><<<b, StepThreads<M>::value, bytes, s>>>(a);
+  k_step<M><<<b, StepThreads<M>::value, bytes, s>>>(a);
   return cudaGetLastError();
 }
 
