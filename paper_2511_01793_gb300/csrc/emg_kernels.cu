@@ -16,6 +16,8 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "emg_fft.cuh"
 #include "emg_internal.h"
 
@@ -994,7 +996,10 @@ struct StepTile : CTile<M, C> {
 // Forward and gradient kernels: whole launches of many positions, so the
 // shared memory is one slab (transposed in place) and as many CTAs share an SM
 // as 64 registers per thread allow.
-template <int M> struct WaveCluster { static constexpr int value = M == 256 ? 8 : M == 128 ? 2 : 1; };
+// m = 128 fits one CTA of 1024 threads (no distributed shared memory): 900
+// simulated positions 54 us against 64 with clusters of 2 and 62 with 4.  m = 256:
+// clusters of 8 with two CTAs per SM 383 us for 1024 positions, of 4 with one 422.
+template <int M> struct WaveCluster { static constexpr int value = M == 256 ? 8 : 1; };
 template <int M>
 struct WaveTile : CTile<M, WaveCluster<M>::value> {
   using B = CTile<M, WaveCluster<M>::value>;
@@ -1124,6 +1129,56 @@ __device__ __forceinline__ void push_halo(cg::cluster_group& cl, int rank, T* y,
   }
 }
 
+// One column of the object under a patch: pixel rows below (row0, col), 0 outside.
+struct ObjectColumn {
+  const float2* base;  // only dereferenced where the pixel exists
+  int row0, n_rows, n_cols;
+  bool col_ok;
+  __device__ __forceinline__ ObjectColumn(const float2* object, int rows, int cols, int r, int c)
+      : base(object + ((ptrdiff_t)r * cols + c)), row0(r), n_rows(rows), n_cols(cols),
+        col_ok((unsigned)c < (unsigned)cols) {}
+  __device__ __forceinline__ float2 at(int dr) const {
+    if (col_ok && (unsigned)(row0 + dr) < (unsigned)n_rows) return base[(ptrdiff_t)dr * n_cols];
+    return czero();
+  }
+};
+
+// I_H^h at fine pixel (r, c) and at the pixels an even number of rows below it,
+// from a coarse row slab with one halo row on each side (y: my first row).
+struct CoarseCell {
+  const float2* y;
+  int dn, dj;  // offsets of the vertical and horizontal neighbours
+  __device__ __forceinline__ CoarseCell(const float2* z, int stride, int width, int r, int c)
+      : y(z + (r >> 1) * stride + (c >> 1)), dn((r & 1) ? stride : -stride),
+        dj((c & 1) ? ((c >> 1) + 1 < width ? 1 : 0) : ((c >> 1) > 0 ? -1 : 0)) {}
+  __device__ __forceinline__ float2 at(int off, bool bilinear) const {
+    const float2* p = y + off;
+    const float2 v = p[0];
+    if (!bilinear) return v;
+    return lerp4<float2>(v, p[dn], p[dj], p[dn + dj]);
+  }
+};
+
+// The same at the pixel pair (r, c), (r, c + 1), c even: rows and centre column shared.
+struct CoarsePair {
+  const float2* y;
+  int dn, jm, jp;
+  __device__ __forceinline__ CoarsePair(const float2* z, int stride, int width, int r, int c)
+      : y(z + (r >> 1) * stride + (c >> 1)), dn((r & 1) ? stride : -stride), jm((c >> 1) > 0 ? -1 : 0),
+        jp((c >> 1) + 1 < width ? 1 : 0) {}
+  __device__ __forceinline__ void at(int off, bool bilinear, float2 (&pro)[2]) const {
+    const float2* p = y + off;
+    const float2 v = p[0];
+    if (!bilinear) {
+      pro[0] = pro[1] = v;
+      return;
+    }
+    const float2 w = p[dn];
+    pro[0] = lerp4<float2>(v, w, p[jm], p[dn + jm]);
+    pro[1] = lerp4<float2>(v, w, p[jp], p[dn + jp]);
+  }
+};
+
 // RIN = true: the revised exit waves R_k and the misfit partials come from the
 // tensor-core DFT pair (a2-a4 done elsewhere); the kernel gathers z_k and runs
 // a5-a7 only.
@@ -1199,13 +1254,6 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   }
   pdl_trigger();
   pdl_wait();  // object, probe, max|Q|^2 and level arrays come from earlier kernels
-  // z_k at my local row lr, column c: the kept copy, or the object (0 outside)
-  auto z_at = [&](int lr, int c) -> float2 {
-    if constexpr (ONE)
-      return gather_obj(a.object, a.n_rows, a.n_cols, o_r + row0 + lr, o_c + c);
-    else
-      return zbuf[lr * M + c];
-  };
   const float MQ = __uint_as_float(*a.mq);
   if constexpr (C > 1) cluster_arrive_relaxed();  // completed (wait) before the first distributed shared memory access
 
@@ -1218,17 +1266,24 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
 #else
   constexpr int kGatherUnroll = M >= 128 ? 8 : 4;
 #endif
+  // A thread's pixels lie in one column, RPT rows apart (NT is a multiple of M),
+  // so every address is a base of the thread plus a constant per pixel.
+  constexpr int RPT = NT / M;
+  static_assert(NT % M == 0, "a thread's pixels share one column");
+  {
+    const int l0 = tid / M, c0 = tid % M;
+    const ObjectColumn zc(a.object, a.n_rows, a.n_cols, o_r + row0 + l0, o_c + c0);
+    float2* rb = rowbuf + l0 * SR + c0;
+    const float2* src = RIN ? a.r_in + (size_t)kb * M * M : a.probe;
+    src += row0 * M + tid;
 #pragma unroll (kGatherUnroll)
-  for (int t = 0; t < PER; ++t) {
-    const int p = tid + t * NT;
-    const int lr = p / M, c = p % M, r = row0 + lr;
-    const float2 zk = gather_obj(a.object, a.n_rows, a.n_cols, o_r + r, o_c + c);
-    if constexpr (!ONE) zbuf[p] = zk;
-    if constexpr (RIN)
-      rowbuf[lr * SR + c] = a.r_in[(size_t)kb * M * M + r * M + c];
-    else
-      rowbuf[lr * SR + c] = cmul(a.probe[r * M + c], zk);
-    mu_l = fmaxf(mu_l, cabs2(zk));
+    for (int t = 0; t < PER; ++t) {
+      const float2 zk = zc.at(t * RPT);
+      if constexpr (!ONE) zbuf[tid + t * NT] = zk;
+      const float2 x = src[t * NT];
+      rb[t * RPT * SR] = RIN ? x : cmul(x, zk);
+      mu_l = fmaxf(mu_l, cabs2(zk));
+    }
   }
   // per-warp maxima of |z_k|^2; the barrier also orders the gather before the row passes
   warp_partial_max(mu_l, redf);
@@ -1300,7 +1355,8 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
 
   if constexpr (!RIN) {
     if (a.prep_clusters > 0) {
-      // the level arrays of this minibatch come from the prep clusters of this launch
+      // the level arrays of this minibatch (with one level the gain G_0 alone) come
+      // from the prep clusters of this launch
       if (tid == 0) {
         const unsigned long long t0 = globaltimer_ns();
         while (ld_acquire_u32(a.sync + 1) < a.prep_target) {
@@ -1315,9 +1371,48 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   }
   // a5: MAGPIE multigrid on row slabs; level-l buffers (l >= 1) in mgbuf.
   // Z_l keeps one halo row above and below my rows for the prolongation.
-  float2* Zl[kMaxLevels];
-  float2* Rl[kMaxLevels];
-  {
+  const bool halo = a.prolong != 0;
+  constexpr int W1 = M / 2, H1 = W1 / C, S1 = W1 + 1;  // level 1: width, my rows, row stride
+  constexpr int W2 = M / 4, H2 = W2 / C, S2 = W2 + 1;  // level 2
+  float2* const Z1 = mgbuf + S1;
+  float2* const R1 = mgbuf + (H1 + 2) * S1;
+  float2* const Z2 = R1 + H1 * S1 + S2;
+  // Level-1 pixels of a thread: one column, RP1 rows apart (even, so the
+  // prolongation's neighbours lie on the same side for all of them).
+  constexpr int P1 = H1 * W1 / NT, RP1 = NT / W1;
+  static_assert(H1 * W1 % NT == 0 && NT % W1 == 0 && RP1 % 2 == 0, "level 1 splits evenly over the threads");
+  const int i1 = tid / W1, j1 = tid % W1;
+  // Level-2 pixels; where a slab has fewer than NT of them the other threads have none.
+  constexpr bool kHas2 = H2 >= 1 && (H2 * W2 % NT == 0 || H2 * W2 < NT);
+  constexpr int P2 = kHas2 && H2 * W2 >= NT ? H2 * W2 / NT : 1, RP2 = NT / W2;
+  const int i2 = tid / W2, j2 = tid % W2;
+  const bool on2 = H2 * W2 >= NT || tid < H2 * W2;
+  // With two levels the coarse step follows the restriction at the same pixel
+  // at once (it needs nothing from other threads).  With three levels every
+  // level array the coarse levels need is loaded into registers beside the
+  // loads of the first restriction, so the coarse phases wait on no load
+  // (ONE: where they are used; the other CTA of the SM covers the wait and the
+  // registers are not there to hold them).  More levels take the general loops.
+  const bool l3 = kHas2 && a.levels == 3;
+  // Copies the rows of the coarse correction at level l (Z: my first row) adjacent
+  // to my slab (from the neighbouring ranks, or my own edge row where the patch ends).
+  auto fill_halo = [&](float2* Z, int l) {
+    const int wl = M >> l, hl = wl / C, sl = wl + 1;
+    const float2* Zup = Z;
+    const float2* Zdn = Z;
+    if constexpr (C > 1) {
+      if (rank > 0) Zup = cl.map_shared_rank(Z, rank - 1);
+      if (rank < C - 1) Zdn = cl.map_shared_rank(Z, rank + 1);
+    }
+    for (int j = tid; j < wl; j += NT) {
+      Z[-sl + j] = rank > 0 ? Zup[(hl - 1) * sl + j] : Z[j];
+      Z[hl * sl + j] = rank < C - 1 ? Zdn[j] : Z[(hl - 1) * sl + j];
+    }
+  };
+  // Levels 1 .. L - 1 for any L, from Z_1 and R_1 to the correction at level 1.
+  auto general_levels = [&]() {
+    float2* Zl[kMaxLevels];
+    float2* Rl[kMaxLevels];
     size_t off = 0;
     for (int l = 1; l < a.levels; ++l) {
       const int wl = M >> l, hl = wl / C, sl = wl + 1;
@@ -1326,161 +1421,6 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
       Rl[l] = mgbuf + off;
       off += (size_t)hl * sl;
     }
-  }
-  // Copies the rows of the coarse correction at level l adjacent to my slab
-  // (from the neighbouring ranks, or my own edge row where the patch ends).
-  auto fill_halo = [&](int l) {
-    const int wl = M >> l, hl = wl / C, sl = wl + 1;
-    float2* Z = Zl[l];
-    const float2* Zup = Z;
-    const float2* Zdn = Z;
-    if constexpr (C > 1) {
-      if (rank > 0) Zup = cl.map_shared_rank(Zl[l], rank - 1);
-      if (rank < C - 1) Zdn = cl.map_shared_rank(Zl[l], rank + 1);
-    }
-    for (int j = tid; j < wl; j += NT) {
-      Z[-sl + j] = rank > 0 ? Zup[(hl - 1) * sl + j] : Z[j];
-      Z[hl * sl + j] = rank < C - 1 ? Zdn[j] : Z[(hl - 1) * sl + j];
-    }
-  };
-  const bool halo = a.prolong != 0;
-  // With three levels (and slabs that split evenly over the threads) every
-  // level array the coarse levels need is loaded into registers here, beside
-  // the loads of the first restriction, so the coarse phases wait on no load
-  // (ONE: where they are used; the other CTA of the SM covers the wait and the
-  // registers are not there to hold them).
-  constexpr int wc1 = M / 2, hc1 = wc1 / C, wc2 = M / 4, hc2 = wc2 / C;
-  constexpr bool kL3 = hc2 >= 1 && hc2 * wc2 >= NT && (hc2 * wc2) % NT == 0 && (hc1 * wc1) % NT == 0;
-  constexpr int Q12 = kL3 ? hc2 * wc2 / NT : 1, QUP = kL3 ? hc1 * wc1 / NT : 1;
-  const bool l3 = kL3 && a.levels == 3;
-  // With two levels the coarse step follows the restriction at the same pixel
-  // at once (it needs nothing from other threads), and its halo rows are pushed.
-  const bool l2 = a.levels == 2;
-  float2 pf_wz1[Q12][2];     // W_z,1 at (2i + dy, 2j .. 2j + 1): (dx 0, dx 1) per dy
-  float4 pf_wr1[Q12][2];     // W_R,1 at the same pixels
-  float2 pf_g2[Q12], pf_q2[Q12], pf_g1[QUP], pf_q1[QUP];
-  auto load_l2 = [&](int t) {
-    const int p = tid + t * NT, i = p / wc2, j = p % wc2;
-#pragma unroll
-    for (int dy = 0; dy < 2; ++dy) {
-      const int r = rank * hc1 + 2 * i + dy, c = 2 * j;
-      const int wi = EMG_INB(r * wc1 + c + 1, wc1 * wc1, kBcLevel) ? r * wc1 + c : 0;
-      pf_wz1[t][dy] = __ldcg(reinterpret_cast<const float2*>(a.lv.Wz[1] + wi));
-      pf_wr1[t][dy] = __ldcg(reinterpret_cast<const float4*>(a.lv.WR[1] + wi));
-    }
-    const int li = EMG_INB((rank * hc2 + i) * wc2 + j, wc2 * wc2, kBcLevel) ? (rank * hc2 + i) * wc2 + j : 0;
-    pf_g2[t] = __ldcg(a.lv.G[2] + li);
-    pf_q2[t] = __ldcg(a.lv.Q[2] + li);
-  };
-  auto load_up = [&](int t) {
-    const int p = tid + t * NT, i = p / wc1, j = p % wc1;
-    const int li = EMG_INB((rank * hc1 + i) * wc1 + j, wc1 * wc1, kBcLevel) ? (rank * hc1 + i) * wc1 + j : 0;
-    pf_g1[t] = __ldcg(a.lv.G[1] + li);
-    pf_q1[t] = __ldcg(a.lv.Q[1] + li);
-  };
-  if (a.levels > 1) {
-    if (l3 && !ONE) {
-#pragma unroll
-      for (int t = 0; t < Q12; ++t) load_l2(t);
-#pragma unroll
-      for (int t = 0; t < QUP; ++t) load_up(t);
-    }
-    {  // restrict level 0 -> 1: z_1 = I_h^H (W_z z_k), R_1 = I_h^H (W_R R)
-      constexpr int wc = M / 2, hc = wc / C, sc = wc + 1;
-      constexpr int PC = hc * wc / NT;
-      static_assert(hc * wc % NT == 0, "coarse slab must split evenly");
-      const float* Wz = a.lv.Wz[0];
-      const float2* WR = a.lv.WR[0];
-      float2* __restrict__ const Z1w = Zl[1];
-      float2* __restrict__ const R1w = Rl[1];
-#pragma unroll
-      for (int t = 0; t < PC; ++t) {
-        const int p = tid + t * NT;
-        const int i = p / wc, j = p % wc;
-        float2 zs = czero(), rs = czero();
-        float2 g1 = czero(), q1 = czero();
-        if (l2) {
-          const int li = EMG_INB((rank * hc + i) * wc + j, wc * wc, kBcLevel) ? (rank * hc + i) * wc + j : 0;
-          g1 = __ldcg(a.lv.G[1] + li);
-          q1 = __ldcg(a.lv.Q[1] + li);
-        }
-#pragma unroll
-        for (int dy = 0; dy < 2; ++dy) {
-          const int lr = 2 * i + dy, r = row0 + lr, c = 2 * j;
-          // the weights of the pixel pair (c, c + 1) in one load each (c is even)
-          const float2 wz = __ldcg(reinterpret_cast<const float2*>(Wz + r * M + c));
-          const float4 wr = __ldcg(reinterpret_cast<const float4*>(WR + r * M + c));
-          zs = cadd(zs, cscale(z_at(lr, c), wz.x));
-          rs = cfma(make_float2(wr.x, wr.y), rowbuf[lr * SR + c], rs);
-          zs = cadd(zs, cscale(z_at(lr, c + 1), wz.y));
-          rs = cfma(make_float2(wr.z, wr.w), rowbuf[lr * SR + c + 1], rs);
-        }
-        const float2 z1 = cscale(zs, 0.25f), r1 = cscale(rs, 0.25f);
-        if (l2) {
-          // coarsest level 1: correction c = G (R - Q z)
-          const float2 cc = cmul(g1, cfnma(q1, z1, r1));
-          Z1w[i * sc + j] = cc;
-          if (halo) push_halo<C>(cl, rank, Z1w, sc, hc, i, j, cc);
-        } else {
-          Z1w[i * sc + j] = z1;
-          R1w[i * sc + j] = r1;
-        }
-      }
-    }
-    if (!l2) __syncthreads();
-    if (l2) {
-    } else if (l3) {
-      {  // restrict 1 -> 2 from the prefetched weights, and at once the coarsest step
-         // on the same level-2 pixel (it needs nothing from other threads)
-        constexpr int sf = wc1 + 1, sc = wc2 + 1;
-        const float2* __restrict__ const Zf = Zl[1];
-        const float2* __restrict__ const Rf = Rl[1];
-        float2* __restrict__ const Zc = Zl[2];
-        if constexpr (ONE) {
-#pragma unroll
-          for (int t = 0; t < Q12; ++t) load_l2(t);
-        }
-#pragma unroll
-        for (int t = 0; t < Q12; ++t) {
-          const int p = tid + t * NT, i = p / wc2, j = p % wc2;
-          float2 zs = czero(), rs = czero();
-#pragma unroll
-          for (int dy = 0; dy < 2; ++dy) {
-            const int lr = 2 * i + dy, c = 2 * j;
-            zs = cadd(zs, cscale(Zf[lr * sf + c], pf_wz1[t][dy].x));
-            rs = cfma(make_float2(pf_wr1[t][dy].x, pf_wr1[t][dy].y), Rf[lr * sf + c], rs);
-            zs = cadd(zs, cscale(Zf[lr * sf + c + 1], pf_wz1[t][dy].y));
-            rs = cfma(make_float2(pf_wr1[t][dy].z, pf_wr1[t][dy].w), Rf[lr * sf + c + 1], rs);
-          }
-          const float2 z2 = cscale(zs, 0.25f), r2 = cscale(rs, 0.25f);
-          // coarsest level 2: correction c = G (R - Q z), stored over z
-          const float2 cc = cmul(pf_g2[t], cfnma(pf_q2[t], z2, r2));
-          Zc[i * sc + j] = cc;
-          if (halo) push_halo<C>(cl, rank, Zc, sc, hc2, i, j, cc);
-        }
-      }
-      if constexpr (ONE) {
-#pragma unroll
-        for (int t = 0; t < QUP; ++t) load_up(t);
-      }
-      if (halo) tile_sync<C>(cl);  // the pushed halo rows of level 2 are in place
-      __syncthreads();
-      {  // back up to level 1
-        constexpr int sl = wc1 + 1, sc = wc2 + 1;
-        float2* __restrict__ const Zw = Zl[1];
-        const float2* __restrict__ const Rw = Rl[1];
-        const float2* __restrict__ const Zc = Zl[2];
-#pragma unroll
-        for (int t = 0; t < QUP; ++t) {
-          const int p = tid + t * NT, i = p / wc1, j = p % wc1;
-          const float2 pro = prolong_halo<float2>(Zc, sc, wc2, i, j, a.prolong);
-          const float2 zp = cadd(Zw[i * sl + j], pro);
-          const float2 cc = cfma(pf_g1[t], cfnma(pf_q1[t], zp, Rw[i * sl + j]), pro);
-          Zw[i * sl + j] = cc;
-          if (halo) push_halo<C>(cl, rank, Zw, sl, hc1, i, j, cc);
-        }
-      }
-    } else {
     for (int l = 1; l + 1 < a.levels; ++l) {
       const int wf = M >> l, sf = wf + 1, hf = wf / C, wc = wf >> 1, hc = wc / C, sc = wc + 1;
       const float* Wz = a.lv.Wz[l];
@@ -1524,7 +1464,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
     for (int l = a.levels - 2; l >= 1; --l) {
       if (halo) {
         tile_sync<C>(cl);
-        fill_halo(l + 1);
+        fill_halo(Zl[l + 1], l + 1);
       }
       __syncthreads();
       const int wl = M >> l, hl = wl / C, sl = wl + 1, wc = wl >> 1, sc = wc + 1;
@@ -1542,10 +1482,139 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
         Zw[i * sl + j] = cadd(pro, cmul(__ldcg(G + li), csub(Rw[i * sl + j], cmul(__ldcg(Q + li), zp))));
       }
     }
-    }  // generic levels
+  };
+  if (a.levels > 1) {
+    float2 pf_wz1[P2][2];     // W_z,1 at (2i + dy, 2j .. 2j + 1): (dx 0, dx 1) per dy
+    float4 pf_wr1[P2][2];     // W_R,1 at the same pixels
+    float2 pf_g2[P2], pf_q2[P2], pf_g1[P1], pf_q1[P1];
+    auto load_down = [&]() {
+#pragma unroll
+      for (int t = 0; t < P2; ++t) {
+        if (!on2) break;
+        const int i = i2 + t * RP2, wb = (rank * H1 + 2 * i) * W1 + 2 * j2, lb = (rank * H2 + i) * W2 + j2;
+#pragma unroll
+        for (int dy = 0; dy < 2; ++dy) {
+          const int wi = EMG_INB(wb + dy * W1 + 1, W1 * W1, kBcLevel) ? wb + dy * W1 : 0;
+          pf_wz1[t][dy] = __ldcg(reinterpret_cast<const float2*>(a.lv.Wz[1] + wi));
+          pf_wr1[t][dy] = __ldcg(reinterpret_cast<const float4*>(a.lv.WR[1] + wi));
+        }
+        const int li = EMG_INB(lb, W2 * W2, kBcLevel) ? lb : 0;
+        pf_g2[t] = __ldcg(a.lv.G[2] + li);
+        pf_q2[t] = __ldcg(a.lv.Q[2] + li);
+      }
+    };
+    auto load_up = [&]() {
+#pragma unroll
+      for (int t = 0; t < P1; ++t) {
+        const int lb = rank * H1 * W1 + tid + t * NT;
+        const int li = EMG_INB(lb, W1 * W1, kBcLevel) ? lb : 0;
+        pf_g1[t] = __ldcg(a.lv.G[1] + li);
+        pf_q1[t] = __ldcg(a.lv.Q[1] + li);
+      }
+    };
+    // restrict level 0 -> 1: z_1 = I_h^H (W_z z_k), R_1 = I_h^H (W_R R); with
+    // two levels at once the coarsest step c = G (R - Q z)
+    auto restrict_top = [&](auto two_levels) {
+      constexpr bool kTwo = decltype(two_levels)::value;
+      const int f0 = 2 * i1, c0 = 2 * j1;  // fine pixel of the first coarse one, 2 RP1 rows apart
+      const float* Wz = a.lv.Wz[0] + (row0 + f0) * M + c0;
+      const float2* WR = a.lv.WR[0] + (row0 + f0) * M + c0;
+      const float2* rb = rowbuf + f0 * SR + c0;
+      const ObjectColumn za(a.object, a.n_rows, a.n_cols, o_r + row0 + f0, o_c + c0);
+      const ObjectColumn zb(a.object, a.n_rows, a.n_cols, o_r + row0 + f0, o_c + c0 + 1);
+      float2* zw = Z1 + i1 * S1 + j1;
+      float2* rw = R1 + i1 * S1 + j1;
+#pragma unroll
+      for (int t = 0; t < P1; ++t) {
+        float2 zs = czero(), rs = czero();
+#pragma unroll
+        for (int dy = 0; dy < 2; ++dy) {
+          const int fr = 2 * RP1 * t + dy;
+          // the weights of the pixel pair (c, c + 1) in one load each (c is even)
+          const float2 wz = __ldcg(reinterpret_cast<const float2*>(Wz + fr * M));
+          const float4 wr = __ldcg(reinterpret_cast<const float4*>(WR + fr * M));
+          float2 z0, z1;
+          if constexpr (ONE) {
+            z0 = za.at(fr);
+            z1 = zb.at(fr);
+          } else {
+            z0 = zbuf[(f0 + fr) * M + c0];
+            z1 = zbuf[(f0 + fr) * M + c0 + 1];
+          }
+          zs = cadd(zs, cscale(z0, wz.x));
+          rs = cfma(make_float2(wr.x, wr.y), rb[fr * SR], rs);
+          zs = cadd(zs, cscale(z1, wz.y));
+          rs = cfma(make_float2(wr.z, wr.w), rb[fr * SR + 1], rs);
+        }
+        const float2 z1 = cscale(zs, 0.25f), r1 = cscale(rs, 0.25f);
+        if constexpr (kTwo) {
+          const float2 cc = cmul(pf_g1[t], cfnma(pf_q1[t], z1, r1));
+          zw[t * RP1 * S1] = cc;
+          if (halo) push_halo<C>(cl, rank, Z1, S1, H1, i1 + t * RP1, j1, cc);
+        } else {
+          zw[t * RP1 * S1] = z1;
+          rw[t * RP1 * S1] = r1;
+        }
+      }
+    };
+    if (a.levels == 2) {
+      load_up();
+      restrict_top(std::true_type{});
+    } else {
+      if (!ONE && l3) {
+        load_down();
+        load_up();
+      }
+      restrict_top(std::false_type{});
+      __syncthreads();
+      if (l3) {
+        if (ONE) load_down();
+        // restrict 1 -> 2 and at once the coarsest step on the same level-2 pixel
+        if (on2) {
+          const float2* zf = Z1 + 2 * i2 * S1 + 2 * j2;
+          const float2* rf = R1 + 2 * i2 * S1 + 2 * j2;
+          float2* zw = Z2 + i2 * S2 + j2;
+#pragma unroll
+          for (int t = 0; t < P2; ++t) {
+            float2 zs = czero(), rs = czero();
+#pragma unroll
+            for (int dy = 0; dy < 2; ++dy) {
+              const int at = (2 * RP2 * t + dy) * S1;
+              zs = cadd(zs, cscale(zf[at], pf_wz1[t][dy].x));
+              rs = cfma(make_float2(pf_wr1[t][dy].x, pf_wr1[t][dy].y), rf[at], rs);
+              zs = cadd(zs, cscale(zf[at + 1], pf_wz1[t][dy].y));
+              rs = cfma(make_float2(pf_wr1[t][dy].z, pf_wr1[t][dy].w), rf[at + 1], rs);
+            }
+            const float2 z2 = cscale(zs, 0.25f), r2 = cscale(rs, 0.25f);
+            // coarsest level 2: correction c = G (R - Q z), stored over z
+            const float2 cc = cmul(pf_g2[t], cfnma(pf_q2[t], z2, r2));
+            zw[t * RP2 * S2] = cc;
+            if (halo) push_halo<C>(cl, rank, Z2, S2, H2, i2 + t * RP2, j2, cc);
+          }
+        }
+        if (ONE) load_up();
+        if (halo) tile_sync<C>(cl);  // the pushed halo rows of level 2 are in place
+        __syncthreads();
+        {  // back up to level 1
+          const CoarseCell cell(Z2, S2, W2, i1, j1);
+          float2* zw = Z1 + i1 * S1 + j1;
+          const float2* rw = R1 + i1 * S1 + j1;
+#pragma unroll
+          for (int t = 0; t < P1; ++t) {
+            const float2 pro = cell.at(t * (RP1 / 2) * S2, halo);
+            const float2 zp = cadd(zw[t * RP1 * S1], pro);
+            const float2 cc = cfma(pf_g1[t], cfnma(pf_q1[t], zp, rw[t * RP1 * S1]), pro);
+            zw[t * RP1 * S1] = cc;
+            if (halo) push_halo<C>(cl, rank, Z1, S1, H1, i1 + t * RP1, j1, cc);
+          }
+        }
+      } else {
+        general_levels();
+      }
+    }
     if (halo) {
       tile_sync<C>(cl);
-      if (!l3 && !l2) fill_halo(1);  // two and three levels: the halo rows were pushed
+      if (a.levels > 2 && !l3) fill_halo(Z1, 1);  // two and three levels: the halo rows were pushed
     }
     __syncthreads();
   }
@@ -1555,7 +1624,6 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   const float inv_mu = mu > 0.f ? 1.f / mu : 0.f;
   float2* zt = a.zt + (size_t)kb * M * M;
   float2* qt = a.qt + (size_t)kb * M * M;
-  const float2* Z1 = Zl[1];
   const float2* G0 = a.lv.G[0];
   float acc_after = 0.f;
   // Groups of UG pixels: the probe and gain loads of a group are issued
@@ -1564,64 +1632,78 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   constexpr int UGM = ONE ? 4 : EMG_UPDATE_GROUP;
   constexpr int UG0 = UGM < PER ? UGM : PER;
   constexpr int UG = PER % UG0 == 0 ? UG0 : 1;
-  // The common case (multigrid, joint step, ordered combine, no verify) runs a
-  // loop without the mode branches over pairs of adjacent pixels, with 16-byte
-  // probe and gain loads and patch stores, and the prolongation's loads shared
-  // by the pair; the arithmetic per pixel is the same as in the general loop.
+  // The common case (ordered combine, no verify) runs a loop without the mode
+  // branches over pairs of adjacent pixels, with 16-byte probe and gain loads
+  // and patch stores, and the prolongation's loads shared by the pair; the
+  // arithmetic per pixel is the same as in the general loop.  A thread's pairs
+  // lie in one column pair, RP rows apart (even).
   constexpr int UGP = UG >= 2 && PER % 2 == 0 ? UG / 2 : 0;
-  const bool pairs = UGP > 0 && a.levels > 1 && a.joint && !a.s_num && !a.verify && slot_ok &&
+  const bool pairs = UGP > 0 && !a.s_num && !a.verify && slot_ok &&
                      ((reinterpret_cast<uintptr_t>(a.probe) | reinterpret_cast<uintptr_t>(G0) |
                        reinterpret_cast<uintptr_t>(zt) | reinterpret_cast<uintptr_t>(qt)) & 15) == 0;
+  auto update_pairs = [&](auto multigrid, auto joint) {
+    constexpr bool kMg = decltype(multigrid)::value, kJoint = decltype(joint)::value;
+    constexpr int PP = PER / 2, RP = 2 * RPT;
+    const int l0 = 2 * tid / M, c0 = 2 * tid % M;
+    const float2* rb = rowbuf + l0 * SR + c0;
+    const ObjectColumn za(a.object, a.n_rows, a.n_cols, o_r + row0 + l0, o_c + c0);
+    const ObjectColumn zb(a.object, a.n_rows, a.n_cols, o_r + row0 + l0, o_c + c0 + 1);
+    const CoarsePair cell(Z1, S1, W1, l0, c0);
+    const int off0 = row0 * M + 2 * tid;
+#pragma unroll 1
+    for (int t0 = 0; t0 < PP; t0 += UGP) {
+      float4 qv[UGP], gv[UGP];
+#pragma unroll
+      for (int u = 0; u < UGP; ++u) {
+        const int off = off0 + 2 * (t0 + u) * NT;
+        qv[u] = __ldg(reinterpret_cast<const float4*>(a.probe + off));
+        gv[u] = __ldcg(reinterpret_cast<const float4*>(G0 + off));
+      }
+      [[maybe_unused]] float4 zv[ONE ? UGP : 1];
+      if constexpr (ONE) {
+#pragma unroll
+        for (int u = 0; u < UGP; ++u) {
+          const float2 z0 = za.at((t0 + u) * RP), z1 = zb.at((t0 + u) * RP);
+          zv[u] = make_float4(z0.x, z0.y, z1.x, z1.y);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < UGP; ++u) {
+        const int t = t0 + u;
+        float4 zk2;
+        if constexpr (ONE)
+          zk2 = zv[u];
+        else
+          zk2 = *reinterpret_cast<const float4*>(zbuf + 2 * tid + 2 * t * NT);
+        // coarse-level correction at both pixels
+        float2 pro[2] = {czero(), czero()};
+        if constexpr (kMg) cell.at(t * (RP / 2) * S1, halo, pro);
+        float2 zo[2], qo[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float2 zk = h ? make_float2(zk2.z, zk2.w) : make_float2(zk2.x, zk2.y);
+          const float2 q = h ? make_float2(qv[u].z, qv[u].w) : make_float2(qv[u].x, qv[u].y);
+          const float2 g0 = h ? make_float2(gv[u].z, gv[u].w) : make_float2(gv[u].x, gv[u].y);
+          update_pixel<kMg, kJoint>(zk, q, g0, rb[t * RP * SR + h], pro[h], inv_mu, zo[h], qo[h]);
+        }
+        const int off = off0 + 2 * t * NT;
+        *reinterpret_cast<float4*>(zt + off) = make_float4(zo[0].x, zo[0].y, zo[1].x, zo[1].y);
+        *reinterpret_cast<float4*>(qt + off) = make_float4(qo[0].x, qo[0].y, qo[1].x, qo[1].y);
+      }
+    }
+  };
   if constexpr (UGP > 0) {
     if (pairs) {
-      constexpr int PP = PER / 2;
-      constexpr int SL1 = M / 2 + 1, WC1 = M / 2;
-#pragma unroll 1
-      for (int t0 = 0; t0 < PP; t0 += UGP) {
-        float4 qv[UGP], gv[UGP];
-#pragma unroll
-        for (int u = 0; u < UGP; ++u) {
-          const int off = row0 * M + 2 * (tid + (t0 + u) * NT);
-          qv[u] = __ldg(reinterpret_cast<const float4*>(a.probe + off));
-          gv[u] = __ldcg(reinterpret_cast<const float4*>(G0 + off));
-        }
-#pragma unroll
-        for (int u = 0; u < UGP; ++u) {
-          const int p0 = 2 * (tid + (t0 + u) * NT);
-          const int lr = p0 / M, c0 = p0 % M, r = row0 + lr;
-          float4 zk2;
-          if constexpr (ONE) {
-            const float2 za = z_at(lr, c0), zb = z_at(lr, c0 + 1);
-            zk2 = make_float4(za.x, za.y, zb.x, zb.y);
-          } else {
-            zk2 = *reinterpret_cast<const float4*>(zbuf + p0);
-          }
-          // coarse-level correction at both pixels: the rows and the centre column are shared
-          float2 pro[2];
-          {
-            const int i = lr >> 1, j = c0 >> 1;
-            const float2* y0 = Z1 + i * SL1;
-            const float2 v = y0[j];
-            if (a.prolong == 0) {
-              pro[0] = pro[1] = v;
-            } else {
-              const float2* y1 = Z1 + ((lr & 1) ? i + 1 : i - 1) * SL1;
-              const int jm = max(j - 1, 0), jp = min(j + 1, WC1 - 1);
-              pro[0] = lerp4<float2>(v, y1[j], y0[jm], y1[jm]);
-              pro[1] = lerp4<float2>(v, y1[j], y0[jp], y1[jp]);
-            }
-          }
-          float2 zo[2], qo[2];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const float2 zk = h ? make_float2(zk2.z, zk2.w) : make_float2(zk2.x, zk2.y);
-            const float2 q = h ? make_float2(qv[u].z, qv[u].w) : make_float2(qv[u].x, qv[u].y);
-            const float2 g0 = h ? make_float2(gv[u].z, gv[u].w) : make_float2(gv[u].x, gv[u].y);
-            update_pixel<true, true>(zk, q, g0, rowbuf[lr * SR + c0 + h], pro[h], inv_mu, zo[h], qo[h]);
-          }
-          *reinterpret_cast<float4*>(zt + r * M + c0) = make_float4(zo[0].x, zo[0].y, zo[1].x, zo[1].y);
-          *reinterpret_cast<float4*>(qt + r * M + c0) = make_float4(qo[0].x, qo[0].y, qo[1].x, qo[1].y);
-        }
+      if (a.levels > 1) {
+        if (a.joint)
+          update_pairs(std::true_type{}, std::true_type{});
+        else
+          update_pairs(std::true_type{}, std::false_type{});
+      } else {
+        if (a.joint)
+          update_pairs(std::false_type{}, std::true_type{});
+        else
+          update_pairs(std::false_type{}, std::false_type{});
       }
     }
   }
@@ -1638,10 +1720,14 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
     const int t = t0 + u;
     const int p = tid + t * NT;
     const int lr = p / M, c = p % M, r = row0 + lr;
-    const float2 zk = z_at(lr, c);
+    float2 zk;
+    if constexpr (ONE)
+      zk = gather_obj(a.object, a.n_rows, a.n_cols, o_r + r, o_c + c);
+    else
+      zk = zbuf[p];
     const float2 q = qv[u];
     const float2 R = rowbuf[lr * SR + c];
-    const float2 pro = a.levels == 1 ? czero() : prolong_halo<float2>(Z1, M / 2 + 1, M / 2, lr, c, a.prolong);
+    const float2 pro = a.levels == 1 ? czero() : prolong_halo<float2>(Z1, S1, W1, lr, c, a.prolong);
     float2 zn, qn;
     if (a.levels == 1) {
       if (a.joint)
@@ -1673,7 +1759,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   // after the last cluster barrier, and each may leave when done.
   if (a.verify) {
     tile_sync<C>(cl);
-  } else if (C > 1 && halo && !l3 && !l2 && a.levels > 1) {
+  } else if (C > 1 && halo && !l3 && a.levels > 2) {
     cluster_arrive_relaxed();
     cluster_wait();
   }
@@ -1715,21 +1801,23 @@ __global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_forw
   const int t = blockIdx.x / C;
   const int row0 = rank * H;
   const float inv_m2 = 1.f / (float)(M * M);
+  // a thread's pixels: one column, RPT rows apart
+  constexpr int RPT = NT / M;
+  static_assert(NT % M == 0, "a thread's pixels share one column");
+  float2* mine = sm + (tid / M) * S + tid % M;
   if constexpr (MODE >= 2) {
-    const float2* x = a.in + (size_t)t * M * M + row0 * M;
+    const float2* x = a.in + (size_t)t * M * M + row0 * M + tid;
 #pragma unroll (PER < 8 ? PER : 8)
     for (int u = 0; u < PER; ++u) {
-      const int p = tid + u * NT;
-      const float2 v = x[p];
-      sm[(p / M) * S + p % M] = MODE == 3 ? make_float2(v.x * inv_m2, -v.y * inv_m2) : v;
+      const float2 v = x[u * NT];
+      mine[u * RPT * S] = MODE == 3 ? make_float2(v.x * inv_m2, -v.y * inv_m2) : v;
     }
   } else {
     const int o_r = a.pos[2 * t], o_c = a.pos[2 * t + 1];
+    const ObjectColumn zc(a.object, a.n_rows, a.n_cols, o_r + row0 + tid / M, o_c + tid % M);
+    const float2* q = a.probe + row0 * M + tid;
 #pragma unroll (PER < 8 ? PER : 8)
-    for (int u = 0; u < PER; ++u) {
-      const int p = tid + u * NT, lr = p / M, c = p % M, r = row0 + lr;
-      sm[lr * S + c] = cmul(a.probe[r * M + c], gather_obj(a.object, a.n_rows, a.n_cols, o_r + r, o_c + c));
-    }
+    for (int u = 0; u < PER; ++u) mine[u * RPT * S] = cmul(q[u * NT], zc.at(u * RPT));
   }
   __syncthreads();
   gpass_a_fwd<M, H, S, 1, NT>(sm, tid);
@@ -1812,16 +1900,18 @@ __global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_grad
   {
     const float* amp = a.amp + (size_t)k * M * M + row0;
 #pragma unroll
-    for (int q = tid; q < M * H / 4; q += NT)
-      cp_async16(ampbuf + 4 * q, amp + (q / (H / 4)) * M + 4 * (q % (H / 4)));
+    for (int i = tid; i < M * H / 4; i += NT)
+      cp_async16(ampbuf + 4 * i, amp + (i / (H / 4)) * M + 4 * (i % (H / 4)));
     cp_async_commit();
   }
-  constexpr int UL = PER < 8 ? PER : 8;
+  // a thread's pixels: one column, RPT rows apart
+  constexpr int UL = PER < 8 ? PER : 8, RPT = NT / M;
+  static_assert(NT % M == 0, "a thread's pixels share one column");
+  const ObjectColumn zc(a.object, a.n_rows, a.n_cols, o_r + row0 + tid / M, o_c + tid % M);
+  const float2* q = a.probe + row0 * M + tid;
+  float2* mine = sm + (tid / M) * S + tid % M;
 #pragma unroll (UL)
-  for (int t = 0; t < PER; ++t) {
-    const int p = tid + t * NT, lr = p / M, c = p % M, r = row0 + lr;
-    sm[lr * S + c] = cmul(a.probe[r * M + c], gather_obj(a.object, a.n_rows, a.n_cols, o_r + r, o_c + c));
-  }
+  for (int t = 0; t < PER; ++t) mine[t * RPT * S] = cmul(q[t * NT], zc.at(t * RPT));
   __syncthreads();
   gpass_a_fwd<M, H, S, 1, NT>(sm, tid);
   cp_async_wait_all();  // a_k; the barriers below show it to the whole CTA
@@ -1869,8 +1959,8 @@ __global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_grad
   __syncthreads();
   gpass_a_inv<M, H, S, 1, NT>(sm, tid);
   __syncthreads();
-  float2* gz = a.gz + (size_t)kb * M * M;
-  float2* gq = a.gq + (size_t)kb * M * M;
+  float2* gz = a.gz + (size_t)kb * M * M + row0 * M + tid;
+  float2* gq = a.gq + (size_t)kb * M * M + row0 * M + tid;
   // patch gradients; the loads of UG pixels of a thread are issued together
   constexpr int UG = PER < 4 ? PER : 4;
 #pragma unroll 1
@@ -1878,16 +1968,14 @@ __global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_grad
     float2 qv[UG], zv[UG];
 #pragma unroll
     for (int u = 0; u < UG; ++u) {
-      const int p = tid + (t0 + u) * NT, r = row0 + p / M, c = p % M;
-      qv[u] = __ldg(a.probe + r * M + c);
-      zv[u] = gather_obj(a.object, a.n_rows, a.n_cols, o_r + r, o_c + c);
+      qv[u] = __ldg(q + (t0 + u) * NT);
+      zv[u] = zc.at((t0 + u) * RPT);
     }
 #pragma unroll
     for (int u = 0; u < UG; ++u) {
-      const int p = tid + (t0 + u) * NT, lr = p / M, c = p % M, r = row0 + lr;
-      const float2 e = csub(cmul(qv[u], zv[u]), sm[lr * S + c]);
-      gz[r * M + c] = cconjmul(qv[u], e);
-      gq[r * M + c] = cconjmul(zv[u], e);
+      const float2 e = csub(cmul(qv[u], zv[u]), mine[(t0 + u) * RPT * S]);
+      gz[(t0 + u) * NT] = cconjmul(qv[u], e);
+      gq[(t0 + u) * NT] = cconjmul(zv[u], e);
     }
   }
   if (rank == 0 && tid == 0) {
