@@ -2379,6 +2379,17 @@ cudaError_t upload_twiddles() {
   }
   cudaError_t e = cudaMemcpyToSymbol(c_twiddle, h, sizeof(h));
   if (e != cudaSuccess) return e;
+  float2 st[16 + 32 + 64 + 128];
+  auto fill = [&](int m, int n1, int n2) {
+    for (int j = 0; j < n1; ++j)
+      for (int k = 0; k < n2; ++k) st[m - 16 + j * n2 + k] = h[(j * k) % m * (256 / m)];
+  };
+  fill(16, FftPlan<16>::N1, FftPlan<16>::N2);
+  fill(32, FftPlan<32>::N1, FftPlan<32>::N2);
+  fill(64, FftPlan<64>::N1, FftPlan<64>::N2);
+  fill(128, FftPlan<128>::N1, FftPlan<128>::N2);
+  e = cudaMemcpyToSymbol(c_stage, st, sizeof(st));
+  if (e != cudaSuccess) return e;
   if ((e = set_cluster_attrs()) != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
   if (e != cudaSuccess) return e;
