@@ -1020,6 +1020,20 @@ __device__ __forceinline__ void tile_sync(cg::cluster_group& cl) {
     cl.sync();
 }
 
+// The same in two halves, so that register work between them hides the cluster
+// barrier's latency (one CTA: the barrier is cheap and the wait does it all).
+template <int C>
+__device__ __forceinline__ void tile_arrive(cg::cluster_group& cl) {
+  if constexpr (C > 1) cl.barrier_arrive();
+}
+template <int C>
+__device__ __forceinline__ void tile_wait(cg::cluster_group& cl) {
+  if constexpr (C == 1)
+    __syncthreads();
+  else
+    cl.barrier_wait();
+}
+
 // `buf` of CTA d of the cluster.
 template <int C, typename V>
 __device__ __forceinline__ V* tile_rank(cg::cluster_group& cl, int rank, V* buf, int d) {
@@ -1055,19 +1069,28 @@ __device__ __forceinline__ void row_pass_b_to_cols(cg::cluster_group& cl, int ra
       for (int i = 0; i < T::N1; ++i) dst[i * T::S] = v[t][i];
     }
   };
-#pragma unroll
-  for (int t = 0; t < T::SLOTS; ++t) {
+  auto get = [&](int t) {
     const int s = tid + t * T::NT;
     const float2* p = rowbuf + (s % T::H) * T::S + T::N1 * (s / T::H);
 #pragma unroll
     for (int i = 0; i < T::N1; ++i) v[t][i] = p[i];
-    Dft<T::N1, false>::run(v[t]);
-    if constexpr (!T::ONE) put(t);
-  }
+  };
   if constexpr (T::ONE) {
-    tile_sync<T::CTAS>(cl);
+#pragma unroll
+    for (int t = 0; t < T::SLOTS; ++t) get(t);
+    tile_arrive<T::CTAS>(cl);  // I have read my slab
+#pragma unroll
+    for (int t = 0; t < T::SLOTS; ++t) Dft<T::N1, false>::run(v[t]);
+    tile_wait<T::CTAS>(cl);
 #pragma unroll
     for (int t = 0; t < T::SLOTS; ++t) put(t);
+  } else {
+#pragma unroll
+    for (int t = 0; t < T::SLOTS; ++t) {
+      get(t);
+      Dft<T::N1, false>::run(v[t]);
+      put(t);
+    }
   }
 }
 
@@ -1082,10 +1105,11 @@ __device__ __forceinline__ void col_pass_a_inv_to_rows(cg::cluster_group& cl, in
   float2 v[T::N2];
 #pragma unroll
   for (int k2 = 0; k2 < T::N2; ++k2) v[k2] = p[T::N1 * k2];
+  if constexpr (T::ONE) tile_arrive<T::CTAS>(cl);  // I have read my slab
 #pragma unroll
   for (int k2 = 1; k2 < T::N2; ++k2) v[k2] = cmulc(v[k2], stage_twiddle<T::SIDE>(j, k2));
   Dft<T::N2, true>::run(v);
-  if constexpr (T::ONE) tile_sync<T::CTAS>(cl);
+  if constexpr (T::ONE) tile_wait<T::CTAS>(cl);
 #pragma unroll
   for (int n2 = 0; n2 < T::N2; ++n2) {
     const int d = T::N1 * n2 / T::H, lr = T::N1 * n2 % T::H + j;
@@ -1593,8 +1617,10 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
           }
         }
         if (ONE) load_up();
-        if (halo) tile_sync<C>(cl);  // the pushed halo rows of level 2 are in place
-        __syncthreads();
+        if (halo)
+          tile_sync<C>(cl);  // the pushed halo rows of level 2 are in place
+        else
+          __syncthreads();
         {  // back up to level 1
           const CoarseCell cell(Z2, S2, W2, i1, j1);
           float2* zw = Z1 + i1 * S1 + j1;
@@ -1612,11 +1638,10 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
         general_levels();
       }
     }
-    if (halo) {
-      tile_sync<C>(cl);
-      if (a.levels > 2 && !l3) fill_halo(Z1, 1);  // two and three levels: the halo rows were pushed
-    }
-    __syncthreads();
+    if (halo) tile_sync<C>(cl);
+    const bool pushed = a.levels == 2 || l3;  // the halo rows of level 1 are in place
+    if (halo && !pushed) fill_halo(Z1, 1);
+    if (!halo || !pushed) __syncthreads();
   }
 
   // a5 (finest level) + a6 + a7; the level-0 gain G_0 = conj(Q)/(u_0 + |Q|^2)
