@@ -488,7 +488,11 @@ emg_status enqueue_minibatch(emg_ctx* c, const int32_t* d_idx, int b, double* d_
   }
   // The probe prep runs inside the cluster step launch (FFT path) when the
   // launch fits in one wave of resident clusters: there it overlaps the gather
-  // and transforms.  Otherwise it is its own kernel before the step.
+  // and transforms.  Otherwise it is its own kernel before the step.  With
+  // large probes and several levels it stays ahead over a few waves too (us per
+  // minibatch, separate against fused: m = 128, 128 positions 55.1 / 50.5, 256
+  // 94.1 / 91.7; m = 256, 64 positions 116.7 / 111.6, 128 217.4 / 214.6, but
+  // 256 positions, seven waves, 393.6 / 397.1).
   PrepArgs pf = pa;
   int fused_tiles = (c->fuse_prep && !c->tc && c->cluster >= 1) ? emg::fused_prep_tiles(pf, c->m, c->cluster) : 0;
   if (fused_tiles > 0) {
@@ -497,7 +501,8 @@ emg_status enqueue_minibatch(emg_ctx* c, const int32_t* d_idx, int b, double* d_
       c->resident_clusters = emg::step_resident_clusters(c->m, c->cluster);
       c->resident_cluster = c->cluster;
     }
-    if (nb + prep_clusters > c->resident_clusters || nb == 0) fused_tiles = 0;
+    const int waves = c->m >= 128 && c->par.levels > 1 ? 4 : 1;
+    if (nb + prep_clusters > waves * c->resident_clusters || nb == 0) fused_tiles = 0;
   }
   if (fused_tiles == 0) {
     {
