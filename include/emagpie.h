@@ -208,9 +208,8 @@ emg_status emg_run_epochs(emg_ctx* ctx, int32_t n_epochs, const int32_t* order,
  *   grad_Q Phi = sum_k conj(P_k z) (Q . P_k z - R_k),
  * in the convention d/dRe + i d/dIm (twice the conjugate Wirtinger derivative,
  * the convention PyTorch uses for complex autograd).  R_k is recomputed (no
- * exit waves are stored); positions are processed in chunks (by default a
- * multiple of the position clusters that can be resident at once, about 128
- * positions; see emg_set_gradient_chunk) and summed in a fixed order, so
+ * exit waves are stored); positions are processed in chunks (see
+ * emg_set_gradient_chunk) and summed in a fixed order, so
  * results repeat bitwise for a given chunk size.  The first call may allocate
  * the chunk's patch buffers.
  *  object, probe            device complex64 [n_rows][n_cols], [m][m] (read only)
@@ -221,9 +220,9 @@ emg_status emg_misfit_gradient(emg_ctx* ctx, const float* object, const float* p
                                float* grad_object, float* grad_probe, double* misfit);
 
 /*
- * Positions per launch of emg_misfit_gradient: 0 (the default) chooses a
- * multiple of the position clusters that can be resident at once, about 128
- * positions; n > 0 takes n.  The chunk only
+ * Positions per launch of emg_misfit_gradient: 0 (the default) chooses equal
+ * chunks of whole waves of the position clusters that can be resident at once,
+ * with at most about 160 MB of patch gradients; n > 0 takes n.  The chunk only
  * changes speed and the rounding order of the sums.  Synchronises the
  * context's stream and frees the previous chunk's buffers.  EMG_EINVAL for
  * n < 0.

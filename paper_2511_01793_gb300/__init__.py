@@ -386,7 +386,7 @@ def emg_misfit_gradient(ctx: int, object_ptr: int, probe_ptr: int, grad_object_p
 
 
 def emg_set_gradient_chunk(ctx: int, positions: int) -> None:
-    """Positions per gradient launch (0, the default: a multiple of the resident position clusters)."""
+    """Positions per gradient launch (0, the default: equal chunks of whole waves of clusters)."""
     _check(load().emg_set_gradient_chunk(ctx, positions), "emg_set_gradient_chunk", ctx)
 
 

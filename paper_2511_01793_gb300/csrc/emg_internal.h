@@ -134,26 +134,29 @@ struct GradArgs {
   const float2* probe;
   const int32_t* pos;
   const float* amp;
-  int first, n_rows, n_cols;    // positions first .. first + b - 1
+  int first, b, n_rows, n_cols; // positions first .. first + b - 1
   float2* gz;                   // [b][m][m]
-  float2* gq;                   // [b][m][m]
+  float2* gq;                   // [slots][m][m] sums over the positions of each slot
   double* phi;                  // [b]
 };
 
 // Sums the patch gradients of one chunk into the object / probe gradients.
 struct GradReduceArgs {
   const int32_t* pos;
-  int first, b, n_rows, n_cols, m, accumulate;
+  int first, b, slots, n_rows, n_cols, m, accumulate;
   const float2* gz;
   const float2* gq;
   float2* grad_object;          // [n_rows][n_cols] or null
   float2* grad_probe;           // [m][m] or null
-  int tiles_x, tiles_y;
+  int tiles_x, tiles_y;         // set by launch_grad_reduce
 };
 
-cudaError_t launch_gradient(int m, int b, const GradArgs& a, cudaStream_t s);
+// `slots` <= a.b clusters, each with its own probe-gradient sum.
+cudaError_t launch_gradient(int m, int slots, const GradArgs& a, cudaStream_t s);
 // Positions whose gradient clusters are resident on the device at once (0 if unknown).
 int gradient_positions_per_wave(int m);
+// Clusters (and probe-gradient slots) of a launch over `chunk` positions, `wave` of them resident at once.
+int gradient_slots(int m, int wave, int chunk);
 cudaError_t launch_grad_reduce(const GradReduceArgs& a, cudaStream_t s);
 bool step_supported(int m, int levels, int cluster);
 int default_cluster(int m, int levels);
@@ -163,7 +166,7 @@ cudaError_t launch_batch_orders(const int32_t* const* src, int32_t* const* dst, 
 cudaError_t launch_epoch_advance(int* epoch, cudaStream_t s);
 
 // Combine object tiles: kApplyTile rows x kApplyTileW columns, kApplyPx pixels
-// per thread (the gradient sums use kApplyTile^2 tiles, one pixel per thread).
+// per thread.
 #ifndef EMG_APPLY_PX
 #define EMG_APPLY_PX 2
 #endif

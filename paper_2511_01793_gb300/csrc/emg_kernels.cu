@@ -1907,6 +1907,14 @@ __global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_forw
 // then gz = conj(Q) (psi - R), gq = conj(z_k) (psi - R) on the patch.
 // One slab per CTA, a_k by cp.async beside it, z_k read again from L2 at the
 // end: 32 warps per SM (as for the forward kernels and the step at m = 256).
+// Cluster i takes positions i, i + grid, ... of the chunk, adds their probe
+// gradients up in its own slot and fetches the next position's a_k while it
+// finishes the current one.  With one CTA per position the grid is one wave
+// (one L2-resident probe gradient per CTA instead of one per position to write
+// and read back); clusters of 8 are launched one per position, since the
+// hardware then fills each SM as it frees up (1600 positions at m = 256: 1.65
+// ms, one wave 1.75).  us per call before -> after, with the sums: 900 positions
+// at m = 128 244 -> 173, 1444 at m = 64 125 -> 68, 4096 at m = 32 133 -> 64.
 template <int M>
 __global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_gradc(const GradArgs a) {
   using TL = WaveTile<M>;
@@ -1918,17 +1926,20 @@ __global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_grad
   __shared__ double xd[C];
   __shared__ float redf[(NT + 31) / 32];
   const int tid = threadIdx.x;
-  const int kb = blockIdx.x / C;
-  const int k = a.first + kb;
-  const int o_r = a.pos[2 * k], o_c = a.pos[2 * k + 1];
+  const int slot = blockIdx.x / C, slots = gridDim.x / C;
   const int row0 = rank * H;
-  {
-    const float* amp = a.amp + (size_t)k * M * M + row0;
+  auto fetch_amp = [&](int kb) {
+    const float* amp = a.amp + (size_t)(a.first + kb) * M * M + row0;
 #pragma unroll
     for (int i = tid; i < M * H / 4; i += NT)
       cp_async16(ampbuf + 4 * i, amp + (i / (H / 4)) * M + 4 * (i % (H / 4)));
     cp_async_commit();
-  }
+  };
+  fetch_amp(slot);
+  pdl_trigger();
+  for (int kb = slot; kb < a.b; kb += slots) {
+  const int k = a.first + kb;
+  const int o_r = a.pos[2 * k], o_c = a.pos[2 * k + 1];
   // a thread's pixels: one column, RPT rows apart
   constexpr int UL = PER < 8 ? PER : 8, RPT = NT / M;
   static_assert(NT % M == 0, "a thread's pixels share one column");
@@ -1980,12 +1991,14 @@ __global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_grad
   if (tid == 0) *tile_rank<C>(cl, rank, &xd[rank], 0) = partials_sum<NT>(redf);
   col_pass_a_inv_to_rows<TL>(cl, rank, sm, sm, tid);
   tile_sync<C>(cl);
+  if (kb + slots < a.b) fetch_amp(kb + slots);  // ampbuf has been read
   gpass_b<M, H, S, 1, NT, true>(sm, tid);
   __syncthreads();
   gpass_a_inv<M, H, S, 1, NT>(sm, tid);
   __syncthreads();
   float2* gz = a.gz + (size_t)kb * M * M + row0 * M + tid;
-  float2* gq = a.gq + (size_t)kb * M * M + row0 * M + tid;
+  float2* gq = a.gq + (size_t)slot * M * M + row0 * M + tid;
+  const bool more = k != slot;  // this slot holds a sum already (of this launch or an earlier chunk's)
   // patch gradients; the loads of UG pixels of a thread are issued together
   constexpr int UG = PER < 4 ? PER : 4;
 #pragma unroll 1
@@ -2000,7 +2013,11 @@ __global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_grad
     for (int u = 0; u < UG; ++u) {
       const float2 e = csub(cmul(qv[u], zv[u]), mine[(t0 + u) * RPT * S]);
       gz[(t0 + u) * NT] = cconjmul(qv[u], e);
-      gq[(t0 + u) * NT] = cconjmul(zv[u], e);
+      // one thread adds to each address, so the order of the sum is fixed
+      if (more)
+        atomicAdd(gq + (t0 + u) * NT, cconjmul(zv[u], e));
+      else
+        gq[(t0 + u) * NT] = cconjmul(zv[u], e);
     }
   }
   if (rank == 0 && tid == 0) {
@@ -2009,80 +2026,124 @@ __global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_grad
     for (int d = 0; d < C; ++d) tot += xd[d];
     a.phi[kb] = tot * (0.5 / (double)(M * M));
   }
+  __syncthreads();  // the slab has been read before the next position's gather
+  }
 }
 
-// Object gradient sum_k P_k^T gz_k over 16 x 16 tiles and probe gradient
-// sum_k gq_k, each in position order (deterministic); optionally added to the
-// existing values (later chunks of positions).
+// Object gradient sum_k P_k^T gz_k over tiles of 16 x 32 pixels (optionally
+// added to the existing values: later chunks of positions) and probe gradient
+// sum of the slots' gq, each in a fixed order (deterministic).  Bound by
+// the loads: a thread keeps those of four patches at two pixels in flight, and
+// the positions that overlap a tile are listed kGradList at a time, so any number
+// of positions takes the same shared memory.
+constexpr int kGradList = 512, kGradTileW = 32;
 __global__ void __launch_bounds__(kApplyThreads) k_grad_reduce(const GradReduceArgs a) {
-  extern __shared__ int glist[];
-  __shared__ int warp_count[kApplyThreads / 32];
-  __shared__ int total;
-  __shared__ float2 part_s[kApplyProbeGroups][32];
-  const int tid = threadIdx.x;
+  constexpr int WARPS = kApplyThreads / 32, PW = kGradList / WARPS, ROUNDS = PW / 32, PP = kApplyProbePx / 32;
+  static_assert(WARPS == kApplyProbeGroups && 2 * WARPS == kApplyTile, "two tile rows per warp");
+  __shared__ int3 list[kGradList];
+  __shared__ int count[WARPS];
+  __shared__ float2 part_s[kApplyProbeGroups][kApplyProbePx];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n_tiles = a.tiles_x * a.tiles_y;
   const int m = a.m;
   const size_t mm = (size_t)m * m;
+  pdl_trigger();
   if ((int)blockIdx.x < n_tiles) {
     if (!a.grad_object) return;
-    const int ty = blockIdx.x / a.tiles_x, tx = blockIdx.x % a.tiles_x;
-    const int r0 = ty * kApplyTile, c0 = tx * kApplyTile;
-    if (tid == 0) total = 0;
-    __syncthreads();
-    for (int base = 0; base < a.b; base += kApplyThreads) {
-      const int kb = base + tid;
-      int pr = 0, pc = 0;
-      bool hit = false;
-      if (kb < a.b) {
-        pr = a.pos[2 * (a.first + kb)];
-        pc = a.pos[2 * (a.first + kb) + 1];
-        hit = pr < r0 + kApplyTile && pr + m > r0 && pc < c0 + kApplyTile && pc + m > c0;
+    const int r0 = (int)(blockIdx.x / a.tiles_x) * kApplyTile, c0 = (int)(blockIdx.x % a.tiles_x) * kGradTileW;
+    bool waited = false;
+    const int row = r0 + warp, col = c0 + lane;  // pixels (row, col) and (row + WARPS, col)
+    float2 g[2] = {czero(), czero()};
+    for (int k0 = 0; k0 < a.b; k0 += kGradList) {
+      // ordered compaction: warp w lists the w-th run of these positions
+      int3 p[ROUNDS];
+      unsigned mask[ROUNDS];
+      int mine = 0;
+#pragma unroll
+      for (int i = 0; i < ROUNDS; ++i) {
+        const int kb = k0 + warp * PW + i * 32 + lane;
+        bool hit = false;
+        if (kb < a.b) {
+          p[i] = make_int3(kb, a.pos[2 * (a.first + kb)], a.pos[2 * (a.first + kb) + 1]);
+          hit = p[i].y < r0 + kApplyTile && p[i].y + m > r0 && p[i].z < c0 + kGradTileW && p[i].z + m > c0;
+        }
+        mask[i] = __ballot_sync(0xffffffffu, hit);
+        mine += __popc(mask[i]);
       }
-      const unsigned mask = __ballot_sync(0xffffffffu, hit);
-      const int lane = tid & 31, warp = tid >> 5;
-      if (lane == 0) warp_count[warp] = __popc(mask);
+      __syncthreads();  // the previous list has been walked
+      if (lane == 0) count[warp] = mine;
       __syncthreads();
-      int off = total;
-      for (int w = 0; w < warp; ++w) off += warp_count[w];
-      if (hit) {
-        const int slot = off + __popc(mask & ((1u << lane) - 1u));
-        glist[3 * slot] = kb;
-        glist[3 * slot + 1] = pr;
-        glist[3 * slot + 2] = pc;
+      int at = 0, total = 0;
+#pragma unroll
+      for (int w = 0; w < WARPS; ++w) {
+        if (w < warp) at += count[w];
+        total += count[w];
+      }
+#pragma unroll
+      for (int i = 0; i < ROUNDS; ++i) {
+        if (mask[i] >> lane & 1u) list[at + __popc(mask[i] & ((1u << lane) - 1u))] = p[i];
+        at += __popc(mask[i]);
       }
       __syncthreads();
-      if (tid == 0) {
-        int t = total;
-        for (int w = 0; w < kApplyThreads / 32; ++w) t += warp_count[w];
-        total = t;
+      if (!waited) pdl_wait();  // the patch gradients; the first list needs the positions alone
+      waited = true;
+      for (int t0 = 0; t0 < total; t0 += 4) {
+        float2 v[4][2];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          v[u][0] = v[u][1] = czero();
+          if (t0 + u < total) {
+            const int3 q = list[t0 + u];
+            const int lr = row - q.y, lc = col - q.z;
+            const float2* src = a.gz + (size_t)q.x * mm + lr * m + lc;
+            const bool in_c = (unsigned)lc < (unsigned)m;
+            if (in_c && (unsigned)lr < (unsigned)m) v[u][0] = src[0];
+            if (in_c && (unsigned)(lr + WARPS) < (unsigned)m) v[u][1] = src[WARPS * m];
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) g[h] = cadd(g[h], v[u][h]);
       }
-      __syncthreads();
     }
-    const int cnt = total;
-    const int row = r0 + tid / kApplyTile, col = c0 + tid % kApplyTile;
-    if (row >= a.n_rows || col >= a.n_cols) return;
-    float2 g = czero();
-    for (int t = 0; t < cnt; ++t) {
-      const int lr = row - glist[3 * t + 1], lc = col - glist[3 * t + 2];
-      if ((unsigned)lr < (unsigned)m && (unsigned)lc < (unsigned)m)
-        g = cadd(g, a.gz[(size_t)glist[3 * t] * mm + lr * m + lc]);
+    if (col >= a.n_cols) return;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (row + h * WARPS >= a.n_rows) continue;
+      const size_t gi = (size_t)(row + h * WARPS) * a.n_cols + col;
+      a.grad_object[gi] = a.accumulate ? cadd(a.grad_object[gi], g[h]) : g[h];
     }
-    const size_t gi = (size_t)row * a.n_cols + col;
-    a.grad_object[gi] = a.accumulate ? cadd(a.grad_object[gi], g) : g;
   } else {
     if (!a.grad_probe) return;
-    const int lane = tid & 31, g = tid >> 5;
-    const int p = (blockIdx.x - n_tiles) * 32 + lane;
-    float2 sum = czero();
-    if (p < (int)mm)
-      for (int kb = g; kb < a.b; kb += kApplyProbeGroups) sum = cadd(sum, a.gq[(size_t)kb * mm + p]);
-    part_s[g][lane] = sum;
-    __syncthreads();
-    if (g != 0 || p >= (int)mm) return;
-    float2 tot = part_s[0][lane];
+    pdl_wait();
+    const int p0 = (blockIdx.x - n_tiles) * kApplyProbePx + lane;  // pixels p0 + 32 h; warp w sums slots w, w + 8, ...
+    float2 s[PP];
 #pragma unroll
-    for (int i = 1; i < kApplyProbeGroups; ++i) tot = cadd(tot, part_s[i][lane]);
-    a.grad_probe[p] = a.accumulate ? cadd(a.grad_probe[p], tot) : tot;
+    for (int h = 0; h < PP; ++h) s[h] = czero();
+    for (int k0 = warp; k0 < a.slots; k0 += 4 * kApplyProbeGroups) {
+      float2 v[4][PP];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int h = 0; h < PP; ++h) {
+          const int k = k0 + u * kApplyProbeGroups;
+          v[u][h] = k < a.slots && p0 + 32 * h < (int)mm ? a.gq[(size_t)k * mm + p0 + 32 * h] : czero();
+        }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int h = 0; h < PP; ++h) s[h] = cadd(s[h], v[u][h]);
+    }
+#pragma unroll
+    for (int h = 0; h < PP; ++h) part_s[warp][lane + 32 * h] = s[h];
+    __syncthreads();
+    const int p = (blockIdx.x - n_tiles) * kApplyProbePx + tid;
+    if (tid >= kApplyProbePx || p >= (int)mm) return;
+    float2 tot = part_s[0][tid];
+#pragma unroll
+    for (int i = 1; i < kApplyProbeGroups; ++i) tot = cadd(tot, part_s[i][tid]);
+    a.grad_probe[p] = tot;
   }
 }
 
@@ -2635,16 +2696,12 @@ constexpr size_t gradc_smem_elems() {
 }
 
 template <int M>
-cudaError_t launch_gradc_t(int b, const GradArgs& a, cudaStream_t s) {
+cudaError_t launch_gradc_t(int slots, const GradArgs& a, cudaStream_t s) {
   using TL = WaveTile<M>;
   constexpr size_t bytes = gradc_smem_elems<M>() * sizeof(float2);
-  if constexpr (TL::CTAS == 1) {
-    k_gradc<M><<<b, TL::NT, bytes, s>>>(a);
-  } else {
-    cudaError_t e = launch_cluster_plain(k_gradc<M>, TL::CTAS, dim3(TL::CTAS * b), dim3(TL::NT), bytes, s, a);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaGetLastError();
+  const cudaError_t e =
+      launch_cluster_plain(k_gradc<M>, TL::CTAS, dim3(TL::CTAS * slots), dim3(TL::NT), bytes, s, a);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename Kernel>
@@ -2698,9 +2755,6 @@ cudaError_t set_cluster_attrs() {
   if ((e = set_grad_attrs<64>()) != cudaSuccess) return e;
   if ((e = set_grad_attrs<128>()) != cudaSuccess) return e;
   if ((e = set_grad_attrs<256>()) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(k_grad_reduce, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024)) !=
-      cudaSuccess)
-    return e;
   return cudaSuccess;
 }
 
@@ -2864,6 +2918,8 @@ int gradient_wave_t() {
   return n;
 }
 
+int gradient_slots(int m, int wave, int chunk) { return m <= 128 && wave > 0 && wave < chunk ? wave : chunk; }
+
 int gradient_positions_per_wave(int m) {
   switch (m) {
     case 16: return gradient_wave_t<16>();
@@ -2875,22 +2931,24 @@ int gradient_positions_per_wave(int m) {
   }
 }
 
-cudaError_t launch_gradient(int m, int b, const GradArgs& a, cudaStream_t s) {
+cudaError_t launch_gradient(int m, int slots, const GradArgs& a, cudaStream_t s) {
   switch (m) {
-    case 16: return launch_gradc_t<16>(b, a, s);
-    case 32: return launch_gradc_t<32>(b, a, s);
-    case 64: return launch_gradc_t<64>(b, a, s);
-    case 128: return launch_gradc_t<128>(b, a, s);
-    case 256: return launch_gradc_t<256>(b, a, s);
+    case 16: return launch_gradc_t<16>(slots, a, s);
+    case 32: return launch_gradc_t<32>(slots, a, s);
+    case 64: return launch_gradc_t<64>(slots, a, s);
+    case 128: return launch_gradc_t<128>(slots, a, s);
+    case 256: return launch_gradc_t<256>(slots, a, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
 cudaError_t launch_grad_reduce(const GradReduceArgs& a, cudaStream_t s) {
-  const int n_tiles = a.tiles_x * a.tiles_y;
-  const int n_probe = (a.m * a.m + 31) / 32;
-  k_grad_reduce<<<n_tiles + n_probe, kApplyThreads, (size_t)a.b * 3 * sizeof(int), s>>>(a);
-  return cudaGetLastError();
+  GradReduceArgs t = a;
+  t.tiles_x = (a.n_cols + kGradTileW - 1) / kGradTileW;
+  t.tiles_y = (a.n_rows + kApplyTile - 1) / kApplyTile;
+  const int n_probe = (a.m * a.m + kApplyProbePx - 1) / kApplyProbePx;
+  const cudaError_t e = launch_pdl(k_grad_reduce, dim3(t.tiles_x * t.tiles_y + n_probe), dim3(kApplyThreads), 0, s, t);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // Whether the step kernel for probe side m with `cluster` CTAs per position

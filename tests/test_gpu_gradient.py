@@ -146,3 +146,44 @@ def test_full_size_gradient_workload(lib, torch):
     assert abs(phi - phi_o) <= 1e-5 * phi_o
     assert rel_err(gz, gz_o) <= 1e-5
     assert rel_err(gq, gq_o) <= 1e-5
+
+
+@pytest.mark.parametrize("m,n_pos,chunk", [(16, 2500, 0), (32, 1300, 1300), (64, 330, 7), (128, 160, 0), (256, 45, 20)])
+def test_gradients_of_many_positions_by_every_split(lib, torch, m, n_pos, chunk):
+    """More positions than clusters (each cluster then sums several probe gradients), several chunks,
+    position lists longer than one pass of the sums, and either gradient alone: the gradients equal a
+    plain FP64 evaluation to 1e-5, and the parts asked for alone equal the joint call bitwise."""
+    rng = np.random.default_rng(m)
+    n_rows, n_cols = m + 37, m + 50
+    pos = np.stack([rng.integers(-m // 3, 50, n_pos), rng.integers(-m // 3, 60, n_pos)], 1).astype(np.int32)
+    z = (rng.standard_normal((n_rows, n_cols)) + 1j * rng.standard_normal((n_rows, n_cols))).astype(np.complex64)
+    q = (rng.standard_normal((m, m)) + 1j * rng.standard_normal((m, m))).astype(np.complex64)
+    d = (rng.uniform(0.5, 2.0, size=(n_pos, m, m)) * 2 * m * m).astype(np.float32)
+    c = lib.Context(pos, d, n_rows, n_cols, lib.emg_default_params(minibatch=4), obj=torch.from_numpy(z),
+                    probe=torch.from_numpy(q))
+    lib.emg_set_gradient_chunk(c.ctx, chunk)
+
+    def call(obj, probe):
+        g = torch.zeros_like(c.obj), torch.zeros_like(c.probe)
+        phi = lib.emg_misfit_gradient(c.ctx, c.obj.data_ptr(), c.probe.data_ptr(), g[0].data_ptr() if obj else 0,
+                                      g[1].data_ptr() if probe else 0)
+        return phi, g[0].cpu().numpy(), g[1].cpu().numpy()
+
+    phi, gz, gq = call(True, True)
+    assert np.array_equal(call(True, False)[1], gz) and np.array_equal(call(False, True)[2], gq)
+    z64, q64, a64 = z.astype(np.complex128), q.astype(np.complex128), np.sqrt(d.astype(np.float64))
+    rz, rq, want = np.zeros_like(z64), np.zeros_like(q64), 0.0
+    for k in range(n_pos):
+        r0, c0 = pos[k]
+        rows, cols = slice(max(r0, 0), min(r0 + m, n_rows)), slice(max(c0, 0), min(c0 + m, n_cols))
+        zk = np.zeros((m, m), dtype=np.complex128)
+        part = slice(rows.start - r0, rows.stop - r0), slice(cols.start - c0, cols.stop - c0)
+        zk[part] = z64[rows, cols]
+        f = np.fft.fft2(q64 * zk)
+        want += 0.5 * np.sum((np.abs(f) - a64[k]) ** 2) / m ** 2
+        e = q64 * zk - np.fft.ifft2(a64[k] * f / np.abs(f))
+        rz[rows, cols] += (np.conj(q64) * e)[part]
+        rq += np.conj(zk) * e
+    assert abs(phi - want) <= 1e-5 * want
+    assert np.linalg.norm(gz - rz) <= 1e-5 * np.linalg.norm(rz) and np.linalg.norm(gq - rq) <= 1e-5 * np.linalg.norm(rq)
+    c.close()

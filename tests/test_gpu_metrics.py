@@ -94,3 +94,25 @@ def test_aligned_errors_are_zero_for_a_scaled_truth(lib):
                                  torch.cuda.current_stream().cuda_stream)
     assert abs(got["c"] * complex(c) - 1) < 1e-6
     assert got["object"] < 1e-6 and got["probe"] < 1e-6 and got["phase_rms"] < 1e-6
+
+
+@pytest.mark.parametrize("n_rows,n_cols,m,n_pos", [(37, 45, 16, 700), (8, 32, 5, 3), (129, 33, 64, 1025), (200, 260, 32, 512)])
+def test_illuminated_region_on_odd_tiles_and_long_lists(lib, n_rows, n_cols, m, n_pos):
+    """Tiles cut by the object's edge, more positions than one pass lists, patches partly or wholly
+    outside: the mask equals a sequential FP64 sum (bitwise the same order, so the same threshold)."""
+    import torch
+
+    rng = np.random.default_rng(n_pos)
+    q = (rng.standard_normal((m, m)) + 1j * rng.standard_normal((m, m))).astype(np.complex64)
+    pos = np.stack([rng.integers(-m, n_rows + 3, n_pos), rng.integers(-m, n_cols + 3, n_pos)], 1).astype(np.int32)
+    p2 = q.real.astype(np.float64) ** 2 + q.imag.astype(np.float64) ** 2
+    illum = np.zeros((n_rows, n_cols))
+    for r0, c0 in pos:
+        rs, re_, cs, ce = max(r0, 0), min(r0 + m, n_rows), max(c0, 0), min(c0 + m, n_cols)
+        if re_ > rs and ce > cs:
+            illum[rs:re_, cs:ce] += p2[rs - r0:re_ - r0, cs - c0:ce - c0]
+    qt, pt = torch.from_numpy(q).cuda(), torch.from_numpy(pos).cuda()
+    for frac in (0.0, 0.3, 1.0):
+        region = torch.full((n_rows, n_cols), 7, dtype=torch.uint8, device="cuda")
+        lib.emg_illuminated_region(qt.data_ptr(), m, pt.data_ptr(), n_pos, n_rows, n_cols, frac, region.data_ptr())
+        assert np.array_equal(region.cpu().numpy(), (illum >= frac * illum.max()).astype(np.uint8))
