@@ -154,12 +154,19 @@ __device__ __forceinline__ float2 cfma_conj(float2 a, float2 b, float2 c) {
 // A floor of 1e-37 under both square roots gives y = 0 for w = 0 without a
 // branch; it changes no result for |w|^2 above about 1e-29.  The sign flip
 // is applied to the sign bit when Re(y conj(x)) < 0.
+// REFINED: both roots take one Newton step, which brings their error from the
+// rsqrt unit's down to the FP32 rounding of a correctly rounded root's.
+template <bool REFINED>
 __device__ __forceinline__ float2 geomean_aligned_root(float2 x, float2 xp) {
   const float2 w = cmul(x, xp);
   const float n = fmaf(w.x, w.x, w.y * w.y);
-  const float mag = n * rsqrtf(n + 1e-37f);
+  const float r = rsqrtf(n + 1e-37f);
+  float mag = n * r;
+  if constexpr (REFINED) mag = fmaf(fmaf(-mag, mag, n), 0.5f * r, mag);
   const float s2 = fabsf(w.x) + mag;
-  const float rr = rsqrtf(s2 + 1e-37f) * 0.70710678118654752f;
+  float q = rsqrtf(s2 + 1e-37f);
+  if constexpr (REFINED) q = fmaf(fmaf(-(s2 * q), q, 1.f), 0.5f * q, q);
+  const float rr = q * 0.70710678118654752f;
   const float t = s2 * rr, vh = w.y * rr;
   const float yx = w.x >= 0.f ? t : vh, yy = w.x >= 0.f ? vh : t;
   const unsigned sbit = fmaf(yx, x.x, yy * x.y) < 0.f ? 0x80000000u : 0u;
@@ -170,7 +177,7 @@ __device__ __forceinline__ float2 geomean_aligned_root(float2 x, float2 xp) {
 // the prolonged coarse correction pro, z^+ = zp + G_0 (R - Q zp) with
 // zp = z_k + pro, else z^+ = z_k + G_0 (R - Q z_k); Q^+ = Q + conj(z_k)(R - Q z_k)/mu_k;
 // with JOINT their aligned geometric means with z_k and Q (Eq. geomean).
-template <bool MG, bool JOINT>
+template <bool MG, bool JOINT, bool REFINED>
 __device__ __forceinline__ void update_pixel(float2 zk, float2 q, float2 g0, float2 R, float2 pro, float inv_mu,
                                              float2& zn, float2& qn) {
   const float2 res = cfnma(q, zk, R);
@@ -183,8 +190,8 @@ __device__ __forceinline__ void update_pixel(float2 zk, float2 q, float2 g0, flo
   }
   const float2 qplus = cfma_conj(zk, cscale(res, inv_mu), q);
   if constexpr (JOINT) {
-    zn = geomean_aligned_root(zk, zplus);
-    qn = geomean_aligned_root(q, qplus);
+    zn = geomean_aligned_root<REFINED>(zk, zplus);
+    qn = geomean_aligned_root<REFINED>(q, qplus);
   } else {
     zn = zplus;
     qn = qplus;
@@ -1666,6 +1673,9 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   const bool pairs = UGP > 0 && !a.s_num && !a.verify && slot_ok &&
                      ((reinterpret_cast<uintptr_t>(a.probe) | reinterpret_cast<uintptr_t>(G0) |
                        reinterpret_cast<uintptr_t>(zt) | reinterpret_cast<uintptr_t>(qt)) & 15) == 0;
+  // Small probes keep the accuracy of correctly rounded roots (their arithmetic before they
+  // came to this kernel) at the cost of a few dependent operations.
+  constexpr bool kRefined = M <= 32;
   auto update_pairs = [&](auto multigrid, auto joint) {
     constexpr bool kMg = decltype(multigrid)::value, kJoint = decltype(joint)::value;
     constexpr int PP = PER / 2, RP = 2 * RPT;
@@ -1709,7 +1719,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
           const float2 zk = h ? make_float2(zk2.z, zk2.w) : make_float2(zk2.x, zk2.y);
           const float2 q = h ? make_float2(qv[u].z, qv[u].w) : make_float2(qv[u].x, qv[u].y);
           const float2 g0 = h ? make_float2(gv[u].z, gv[u].w) : make_float2(gv[u].x, gv[u].y);
-          update_pixel<kMg, kJoint>(zk, q, g0, rb[t * RP * SR + h], pro[h], inv_mu, zo[h], qo[h]);
+          update_pixel<kMg, kJoint, kRefined>(zk, q, g0, rb[t * RP * SR + h], pro[h], inv_mu, zo[h], qo[h]);
         }
         const int off = off0 + 2 * t * NT;
         *reinterpret_cast<float4*>(zt + off) = make_float4(zo[0].x, zo[0].y, zo[1].x, zo[1].y);
@@ -1756,14 +1766,14 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
     float2 zn, qn;
     if (a.levels == 1) {
       if (a.joint)
-        update_pixel<false, true>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
+        update_pixel<false, true, kRefined>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
       else
-        update_pixel<false, false>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
+        update_pixel<false, false, kRefined>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
     } else {
       if (a.joint)
-        update_pixel<true, true>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
+        update_pixel<true, true, kRefined>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
       else
-        update_pixel<true, false>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
+        update_pixel<true, false, kRefined>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
     }
     if (a.s_num)
       scatter_atomic(a.s_num, a.s_den, a.combine, a.n_rows, a.n_cols, o_r + r, o_c + c, zn, zk, fmaf(a.w_eps, MQ, cabs2(q)));
