@@ -486,6 +486,17 @@ __device__ __forceinline__ void umma_bf16_n(uint32_t tmem_d, uint64_t adesc, uin
       : "memory");
 }
 
+// True in one thread of a converged warp (the same one at every call).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.b32 %0, 1, 0, p;\n\t}"
+      : "=r"(e));
+  return e != 0;
+}
+
 // 16 consecutive FP32 columns of the warp's 32 TMEM lanes; completes with tmem_ld_wait.
 __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
@@ -615,78 +626,86 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      bool ok = mbar_wait(&b_bar, 0, &abort_sh);
-      uint32_t it = 0;
-      int local = 0;
-      for (int blk = blockIdx.x; ok && blk < n_blocks; blk += gridDim.x, ++local) {
-        if (local > 0 && !mbar_wait(&acce_bar, (local - 1) & 1, &abort_sh)) {
+    // The whole warp runs the loop and an elected thread issues, so that the
+    // descriptors are computed in uniform registers, where the MMA takes them.
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      return __all_sync(0xffffffffu, mbar_wait(bar, parity, &abort_sh)) != 0;
+    };
+    bool ok = wait(&b_bar, 0);
+    uint32_t it = 0;
+    int local = 0;
+    for (int blk = blockIdx.x; ok && blk < n_blocks; blk += gridDim.x, ++local) {
+      if (local > 0 && !wait(&acce_bar, (local - 1) & 1)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      // stage 1: for each n2, a 16-point DFT of the 128 rows' n1 elements;
+      // half h of the k1 range lands in columns h * 256 + n2 * 16
+#pragma unroll 1
+      for (int n2 = 0; n2 < 16; ++n2) {
+        const bool staged = r16_staged(n2);
+        const uint32_t s = it % kR16Stages;
+        if (!wait(staged ? &x_bar[n2 - kR16XFirst] : &full_bar[s],
+                  staged ? (uint32_t)(local & 1) : (it / kR16Stages) & 1)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        // stage 1: for each n2, a 16-point DFT of the 128 rows' n1 elements;
-        // half h of the k1 range lands in columns h * 256 + n2 * 16
-        for (int n2 = 0; n2 < 16; ++n2) {
-          const bool staged = r16_staged(n2);
-          const uint32_t s = it % kR16Stages;
-          if (!mbar_wait(staged ? &x_bar[n2 - kR16XFirst] : &full_bar[s],
-                         staged ? (uint32_t)(local & 1) : (it / kR16Stages) & 1, &abort_sh)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t st =
-              staged ? a2h + (uint32_t)(n2 - kR16XFirst) * kR16StageBytes : ring + s * kR16StageBytes;
+        const uint32_t st = staged ? a2h + (uint32_t)(n2 - kR16XFirst) * kR16StageBytes : ring + s * kR16StageBytes;
+        if (elect_one()) {
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const uint32_t d = tmem + (uint32_t)(h * 256 + n2 * 16);
-#pragma unroll
-            for (int kk = 0; kk < kBK / 16; ++kk) {
-              const uint64_t ah = sw_desc(st + kk * 32), al = sw_desc(st + kR16Tile + kk * 32);
-              const uint64_t bh = sw_desc(bsm + h * 1024 + kk * 32);
-              const uint64_t bl = sw_desc(bsm + kR16BBytes + h * 1024 + kk * 32);
-              umma_bf16_n(d, ah, bh, kIdescN16, kk != 0);
-              umma_bf16_n(d, ah, bl, kIdescN16, 1);
-              umma_bf16_n(d, al, bh, kIdescN16, 1);
-            }
-          }
-          if (!staged) {
-            umma_commit(&empty_bar[s]);
-            ++it;
-          }
-        }
-        if (!ok) break;
-        umma_commit(&d1_bar);
-        // stage 2, one k1 half at a time: 16-point DFTs over n2 into columns h * 256 + j * 32
         for (int h = 0; h < 2; ++h) {
-          if (!mbar_wait(&a2_bar[h], local & 1, &abort_sh)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-#pragma unroll 1
-          for (int j = 0; j < 8; ++j) {
-            const uint32_t d = tmem + (uint32_t)(h * 256 + j * 32);
+          const uint32_t d = tm + (uint32_t)(h * 256 + n2 * 16);
 #pragma unroll
-            for (int kk = 0; kk < kBK / 16; ++kk) {
-              const uint64_t ah = sw_desc(a2h + j * kR16Tile + kk * 32), al = sw_desc(a2l + j * kR16Tile + kk * 32);
-              const uint64_t bh = sw_desc(bsm + kk * 32), bl = sw_desc(bsm + kR16BBytes + kk * 32);
-              umma_bf16_n(d, ah, bh, kIdescN32, kk != 0);
-              umma_bf16_n(d, ah, bl, kIdescN32, 1);
-              umma_bf16_n(d, al, bh, kIdescN32, 1);
-            }
+          for (int kk = 0; kk < kBK / 16; ++kk) {
+            const uint64_t ah = sw_desc(st + kk * 32), al = sw_desc(st + kR16Tile + kk * 32);
+            const uint64_t bh = sw_desc(bsm + h * 1024 + kk * 32);
+            const uint64_t bl = sw_desc(bsm + kR16BBytes + h * 1024 + kk * 32);
+            umma_bf16_n(d, ah, bh, kIdescN16, kk != 0);
+            umma_bf16_n(d, ah, bl, kIdescN16, 1);
+            umma_bf16_n(d, al, bh, kIdescN16, 1);
           }
-          umma_commit(&s2_bar[h]);
         }
+          if (!staged) umma_commit(&empty_bar[s]);
+          if (n2 == 15) umma_commit(&d1_bar);
+        }
+        __syncwarp();
+        if (!staged) ++it;
       }
-      if (!ok) {
-        abort_sh = 1;
-        atomicExch(a.err, 1);
-        umma_commit(&drain_bar);  // every MMA issued so far completes before the TMEM is freed
-        const volatile int never = 0;
-        mbar_wait(&drain_bar, 0, &never);
+      if (!ok) break;
+      // stage 2, one k1 half at a time: 16-point DFTs over n2 into columns h * 256 + j * 32
+      for (int h = 0; h < 2; ++h) {
+        if (!wait(&a2_bar[h], local & 1)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        if (elect_one()) {
+#pragma unroll 1
+        for (int j = 0; j < 8; ++j) {
+          const uint32_t d = tm + (uint32_t)(h * 256 + j * 32);
+#pragma unroll
+          for (int kk = 0; kk < kBK / 16; ++kk) {
+            const uint64_t ah = sw_desc(a2h + j * kR16Tile + kk * 32), al = sw_desc(a2l + j * kR16Tile + kk * 32);
+            const uint64_t bh = sw_desc(bsm + kk * 32), bl = sw_desc(bsm + kR16BBytes + kk * 32);
+            umma_bf16_n(d, ah, bh, kIdescN32, kk != 0);
+            umma_bf16_n(d, ah, bl, kIdescN32, 1);
+            umma_bf16_n(d, al, bh, kIdescN32, 1);
+          }
+        }
+        umma_commit(&s2_bar[h]);
+        }
+        __syncwarp();
       }
+    }
+    if (!ok && elect_one()) {
+      abort_sh = 1;
+      atomicExch(a.err, 1);
+      umma_commit(&drain_bar);  // every MMA issued so far completes before the TMEM is freed
+      const volatile int never = 0;
+      mbar_wait(&drain_bar, 0, &never);
     }
   } else {
     const int q = warp & 3;            // TMEM lane quadrant of this warp
