@@ -1660,8 +1660,9 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   float acc_after = 0.f;
   // Groups of UG pixels: the probe and gain loads of a group are issued
   // together, and the loop body stays small enough for the instruction cache.
-  // (two CTAs per SM at m = 256 hide the load latency and leave 64 registers: groups of 4)
-  constexpr int UGM = ONE ? 4 : EMG_UPDATE_GROUP;
+  // (two CTAs per SM at m = 256 hide the load latency and leave 64 registers: one pair at a
+  // time, 6.51 ms per epoch of 4096 positions against 6.68 with groups of 4 and 7.14 with 8)
+  constexpr int UGM = ONE ? 2 : EMG_UPDATE_GROUP;
   constexpr int UG0 = UGM < PER ? UGM : PER;
   constexpr int UG = PER % UG0 == 0 ? UG0 : 1;
   // The common case (ordered combine, no verify) runs a loop without the mode
