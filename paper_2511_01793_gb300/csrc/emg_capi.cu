@@ -836,7 +836,7 @@ emg_status run_epochs_impl(emg_ctx* c, int32_t n_epochs, const int32_t* order, d
       c->launches[kKindOther] += 2;
       cudaError_t ce = emg::launch_misfit(c->m, c->object, c->probe, c->d_pos, c->d_amp, c->n_rows,
                                           c->n_cols, N, c->d_partial, c->stream);
-      if (ce != cudaSuccess) return cuda_fail(c, ce, "k_misfit launch");
+      if (ce != cudaSuccess) return cuda_fail(c, ce, "k_forward launch");
       ce = emg::launch_sum(c->d_partial, N, 1.0, c->d_hist + c->cap_hist + e, c->stream);
       if (ce != cudaSuccess) return cuda_fail(c, ce, "k_sum launch");
     }
@@ -937,7 +937,7 @@ emg_status read_misfit_sum(emg_ctx* c, int n, double* out) {
 emg_status misfit_now(emg_ctx* c, double* out) {
   cudaError_t e = emg::launch_misfit(c->m, c->object, c->probe, c->d_pos, c->d_amp, c->n_rows, c->n_cols,
                                      c->n_pos, c->d_partial, c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "k_misfit launch");
+  if (e != cudaSuccess) return cuda_fail(c, e, "k_forward launch");
   e = emg::launch_sum(c->d_partial, c->n_pos, 1.0, c->d_scalar, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "k_sum launch");
   EMG_CUDA(c, cudaMemcpyAsync(c->h_scalar, c->d_scalar, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -1209,7 +1209,7 @@ emg_status emg_misfit(emg_ctx* c, double* out) {
   DeviceGuard g(c->device);
   cudaError_t e = emg::launch_misfit(c->m, c->object, c->probe, c->d_pos, c->d_amp, c->n_rows, c->n_cols,
                                      c->n_pos, c->d_partial, c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "k_misfit launch");
+  if (e != cudaSuccess) return cuda_fail(c, e, "k_forward launch");
   e = emg::launch_sum(c->d_partial, c->n_pos, 1.0, c->d_scalar, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "k_sum launch");
   EMG_CUDA(c, cudaMemcpyAsync(c->h_scalar, c->d_scalar, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
