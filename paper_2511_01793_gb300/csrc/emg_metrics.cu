@@ -239,8 +239,8 @@ __global__ void __launch_bounds__(kMetThreads) k_illumination(const double* __re
       bool hit = false;
       if (k < n_pos) {
         p[i] = make_int2(pos[2 * k], pos[2 * k + 1]);
-        hit = p[i].x < r0 + kIllumRows && (long long)p[i].x + m > r0 && p[i].y < c0 + kIllumCols &&
-              (long long)p[i].y + m > c0;
+        hit = p[i].x < (long long)r0 + kIllumRows && (long long)p[i].x + m > r0 &&
+              p[i].y < (long long)c0 + kIllumCols && (long long)p[i].y + m > c0;
       }
       mask[i] = __ballot_sync(0xffffffffu, hit);
       mine += __popc(mask[i]);
@@ -357,7 +357,8 @@ extern "C" emg_status emg_illuminated_region(const float* probe_ref, int32_t m, 
     return EMG_EINVAL;
   const cudaStream_t s = (cudaStream_t)stream;
   const size_t n = (size_t)n_rows * n_cols, nq = (size_t)m * m;
-  const size_t tiles_x = (n_cols + kIllumCols - 1) / kIllumCols, tiles_y = (n_rows + kIllumRows - 1) / kIllumRows;
+  const size_t tiles_x = ((size_t)n_cols + kIllumCols - 1) / kIllumCols;
+  const size_t tiles_y = ((size_t)n_rows + kIllumRows - 1) / kIllumRows;
   double* scratch = nullptr;  // illumination, |Q_ref|^2, the maximum
   if (scratch_alloc(&scratch, n + nq + 1, s) != cudaSuccess) return EMG_ENOMEM;
   double* p2 = scratch + n;
