@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import oracle as O
-from emg_cases import Case, make_context, oracle_inputs, oracle_params, rel_err, state
+from emg_cases import Case, covered_mask, make_context, oracle_inputs, oracle_params, rel_err, state
 
 pytestmark = pytest.mark.gpu
 
@@ -330,6 +330,42 @@ def test_fused_probe_prep_with_one_level_waits_for_the_gain(lib, torch, m, cl):
         out.append(state(c))
         c.close()
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("m,side,b", [(128, 10, 90), (256, 7, 45)])
+def test_fused_probe_prep_over_several_waves(lib, torch, m, side, b):
+    """More positions than clusters fit at once: the prep still runs inside the launch (its clusters
+    take the first tickets) and gives bitwise the results of the separate kernel."""
+    case = Case(n=2 * m + 40, m=m, side=side, step=8, seed=115 + m)
+    p = oracle_params(minibatch=b, levels=3, prolong="bilinear")
+    out = []
+    for fuse in (1, 0):
+        c = make_context(lib, case, p, seed=3)
+        lib.emg_set_prep_fusion(c.ctx, fuse)
+        lib.emg_run_epochs(c.ctx, 2)
+        out.append(state(c))
+        c.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("m,cl", [(16, 1), (16, 2), (32, 1), (32, 2), (64, 2), (64, 4)])
+@pytest.mark.parametrize("levels,prolong,joint", [(1, "const", True), (2, "const", False), (2, "bilinear", True),
+                                                  (3, "const", True), (3, "bilinear", False), (3, "bilinear", True)])
+def test_small_probes_at_every_tiling_match_the_oracle(lib, torch, m, cl, levels, prolong, joint):
+    """Slabs with fewer coarse pixels than threads, the two-level pass and the pair update of every mode."""
+    case = Case(n=2 * m + 41, m=m, side=4, seed=120 + m)
+    p = oracle_params(minibatch=7, levels=levels, prolong=prolong, joint=joint)
+    c = make_context(lib, case, p)
+    lib.emg_set_cluster(c.ctx, cl)
+    idx = [0, 3, 5, 9, 12, 16, 19]
+    lib.emg_step_minibatch(c.ctx, idx)
+    z, q = state(c)
+    c.close()
+    z64, q64, pos, a, po = oracle_inputs(case, p)
+    zo, qo = O.minibatch_step(z64, q64, pos, a, idx, po)
+    mask = covered_mask(case, idx)
+    assert rel_err(z, zo, mask) <= 1e-5 and rel_err(q, qo) <= 1e-5
+    assert np.array_equal(z[~mask], case.z0.astype(np.complex128)[~mask])
 
 
 @pytest.mark.parametrize("b", [1, 64, 65, 2048, 2049])
