@@ -898,50 +898,76 @@ __global__ void __launch_bounds__(256) k_tc_psi(const float2* __restrict__ objec
 // block permutes kR16Rows rows at a time: they are read in natural order
 // (coalesced, all loads of a thread in flight together), permuted in shared
 // memory (padded by one word per 16 against bank conflicts) and written in
-// stored order (coalesced).  With object == nullptr the rows come from `in`
-// (tc_dft2); otherwise they are psi_k = Q . P_k z of minibatch slot kb.
-constexpr int kR16Rows = 4;
+// stored order (16 bytes a thread).  With object == nullptr the rows come from
+// `in` (tc_dft2); otherwise they are psi_k = Q . P_k z of minibatch slot kb.
+// A block takes the same rows of `group` tiles, so that the probe's rows are
+// loaded once for all of them: the kernel is bound by its L2 traffic (256 positions:
+// 134 MB each of object reads, probe reads and stores in 47 us; with groups of 4
+// and 16-byte stores an epoch of four such minibatches went from 2496 to 2455 us).
+constexpr int kR16Rows = 4, kR16Group = 4;
 __global__ void __launch_bounds__(256) k_tc_rows16(const float2* __restrict__ in, const float2* __restrict__ object,
                                                    const float2* __restrict__ probe, const int32_t* __restrict__ pos,
                                                    const int32_t* __restrict__ order, int n_rows, int n_cols,
-                                                   int n_tiles, uint32_t* __restrict__ hi, uint32_t* __restrict__ lo) {
+                                                   int n_tiles, int group, uint32_t* __restrict__ hi,
+                                                   uint32_t* __restrict__ lo) {
   constexpr int m = 256, R = kR16Rows;
-  __shared__ uint32_t sh[R][2][m + m / 16];
+  static_assert(R * m == 256 * 4, "one 16-byte store of each part per thread and tile");
+  __shared__ uint32_t sh[2][R][2][m + m / 16];
   const int c = threadIdx.x;
-  const int pc = r16_perm(c);
-  for (int row0 = blockIdx.x * R; row0 < n_tiles * m; row0 += gridDim.x * R) {  // m is a multiple of R
-    float2 x[R];
+  const int pc = r16_perm(c), sc = pc + (pc >> 4);
+  const int r0 = (int)(blockIdx.x % (m / R)) * R;
+  const int kb0 = (int)(blockIdx.x / (m / R)) * group;
+  const int kb1 = min(kb0 + group, n_tiles);
+  const int wr = c / (m / 4), wc = c % (m / 4) * 4, ws = wc + (wc >> 4);  // the 4 stored elements this thread writes
+  float2 q[R];
+  if (object != nullptr) {
 #pragma unroll
-    for (int i = 0; i < R; ++i) {
-      const int row = row0 + i, kb = row / m, r = row % m;
-      if (object == nullptr) {
-        x[i] = in[(size_t)row * m + c];
-      } else {
-        const int k = order[kb];
-        const int orow = pos[2 * k] + r, ocol = pos[2 * k + 1] + c;
-        float2 z = make_float2(0.f, 0.f);
-        if (orow >= 0 && orow < n_rows && ocol >= 0 && ocol < n_cols) z = object[(size_t)orow * n_cols + ocol];
-        const float2 q = probe[r * m + c];
-        x[i] = make_float2(q.x * z.x - q.y * z.y, q.x * z.y + q.y * z.x);
+    for (int i = 0; i < R; ++i) q[i] = probe[(r0 + i) * m + c];
+  }
+  for (int kb = kb0; kb < kb1; ++kb) {
+    float2 x[R];
+    if (object == nullptr) {
+#pragma unroll
+      for (int i = 0; i < R; ++i) x[i] = in[((size_t)kb * m + r0 + i) * m + c];
+    } else {
+      const int k = order[kb];
+      const int orow = pos[2 * k] + r0, ocol = pos[2 * k + 1] + c;
+      float2 z[R];
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        z[i] = make_float2(0.f, 0.f);
+        if (orow + i >= 0 && orow + i < n_rows && ocol >= 0 && ocol < n_cols)
+          z[i] = object[(size_t)(orow + i) * n_cols + ocol];
       }
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+        x[i] = make_float2(q[i].x * z[i].x - q[i].y * z[i].y, q[i].x * z[i].y + q[i].y * z[i].x);
     }
+    uint32_t(*buf)[2][m + m / 16] = sh[kb & 1];  // the other buffer may still be read
 #pragma unroll
     for (int i = 0; i < R; ++i) {
       uint32_t h, l;
       split_pair(x[i].x, x[i].y, h, l);
-      sh[i][0][pc + (pc >> 4)] = h;
-      sh[i][1][pc + (pc >> 4)] = l;
+      buf[i][0][sc] = h;
+      buf[i][1][sc] = l;
     }
     __syncthreads();
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-      const int row = row0 + i, kb = row / m, r = row % m;
-      const size_t o = ((size_t)kb * m + r16_perm(r)) * m + c;
-      hi[o] = sh[i][0][c + (c >> 4)];
-      lo[o] = sh[i][1][c + (c >> 4)];
-    }
-    __syncthreads();
+    const size_t o = ((size_t)kb * m + r16_perm(r0 + wr)) * m + wc;
+    const uint32_t* bh = &buf[wr][0][ws];
+    const uint32_t* bl = &buf[wr][1][ws];
+    *reinterpret_cast<uint4*>(hi + o) = make_uint4(bh[0], bh[1], bh[2], bh[3]);
+    *reinterpret_cast<uint4*>(lo + o) = make_uint4(bl[0], bl[1], bl[2], bl[3]);
   }
+}
+
+// Grid and tiles per block of k_tc_rows16: grouped only while every SM keeps its eight blocks twice over.
+inline int rows16_group(int n_tiles) {
+  const int g = n_tiles * (256 / kR16Rows) / (152 * 16);
+  return g < 1 ? 1 : g > kR16Group ? kR16Group : g;
+}
+inline int rows16_grid(int n_tiles) {
+  const int g = rows16_group(n_tiles);
+  return (n_tiles + g - 1) / g * (256 / kR16Rows);
 }
 
 // The amplitudes in the layout the dense modulus pass reads: a_k^T[v][u] = sqrt(max(d_k[u][v], 0)).
@@ -1314,8 +1340,8 @@ cudaError_t tc_dft2(TcWork* w, const float2* in, float2* out, int count, int inv
   const size_t n = (size_t)count * m * m;
   const bool r16 = tc_radix16(m);
   if (r16)
-    k_tc_rows16<<<rows / kR16Rows, 256, 0, s>>>(in, nullptr, nullptr, nullptr, nullptr, 0, 0, count, w->buf[0][0],
-                                               w->buf[0][1]);
+    k_tc_rows16<<<rows16_grid(count), 256, 0, s>>>(in, nullptr, nullptr, nullptr, nullptr, 0, 0, count,
+                                                   rows16_group(count), w->buf[0][0], w->buf[0][1]);
   else
     k_tc_split<<<grid_for(n), 256, 0, s>>>(in, w->buf[0][0], w->buf[0][1], n);
   cudaError_t e = cudaGetLastError();
@@ -1357,8 +1383,8 @@ cudaError_t tc_exit_waves(TcWork* w, const TcStepArgs& t, cudaStream_t s) {
   const size_t n = (size_t)t.b * m * m;
   const bool r16 = tc_radix16(m);
   if (r16)
-    k_tc_rows16<<<rows / kR16Rows, 256, 0, s>>>(nullptr, t.object, t.probe, t.pos, t.order, t.n_rows, t.n_cols,
-                                                t.b, w->buf[0][0], w->buf[0][1]);
+    k_tc_rows16<<<rows16_grid(t.b), 256, 0, s>>>(nullptr, t.object, t.probe, t.pos, t.order, t.n_rows, t.n_cols, t.b,
+                                                 rows16_group(t.b), w->buf[0][0], w->buf[0][1]);
   else
     k_tc_psi<<<grid_for(n), 256, 0, s>>>(t.object, t.probe, t.pos, t.order, t.n_rows, t.n_cols, m, t.b,
                                          w->buf[0][0], w->buf[0][1]);

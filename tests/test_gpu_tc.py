@@ -96,6 +96,17 @@ def test_tc_dft2_of_a_delta_is_flat(lib, torch, m, r0, c0):
     assert np.max(np.abs(got - ref)) <= 3 * U * U * 4 * products(m)
 
 
+@pytest.mark.parametrize("count", [75, 77, 115, 155])
+def test_tc_tiles_do_not_depend_on_the_others(lib, torch, count):
+    """m = 256: blocks that take the same rows of 1 to 4 tiles, whole or remainder groups: bitwise
+    what each tile gives in a call of its own."""
+    rng = np.random.default_rng(count)
+    x = (rng.standard_normal((count, 256, 256)) + 1j * rng.standard_normal((count, 256, 256))).astype(np.complex64)
+    got = _run(lib, torch, x, 0)
+    for k in sorted({0, 1, 2, 3, 4, count // 2, count - 3, count - 2, count - 1}):
+        assert np.array_equal(got[k], _run(lib, torch, x[k:k + 1], 0)[0])
+
+
 _DENSE_256 = """
 import sys
 sys.path.insert(0, ".")
@@ -189,6 +200,24 @@ def test_tc_step_matches_the_oracle(lib, torch, m, levels, prolong, nb):
         assert abs(stats[i, 2] - st["mu"]) <= 1e-6 * st["mu"]
         assert abs(stats[i, 0] - st["surrogate_before"]) <= t * st["surrogate_before"]
         assert abs(stats[i, 1] - st["surrogate_after"]) <= t * st["surrogate_before"]
+
+
+def test_tc_positions_of_a_large_minibatch_equal_those_of_small_ones(lib, torch):
+    """m = 256, 79 positions in one minibatch (blocks of several positions, the last group not full,
+    patches across every edge) against the same positions in minibatches of at most 20: each
+    position's surrogate comes from the same state, so it is bitwise the same."""
+    case = Case(n=552, m=256, side=9, step=8, noise_peak=1e5, seed=17)
+    idx = list(range(6, case.n_pos))
+    p = oracle_params(alpha=0.05, levels=2, minibatch=len(idx), prolong="bilinear")
+
+    def surrogate(part):
+        ctx = make_context(lib, case, p, dft=1)
+        lib.emg_step_minibatch(ctx.ctx, part)
+        s = np.array(lib.emg_position_stats(ctx.ctx, len(part)))[:, 0]
+        ctx.close()
+        return s
+
+    assert np.array_equal(surrogate(idx), np.concatenate([surrogate(idx[i:i + 20]) for i in range(0, len(idx), 20)]))
 
 
 def test_tc_epochs_are_bitwise_repeatable(lib, torch):
