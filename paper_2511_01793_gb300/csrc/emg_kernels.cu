@@ -98,6 +98,15 @@ __device__ __forceinline__ float2 czero() { return make_float2(0.f, 0.f); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Cluster barrier arrive without release semantics, for barriers that order
+// execution only (every CTA of the cluster resident; no CTA exits while a
+// neighbour still reads its shared memory).  A release arrive would first
+// wait for all of the thread's outstanding loads and stores.
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
+
 // 16-byte asynchronous copies into shared memory (both addresses 16-byte aligned).
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
@@ -530,6 +539,7 @@ __global__ void __launch_bounds__(kSeedThreads) k_seed(const float2* __restrict_
   __shared__ float part[kSeedCtas];
   cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
   const int rank = (int)cl.block_rank(), ctas = (int)cl.num_blocks(), tid = threadIdx.x;
+  if (ctas > 1) cluster_arrive_relaxed();  // completed (wait) before the first distributed shared memory access
   pdl_wait();  // the probe and the counters belong to the previous kernel until it has ended
   float mx = 0.f;
 #pragma unroll 8
@@ -537,6 +547,7 @@ __global__ void __launch_bounds__(kSeedThreads) k_seed(const float2* __restrict_
   warp_partial_max(mx, redf);
   __syncthreads();
   if (ctas > 1) {
+    cluster_wait();  // rank 0's CTA has started: its shared memory may be written
     if (tid == 0) *cl.map_shared_rank(&part[rank], 0) = partials_max<kSeedThreads>(redf);
     cl.sync();
   } else if (tid == 0) {
@@ -941,16 +952,6 @@ namespace cg = cooperative_groups;
 #ifndef EMG_UPDATE_GROUP
 #define EMG_UPDATE_GROUP 8
 #endif
-
-
-// Cluster barrier arrive without release semantics, for barriers that order
-// execution only (every CTA of the cluster resident; no CTA exits while a
-// neighbour still reads its shared memory).  A release arrive would first
-// wait for all of the thread's outstanding loads and stores.
-__device__ __forceinline__ void cluster_arrive_relaxed() {
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
 
 template <int M, int C>
 struct CTile {

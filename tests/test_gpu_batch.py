@@ -395,6 +395,26 @@ def test_minibatch_indices_reach_the_step_by_every_route(lib, torch, b):
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
 
 
+@pytest.mark.parametrize("m", [64, 128, 256])
+def test_the_seed_finds_the_probe_maximum_in_every_share(lib, torch, m):
+    """The seed of a call splits the probe over the CTAs of a cluster (m >= 128), 512 pixels at a time:
+    one bright pixel in each CTA's share in turn decides max|Q|^2 and with it every weight of the step."""
+    case = Case(n=m + 24, m=m, side=2, step=8, seed=130 + m, edge=False)
+    p = oracle_params(alpha=0.5, minibatch=2)
+    for rank in range(8):
+        flat = case.q_true.copy().reshape(-1)
+        flat[rank * 512 + 37 * rank + (m * m // 4096 - 1) * 4096] = 8.0
+        case.q0 = flat.reshape(m, m)
+        for _ in range(3):
+            c = make_context(lib, case, p)
+            lib.emg_step_minibatch(c.ctx, [0, 3])
+            z, q = state(c)
+            c.close()
+            z64, q64, pos, a, po = oracle_inputs(case, p)
+            zo, qo = O.minibatch_step(z64, q64, pos, a, [0, 3], po)
+            assert rel_err(z, zo) <= 1e-5 and rel_err(q, qo) <= 1e-5
+
+
 def test_host_buffer_call_reports_a_wait_that_gave_up_and_recovers(lib, torch):
     """The host-buffer entry point queues its downloads and waits once; a bounded
     wait that gave up in the step kernel (made to run out) still makes it return
