@@ -257,25 +257,6 @@ __device__ __forceinline__ float block_max(float v, float* sh) {
   return r;
 }
 
-// Sum over the block of per-thread FP32 partials: FP32 warp trees, then the
-// NT/32 warp sums added in FP64 by one thread in a fixed order; the result is
-// broadcast.  Deterministic; avoids FP64 work in every thread.
-template <int NT>
-__device__ __forceinline__ double block_sum_f(float v, float* shf, double* shd) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) shf[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double r = 0.0;
-#pragma unroll
-    for (int i = 0; i < NT / 32; ++i) r += (double)shf[i];
-    shd[0] = r;
-  }
-  __syncthreads();
-  return shd[0];
-}
-
 // FP64 block sum, broadcast: warp trees, then one warp's tree over the NT/32
 // warp sums.  (The FP64 pipe takes two results per SM and clock: every thread
 // adding all warp sums cost 8 us in a block of 1024.)
@@ -315,14 +296,15 @@ __device__ __forceinline__ double warp_sum_exact(float hi) {
 // ---------------------------------------------------------------------------
 // a_k in storage order: amp[k][e_r][e_c] = sqrt(max(d[k][f(e_r)][f(e_c)], 0)).
 // Warp-level max (sum) of v, written by lane 0 of each warp to sh[warp]; after
-// a barrier, partials_max / partials_sum combine them in warp order, as
-// block_max and block_sum_f do, so a caller can let one existing barrier serve.
+// a barrier, partials_max / partials_sum combine them in warp order (the sums in
+// FP64), so a caller can let one existing barrier serve.
 __device__ __forceinline__ void warp_partial_max(float v, float* sh) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
 }
-__device__ __forceinline__ void warp_partial_sum(float v, float* sh) {
+template <typename V>
+__device__ __forceinline__ void warp_partial_sum(V v, V* sh) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
@@ -334,8 +316,8 @@ __device__ __forceinline__ float partials_max(const float* sh) {
   for (int i = 1; i < NT / 32; ++i) r = fmaxf(r, sh[i]);
   return r;
 }
-template <int NT>
-__device__ __forceinline__ double partials_sum(const float* sh) {
+template <int NT, typename V>
+__device__ __forceinline__ double partials_sum(const V* sh) {
   double r = 0.0;
 #pragma unroll
   for (int i = 0; i < NT / 32; ++i) r += (double)sh[i];
@@ -1230,9 +1212,18 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   float2* zbuf = sm + 2 * TL::slab;                           // !ONE: H x M, z_k on my rows (gathered once)
   __shared__ float xf[C];
   __shared__ double xd[C], xd2[C];
-  __shared__ double redd[2];
   __shared__ float redf[NT / 32];
   __shared__ int ticket_sh;
+  // Phi_k of small probes: the threads' partials are added in FP64 (few warps, so the FP64
+  // pipe's two results per clock and SM suffice); larger ones in FP32 warp trees.
+  constexpr bool kSum64 = M <= 32;
+  using Part = std::conditional_t<kSum64, double, float>;
+  __shared__ double red64[kSum64 ? NT / 32 : 1];
+  Part* sums;
+  if constexpr (kSum64)
+    sums = red64;
+  else
+    sums = redf;
   const int tid = threadIdx.x;
   int kb = blockIdx.x / C;
   if constexpr (!RIN) {
@@ -1373,11 +1364,11 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
     for (int i = 0; i < N1; ++i) p[i] = v[i];
   }
   // per-warp misfit partials; the barrier also orders the pass before the next one
-  warp_partial_sum(acc, redf);
+  warp_partial_sum<Part>(acc, sums);
   __syncthreads();
   // inverse column pass A, outputs to the row slabs
   col_pass_a_inv_to_rows<TL>(cl, rank, colbuf, rowbuf, tid);
-  if (tid == 0) cluster_publish<C>(cl, rank, xd, partials_sum<NT>(redf));
+  if (tid == 0) cluster_publish<C>(cl, rank, xd, partials_sum<NT>(sums));
   tile_sync<C>(cl);
   // a4: inverse row passes -> R (natural order) on my rows
   gpass_b<M, H, SR, 1, NT, true>(rowbuf, tid);
@@ -1787,8 +1778,9 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   }
   }
   if (a.verify) {
-    const double part = 0.5 * block_sum_f<NT>(acc_after, redf, redd);
-    if (tid == 0) cluster_publish<C>(cl, rank, xd2, part);
+    warp_partial_sum<Part>(acc_after, sums);
+    __syncthreads();
+    if (tid == 0) cluster_publish<C>(cl, rank, xd2, 0.5 * partials_sum<NT>(sums));
   }
   // With halo rows read from the neighbours (bilinear prolongation, other
   // than two or three levels) a neighbour may still read my coarse rows: no CTA leaves

@@ -522,6 +522,49 @@ def test_pinned_host_intensity_equals_device_intensity(lib, torch, m, levels):
     c1.close()
 
 
+@pytest.mark.parametrize("cl", [1, 2])
+@pytest.mark.parametrize("m", [16, 32])
+def test_small_probe_surrogates_are_summed_in_64_bits(lib, torch, m, cl):
+    """At most 16 pixels per thread with integer a_k^2 below 2^20 (z = 0, so Phi_k is half the mean of
+    a_k^2): every thread's FP32 partial is exact, their sum needs more than 24 bits and comes out exact."""
+    rng = np.random.default_rng(7 * m + cl)
+    n_pos = 6
+    a = rng.integers(400, 1000, size=(n_pos, m, m)).astype(np.float64)
+    pos = rng.integers(0, m, size=(n_pos, 2)).astype(np.int32)
+    q = (rng.standard_normal((m, m)) + 1j * rng.standard_normal((m, m))).astype(np.complex64)
+    c = lib.Context(pos, (a * a).astype(np.float32), 2 * m, 2 * m, lib.emg_default_params(minibatch=n_pos),
+                    obj=torch.zeros((2 * m, 2 * m), dtype=torch.complex64), probe=torch.from_numpy(q))
+    lib.emg_set_cluster(c.ctx, cl)
+    lib.emg_step_minibatch(c.ctx, np.arange(n_pos))
+    got = lib.emg_position_stats(c.ctx, n_pos)[:, 0]
+    c.close()
+    assert np.array_equal(got, 0.5 * np.sum(a * a, axis=(1, 2)) / m ** 2)
+
+
+@pytest.mark.parametrize("cl", [1, 2])
+@pytest.mark.parametrize("m", [16, 32])
+def test_small_probe_surrogates_after_the_step_are_summed_in_64_bits(lib, torch, m, cl):
+    """z = 0 and amplitudes at four column frequencies: every row of R_k repeats 4 Gaussian integers, one
+    of them 2^10 times the others, and z~ = 0.  The surrogate after the step is half the sum of |R_k|^2,
+    whose FP32 partials per thread are exact and whose sum needs more than 24 bits."""
+    n_pos = 8
+    rng = np.random.default_rng(31 * m + cl)
+    x = np.zeros((n_pos, 4), dtype=np.int64)
+    x[:, :3] = rng.integers(-60, 60, size=(n_pos, 3))
+    x[:, 3] = -x.sum(axis=1)
+    a = np.zeros((n_pos, m, m))
+    a[:, 0, ::m // 4] = (x + 256 * rng.integers(9, 15, size=(n_pos, 1))) * m * m
+    c = lib.Context(np.zeros((n_pos, 2), dtype=np.int32), (a * a).astype(np.float32), m, m,
+                    lib.emg_default_params(minibatch=n_pos), obj=torch.zeros((m, m), dtype=torch.complex64),
+                    probe=torch.ones((m, m), dtype=torch.complex64))
+    lib.emg_set_cluster(c.ctx, cl)
+    lib.emg_set_verify(c.ctx, True)
+    lib.emg_step_minibatch(c.ctx, np.arange(n_pos))
+    got = lib.emg_position_stats(c.ctx, n_pos)[:, 1]
+    c.close()
+    assert np.array_equal(got, 0.5 * np.sum(np.round(np.abs(np.fft.ifft2(a)) ** 2), axis=(1, 2)))
+
+
 @pytest.mark.parametrize("scatter,dft", [(0, 0), (1, 1)])
 def test_create_releases_everything_when_an_allocation_fails(lib, torch, scatter, dft):
     """Host-side fault injection: each device allocation of emg_create fails in
