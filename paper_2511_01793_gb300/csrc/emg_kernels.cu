@@ -163,30 +163,47 @@ __device__ __forceinline__ float2 cfma_conj(float2 a, float2 b, float2 c) {
 // A floor of 1e-37 under both square roots gives y = 0 for w = 0 without a
 // branch; it changes no result for |w|^2 above about 1e-29.  The sign flip
 // is applied to the sign bit when Re(y conj(x)) < 0.
-// REFINED: both roots take one Newton step, which brings their error from the
-// rsqrt unit's down to the FP32 rounding of a correctly rounded root's.
-template <bool REFINED>
 __device__ __forceinline__ float2 geomean_aligned_root(float2 x, float2 xp) {
   const float2 w = cmul(x, xp);
   const float n = fmaf(w.x, w.x, w.y * w.y);
-  const float r = rsqrtf(n + 1e-37f);
-  float mag = n * r;
-  if constexpr (REFINED) mag = fmaf(fmaf(-mag, mag, n), 0.5f * r, mag);
+  const float mag = n * rsqrtf(n + 1e-37f);
   const float s2 = fabsf(w.x) + mag;
-  float q = rsqrtf(s2 + 1e-37f);
-  if constexpr (REFINED) q = fmaf(fmaf(-(s2 * q), q, 1.f), 0.5f * q, q);
-  const float rr = q * 0.70710678118654752f;
+  const float rr = rsqrtf(s2 + 1e-37f) * 0.70710678118654752f;
   const float t = s2 * rr, vh = w.y * rr;
   const float yx = w.x >= 0.f ? t : vh, yy = w.x >= 0.f ? vh : t;
   const unsigned sbit = fmaf(yx, x.x, yy * x.y) < 0.f ? 0x80000000u : 0u;
   return make_float2(__uint_as_float(__float_as_uint(yx) ^ sbit), __uint_as_float(__float_as_uint(yy) ^ sbit));
 }
 
+// geometric_mean_aligned without its branches and the slow paths of IEEE roots and division: from the
+// rsqrt unit, with one Newton step each for |w|, t and v h, which leaves about the rounding of correctly
+// rounded operations.  Where |w|^2 is an FP32 number at all the lower bounds under the roots change
+// nothing (s >= |w| / 2 >= 5.4e-20), so there is no floor; w = 0 gives 0, a tie keeps the principal root.
+__device__ __forceinline__ float2 geometric_mean_rounded(float2 x, float2 xp) {
+  const float2 w = cmul(x, xp);
+  const float n = fmaf(w.x, w.x, w.y * w.y);
+  const float r = rsqrtf(fmaxf(n, 1.17549435e-38f));
+  float mag = n * r;
+  mag = fmaf(0.5f * mag, fmaf(-mag, r, 1.f), mag);  // the residual of r, of size 1: it never underflows
+  const float s = 0.5f * (fabsf(w.x) + mag);
+  const float q = rsqrtf(fmaxf(s, 5e-20f)), h = 0.5f * q;  // h = 1 / (2 t)
+  float t = s * q;
+  t = fmaf(fmaf(-t, t, s), h, t);
+  float vh = w.y * h;
+  vh = fmaf(fmaf(-2.f * t, vh, w.y), h, vh);
+  const unsigned sv = w.x < 0.f ? __float_as_uint(w.y) & 0x80000000u : 0u;  // (|v h|, t sign(v)) when u < 0
+  const float yx = w.x < 0.f ? vh : t, yy = w.x < 0.f ? t : vh;
+  const float2 y = make_float2(__uint_as_float(__float_as_uint(yx) ^ sv), __uint_as_float(__float_as_uint(yy) ^ sv));
+  const unsigned sbit = fmaf(y.x, x.x, y.y * x.y) < 0.f ? 0x80000000u : 0u;
+  return make_float2(__uint_as_float(__float_as_uint(y.x) ^ sbit), __uint_as_float(__float_as_uint(y.y) ^ sbit));
+}
+
 // a5 (finest level) + a6 + a7 at one pixel: with MG the fine MAGPIE step from
 // the prolonged coarse correction pro, z^+ = zp + G_0 (R - Q zp) with
 // zp = z_k + pro, else z^+ = z_k + G_0 (R - Q z_k); Q^+ = Q + conj(z_k)(R - Q z_k)/mu_k;
-// with JOINT their aligned geometric means with z_k and Q (Eq. geomean).
-template <bool MG, bool JOINT, bool REFINED>
+// with JOINT their aligned geometric means with z_k and Q (Eq. geomean), to the
+// accuracy of correctly rounded roots (ROUNDED) or of the rsqrt unit.
+template <bool MG, bool JOINT, bool ROUNDED>
 __device__ __forceinline__ void update_pixel(float2 zk, float2 q, float2 g0, float2 R, float2 pro, float inv_mu,
                                              float2& zn, float2& qn) {
   const float2 res = cfnma(q, zk, R);
@@ -198,9 +215,12 @@ __device__ __forceinline__ void update_pixel(float2 zk, float2 q, float2 g0, flo
     zplus = cfma(g0, res, zk);
   }
   const float2 qplus = cfma_conj(zk, cscale(res, inv_mu), q);
-  if constexpr (JOINT) {
-    zn = geomean_aligned_root<REFINED>(zk, zplus);
-    qn = geomean_aligned_root<REFINED>(q, qplus);
+  if constexpr (JOINT && ROUNDED) {
+    zn = geometric_mean_rounded(zk, zplus);
+    qn = geometric_mean_rounded(q, qplus);
+  } else if constexpr (JOINT) {
+    zn = geomean_aligned_root(zk, zplus);
+    qn = geomean_aligned_root(q, qplus);
   } else {
     zn = zplus;
     qn = qplus;
@@ -1667,9 +1687,11 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   const bool pairs = UGP > 0 && !a.s_num && !a.verify && slot_ok &&
                      ((reinterpret_cast<uintptr_t>(a.probe) | reinterpret_cast<uintptr_t>(G0) |
                        reinterpret_cast<uintptr_t>(zt) | reinterpret_cast<uintptr_t>(qt)) & 15) == 0;
-  // Small probes keep the accuracy of correctly rounded roots (their arithmetic before they
-  // came to this kernel) at the cost of a few dependent operations.
-  constexpr bool kRefined = M <= 32;
+  // Small probes take the accuracy of correctly rounded roots, as the allocation-free step does: no
+  // floor under the squares (an object in units of 1e-9 has |z z+|^2 of 1e-36), and at an exact tie the
+  // principal root.  (An epoch of 100 positions at m = 32, minibatches of 10: 85.5 us, with IEEE roots
+  // and division 107, with one Newton step under the floor 83.8.)
+  constexpr bool kRounded = M <= 32;
   auto update_pairs = [&](auto multigrid, auto joint) {
     constexpr bool kMg = decltype(multigrid)::value, kJoint = decltype(joint)::value;
     constexpr int PP = PER / 2, RP = 2 * RPT;
@@ -1713,7 +1735,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
           const float2 zk = h ? make_float2(zk2.z, zk2.w) : make_float2(zk2.x, zk2.y);
           const float2 q = h ? make_float2(qv[u].z, qv[u].w) : make_float2(qv[u].x, qv[u].y);
           const float2 g0 = h ? make_float2(gv[u].z, gv[u].w) : make_float2(gv[u].x, gv[u].y);
-          update_pixel<kMg, kJoint, kRefined>(zk, q, g0, rb[t * RP * SR + h], pro[h], inv_mu, zo[h], qo[h]);
+          update_pixel<kMg, kJoint, kRounded>(zk, q, g0, rb[t * RP * SR + h], pro[h], inv_mu, zo[h], qo[h]);
         }
         const int off = off0 + 2 * t * NT;
         *reinterpret_cast<float4*>(zt + off) = make_float4(zo[0].x, zo[0].y, zo[1].x, zo[1].y);
@@ -1760,14 +1782,14 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
     float2 zn, qn;
     if (a.levels == 1) {
       if (a.joint)
-        update_pixel<false, true, kRefined>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
+        update_pixel<false, true, kRounded>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
       else
-        update_pixel<false, false, kRefined>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
+        update_pixel<false, false, kRounded>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
     } else {
       if (a.joint)
-        update_pixel<true, true, kRefined>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
+        update_pixel<true, true, kRounded>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
       else
-        update_pixel<true, false, kRefined>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
+        update_pixel<true, false, kRounded>(zk, q, gv[u], R, pro, inv_mu, zn, qn);
     }
     if (a.s_num)
       scatter_atomic(a.s_num, a.s_den, a.combine, a.n_rows, a.n_cols, o_r + r, o_c + c, zn, zk, fmaf(a.w_eps, MQ, cabs2(q)));

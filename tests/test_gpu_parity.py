@@ -565,6 +565,46 @@ def test_small_probe_surrogates_after_the_step_are_summed_in_64_bits(lib, torch,
     assert np.array_equal(got, 0.5 * np.sum(np.round(np.abs(np.fft.ifft2(a)) ** 2), axis=(1, 2)))
 
 
+@pytest.mark.parametrize("m,cl", [(16, 1), (16, 2), (32, 1), (32, 2)])
+def test_small_probe_roots_of_faint_objects(lib, torch, m, cl):
+    """A positive object in units of 1e-9 under a flat probe (z z+ real, of about 1e-18, so its square is a
+    normal FP32 number): the joint step's roots keep FP32 accuracy."""
+    rng = np.random.default_rng(m)
+    z0, z_true = (c64(1e-9 * rng.uniform(0.8, 1.2, size=(m, m))) for _ in range(2))
+    d = (np.abs(np.fft.fft2(z_true.astype(np.complex128))) ** 2).astype(np.float32)[None]
+    q0 = np.ones((m, m), dtype=np.complex64)
+    p = oracle_params(minibatch=1)
+    pos = np.zeros((1, 2), dtype=np.int32)
+    c = lib.Context(pos, d, m, m, gpu_params(lib, p), obj=torch.from_numpy(z0), probe=torch.from_numpy(q0))
+    lib.emg_set_cluster(c.ctx, cl)
+    lib.emg_step_minibatch(c.ctx, [0])
+    z, q = state(c)
+    c.close()
+    zo, qo = O.minibatch_step(z0.astype(np.complex128), q0.astype(np.complex128), pos, np.sqrt(d.astype(np.float64)),
+                              [0], O.Params(alpha=float(np.float32(0.05)), minibatch=1, w_eps=float(np.float32(1e-6))))
+    assert rel_err(z, zo) <= STEP_TOL and rel_err(q, qo) <= STEP_TOL
+
+
+@pytest.mark.parametrize("m,cl", [(16, 1), (16, 2), (32, 1), (32, 2)])
+def test_small_probe_roots_keep_the_principal_one_at_a_tie(lib, torch, m, cl):
+    """Q = 1 and spectra of powers of two give z+ = R_k = -z_k = 2 + i exactly on every other pixel of
+    every other row: both roots of z_k z+ = -3 - 4i are orthogonal to z_k, and the principal one, 1 - 2i,
+    is kept."""
+    s = (-1.0) ** np.arange(m)
+    z = (2 + 4 * s)[None, :] + 1j * s[:, None] * (1 + 2 * s)[None, :]
+    assert np.all(z[::2, 1::2] == -2 - 1j)
+    a = np.zeros((m, m))
+    a[0, 0], a[0, m // 2], a[m // 2, 0], a[m // 2, m // 2] = 4 * m * m, 2 * m * m, 2 * m * m, m * m
+    c = lib.Context(np.zeros((1, 2), dtype=np.int32), (a * a)[None].astype(np.float32), m, m,
+                    lib.emg_default_params(minibatch=1, w_eps=0.0), obj=torch.from_numpy(c64(z)),
+                    probe=torch.ones((m, m), dtype=torch.complex64))
+    lib.emg_set_cluster(c.ctx, cl)
+    lib.emg_step_minibatch(c.ctx, [0])
+    got, _ = state(c)
+    c.close()
+    assert np.max(np.abs(got[::2, 1::2] - (1 - 2j))) <= 1e-6
+
+
 @pytest.mark.parametrize("scatter,dft", [(0, 0), (1, 1)])
 def test_create_releases_everything_when_an_allocation_fails(lib, torch, scatter, dft):
     """Host-side fault injection: each device allocation of emg_create fails in
