@@ -298,11 +298,12 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return r;
 }
 
-// Warp sum of FP32 values to FP64 accuracy without the FP64 pipe: each tree
+// Warp sum of FP32 values without the FP64 pipe, to about 48 bits: each tree
 // level adds exactly (Knuth's TwoSum) and carries the rounding errors along.
-// Lane 0 gets the value.
-__device__ __forceinline__ double warp_sum_exact(float hi) {
-  float lo = 0.f;
+// Every lane has the same `hi`, so where the sum leaves the FP32 range (or a value
+// is not finite) the whole warp adds in FP64.  Lane 0 gets the value.
+__device__ __forceinline__ double warp_sum_exact(float v) {
+  float hi = v, lo = 0.f;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const float b = __shfl_xor_sync(0xffffffffu, hi, o), bl = __shfl_xor_sync(0xffffffffu, lo, o);
@@ -310,7 +311,10 @@ __device__ __forceinline__ double warp_sum_exact(float hi) {
     lo += bl + ((hi - (s - t)) + (b - t));
     hi = s;
   }
-  return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+  if (isfinite(hi)) return (double)hi + (double)lo;
+  double s = v;
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
 }
 
 // ---------------------------------------------------------------------------

@@ -605,6 +605,19 @@ def test_small_probe_roots_keep_the_principal_one_at_a_tie(lib, torch, m, cl):
     assert np.max(np.abs(got[::2, 1::2] - (1 - 2j))) <= 1e-6
 
 
+@pytest.mark.parametrize("m", [16, 32, 64, 128, 256])
+def test_misfit_sums_beyond_the_fp32_range(lib, torch, m):
+    """Intensities of 4e36 (z = 0, so Phi_k is half their mean): a warp's sum of a_k^2 exceeds the largest
+    FP32 number, a thread's does not; the misfit is their FP64 sum."""
+    d = np.random.default_rng(m).uniform(3e36, 4e36, size=(3, m, m)).astype(np.float32)
+    c = lib.Context(np.zeros((3, 2), dtype=np.int32), d, m, m, lib.emg_default_params(minibatch=3),
+                    obj=torch.zeros((m, m), dtype=torch.complex64), probe=torch.ones((m, m), dtype=torch.complex64))
+    got = lib.emg_misfit(c.ctx)
+    c.close()
+    want = 0.5 * np.sum(d.astype(np.float64)) / m ** 2
+    assert abs(got - want) <= 1e-6 * want
+
+
 @pytest.mark.parametrize("scatter,dft", [(0, 0), (1, 1)])
 def test_create_releases_everything_when_an_allocation_fails(lib, torch, scatter, dft):
     """Host-side fault injection: each device allocation of emg_create fails in
