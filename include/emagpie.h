@@ -211,7 +211,8 @@ emg_status emg_run_epochs(emg_ctx* ctx, int32_t n_epochs, const int32_t* order,
  * exit waves are stored); positions are processed in chunks (see
  * emg_set_gradient_chunk) and summed in a fixed order, so
  * results repeat bitwise for a given chunk size.  The first call may allocate
- * the chunk's patch buffers.
+ * the chunk's patch buffers; where an automatic chunk's do not fit, the chunk
+ * becomes the minibatch, whose buffers the context has.
  *  object, probe            device complex64 [n_rows][n_cols], [m][m] (read only)
  *  grad_object, grad_probe  device complex64, same shapes, overwritten; either may be NULL
  *  misfit                   host double or NULL (synchronises when not NULL)
@@ -222,10 +223,11 @@ emg_status emg_misfit_gradient(emg_ctx* ctx, const float* object, const float* p
 /*
  * Positions per launch of emg_misfit_gradient: 0 (the default) chooses equal
  * chunks of whole waves of the position clusters that can be resident at once,
- * with at most about 160 MB of patch gradients; n > 0 takes n.  The chunk only
- * changes speed and the rounding order of the sums.  Synchronises the
- * context's stream and frees the previous chunk's buffers.  EMG_EINVAL for
- * n < 0.
+ * with at most about 160 MB of object patch gradients (at m = 256 the probe's
+ * take as much again); n > 0 takes n, and the gradient call returns EMG_ENOMEM
+ * when its buffers do not fit.  The chunk only changes speed and the rounding
+ * order of the sums.  Synchronises the context's stream and frees the previous
+ * chunk's buffers.  EMG_EINVAL for n < 0.
  */
 emg_status emg_set_gradient_chunk(emg_ctx* ctx, int32_t positions);
 

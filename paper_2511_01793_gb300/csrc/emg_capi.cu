@@ -27,7 +27,9 @@ enum { kKindPrep = 0, kKindStep = 1, kKindApply = 2, kKindOther = 3, kKindDft = 
 // Epochs whose misfit histories emg_reconstruct_host stages in the pinned scratch
 // (h_scalar holds 64 doubles: two histories and the wait flag).
 constexpr int kHostStageEpochs = 31;
-// Patch gradients of one chunk of emg_misfit_gradient, at most (when chosen automatically).
+// Object patch gradients of one chunk of emg_misfit_gradient, at most (when chosen automatically).
+// At m = 256 the probe-gradient sums (one per position of the chunk) take as much again: 302 MB in all
+// for 1600 positions.  Half the chunk would halve both and costs 6 % (1.65 against 1.75 ms).
 constexpr size_t kGradPatchBytes = (size_t)160 << 20;
 
 // A captured epoch and the state it was captured for.
@@ -1439,14 +1441,20 @@ emg_status emg_misfit_gradient(emg_ctx* c, const float* object, const float* pro
       chunk = c->par.minibatch;
     }
     if (chunk > N) chunk = N;
-    const int slots = emg::gradient_slots(c->m, pw, chunk);
+    int slots = emg::gradient_slots(c->m, pw, chunk);
     if (chunk > c->par.minibatch) {
-      const size_t mm = (size_t)c->m * c->m * sizeof(float2);
-      if (cudaMalloc(&c->d_gz, chunk * mm) != cudaSuccess || cudaMalloc(&c->d_gq, slots * mm) != cudaSuccess) {
+      const size_t mm = (size_t)c->m * c->m;
+      cudaError_t e = dmalloc(&c->d_gz, chunk * mm);
+      if (e == cudaSuccess) e = dmalloc(&c->d_gq, slots * mm);
+      if (e != cudaSuccess) {
         cudaFree(c->d_gz);
-        c->d_gz = nullptr;
+        c->d_gz = c->d_gq = nullptr;
         cudaGetLastError();
-        return fail(c, EMG_ENOMEM, "cudaMalloc(gradient patches) failed");
+        if (c->grad_chunk_req > 0 || e != cudaErrorMemoryAllocation)
+          return fail(c, EMG_ENOMEM, "cudaMalloc(gradient patches) failed");
+        // the device is nearly full: chunks that the minibatch buffers hold
+        chunk = c->par.minibatch;
+        slots = emg::gradient_slots(c->m, pw, chunk);
       }
     }
     c->grad_chunk = chunk;

@@ -187,3 +187,35 @@ def test_gradients_of_many_positions_by_every_split(lib, torch, m, n_pos, chunk)
     assert abs(phi - want) <= 1e-5 * want
     assert np.linalg.norm(gz - rz) <= 1e-5 * np.linalg.norm(rz) and np.linalg.norm(gq - rq) <= 1e-5 * np.linalg.norm(rq)
     c.close()
+
+
+@pytest.mark.parametrize("m", [32, 256])
+@pytest.mark.parametrize("after", [0, 1])
+def test_gradient_without_room_for_its_chunk_takes_the_minibatch(lib, torch, m, after):
+    """Host-side fault injection: one of the automatic chunk's two buffers does not fit.  The call runs in
+    chunks that the minibatch buffers hold, with bitwise their sums, and keeps no part of the failed
+    allocation; a chunk that was asked for is still refused."""
+    case = Case(n=2 * m + 40, m=m, side=4, seed=150 + m)
+    p = oracle_params(minibatch=5)
+
+    def call(chunk, fail):
+        ctx = make_context(lib, case, p)
+        lib.emg_set_gradient_chunk(ctx.ctx, chunk)
+        free = torch.cuda.mem_get_info()[0]
+        try:
+            lib.emg_debug_fail_alloc(after if fail else -1)
+            out = _gpu_gradient(lib, torch, ctx, case.z0, case.q0)
+        finally:
+            lib.emg_debug_fail_alloc(-1)
+            lost = free - torch.cuda.mem_get_info()[0]
+            ctx.close()
+        return out, lost
+
+    call(0, False)                                          # lazy CUDA state in place
+    (phi, gz, gq), lost = call(0, True)
+    want = call(5, False)[0]
+    assert phi == want[0] and np.array_equal(gz, want[1]) and np.array_equal(gq, want[2])
+    assert lost <= 4 << 20
+    with pytest.raises(lib.EmgError) as e:
+        call(case.n_pos, True)
+    assert e.value.status == lib.EMG_ENOMEM
