@@ -2061,16 +2061,22 @@ __global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_grad
   }
 }
 
-// Object gradient sum_k P_k^T gz_k over tiles of 16 x 32 pixels (optionally
+// Object gradient sum_k P_k^T gz_k over tiles of 8 PX x 32 pixels (optionally
 // added to the existing values: later chunks of positions) and probe gradient
 // sum of the slots' gq, each in a fixed order (deterministic).  Bound by
-// the loads: a thread keeps those of four patches at two pixels in flight, and
+// the loads: a thread keeps those of U patches at PX pixels in flight, and
 // the positions that overlap a tile are listed kGradList at a time, so any number
-// of positions takes the same shared memory.
-constexpr int kGradList = 512, kGradTileW = 32;
+// of positions takes the same shared memory.  PX = 2, U = 4; objects with fewer
+// than kGradSmallTiles such tiles (two per SM) take PX = 1, U = 8, or they would
+// leave SMs idle (us per call of 1444 positions: object 192^2 and m = 64 142 / 113,
+// 320^2 and m = 128 443 / 371).  Each tile reads all positions, so more tiles
+// cost more where many positions miss them: 512^2, 4096 positions, m = 32 51 / 58.
+constexpr int kGradList = 512, kGradSmallTiles = 304, kGradTileW = 32, kGradTileH = kApplyThreads / 32;
+template <int PX, int U>
 __global__ void __launch_bounds__(kApplyThreads) k_grad_reduce(const GradReduceArgs a) {
   constexpr int WARPS = kApplyThreads / 32, PW = kGradList / WARPS, ROUNDS = PW / 32, PP = kApplyProbePx / 32;
-  static_assert(WARPS == kApplyProbeGroups && 2 * WARPS == kApplyTile, "two tile rows per warp");
+  constexpr int TILE_H = PX * WARPS;
+  static_assert(WARPS == kApplyProbeGroups && (PX == 1 || PX == 2), "one or two tile rows per warp");
   __shared__ int3 list[kGradList];
   __shared__ int count[WARPS];
   __shared__ float2 part_s[kApplyProbeGroups][kApplyProbePx];
@@ -2081,10 +2087,12 @@ __global__ void __launch_bounds__(kApplyThreads) k_grad_reduce(const GradReduceA
   pdl_trigger();
   if ((int)blockIdx.x < n_tiles) {
     if (!a.grad_object) return;
-    const int r0 = (int)(blockIdx.x / a.tiles_x) * kApplyTile, c0 = (int)(blockIdx.x % a.tiles_x) * kGradTileW;
+    const int r0 = (int)(blockIdx.x / a.tiles_x) * TILE_H, c0 = (int)(blockIdx.x % a.tiles_x) * kGradTileW;
     bool waited = false;
-    const int row = r0 + warp, col = c0 + lane;  // pixels (row, col) and (row + WARPS, col)
-    float2 g[2] = {czero(), czero()};
+    const int row = r0 + warp, col = c0 + lane;  // pixels (row + h WARPS, col)
+    float2 g[PX];
+#pragma unroll
+    for (int h = 0; h < PX; ++h) g[h] = czero();
     for (int k0 = 0; k0 < a.b; k0 += kGradList) {
       // ordered compaction: warp w lists the w-th run of these positions
       int3 p[ROUNDS];
@@ -2096,7 +2104,7 @@ __global__ void __launch_bounds__(kApplyThreads) k_grad_reduce(const GradReduceA
         bool hit = false;
         if (kb < a.b) {
           p[i] = make_int3(kb, a.pos[2 * (a.first + kb)], a.pos[2 * (a.first + kb) + 1]);
-          hit = p[i].y < r0 + kApplyTile && p[i].y + m > r0 && p[i].z < c0 + kGradTileW && p[i].z + m > c0;
+          hit = p[i].y < r0 + TILE_H && p[i].y + m > r0 && p[i].z < c0 + kGradTileW && p[i].z + m > c0;
         }
         mask[i] = __ballot_sync(0xffffffffu, hit);
         mine += __popc(mask[i]);
@@ -2118,29 +2126,30 @@ __global__ void __launch_bounds__(kApplyThreads) k_grad_reduce(const GradReduceA
       __syncthreads();
       if (!waited) pdl_wait();  // the patch gradients; the first list needs the positions alone
       waited = true;
-      for (int t0 = 0; t0 < total; t0 += 4) {
-        float2 v[4][2];
+      for (int t0 = 0; t0 < total; t0 += U) {
+        float2 v[U][PX];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          v[u][0] = v[u][1] = czero();
+        for (int u = 0; u < U; ++u) {
+          v[u][0] = v[u][PX - 1] = czero();
           if (t0 + u < total) {
             const int3 q = list[t0 + u];
             const int lr = row - q.y, lc = col - q.z;
             const float2* src = a.gz + (size_t)q.x * mm + lr * m + lc;
             const bool in_c = (unsigned)lc < (unsigned)m;
             if (in_c && (unsigned)lr < (unsigned)m) v[u][0] = src[0];
-            if (in_c && (unsigned)(lr + WARPS) < (unsigned)m) v[u][1] = src[WARPS * m];
+            if constexpr (PX > 1)
+              if (in_c && (unsigned)(lr + WARPS) < (unsigned)m) v[u][1] = src[WARPS * m];
           }
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < U; ++u)
 #pragma unroll
-          for (int h = 0; h < 2; ++h) g[h] = cadd(g[h], v[u][h]);
+          for (int h = 0; h < PX; ++h) g[h] = cadd(g[h], v[u][h]);
       }
     }
     if (col >= a.n_cols) return;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < PX; ++h) {
       if (row + h * WARPS >= a.n_rows) continue;
       const size_t gi = (size_t)(row + h * WARPS) * a.n_cols + col;
       a.grad_object[gi] = a.accumulate ? cadd(a.grad_object[gi], g[h]) : g[h];
@@ -2976,9 +2985,13 @@ cudaError_t launch_gradient(int m, int slots, const GradArgs& a, cudaStream_t s)
 cudaError_t launch_grad_reduce(const GradReduceArgs& a, cudaStream_t s) {
   GradReduceArgs t = a;
   t.tiles_x = (a.n_cols + kGradTileW - 1) / kGradTileW;
-  t.tiles_y = (a.n_rows + kApplyTile - 1) / kApplyTile;
+  t.tiles_y = (a.n_rows + 2 * kGradTileH - 1) / (2 * kGradTileH);
   const int n_probe = (a.m * a.m + kApplyProbePx - 1) / kApplyProbePx;
-  const cudaError_t e = launch_pdl(k_grad_reduce, dim3(t.tiles_x * t.tiles_y + n_probe), dim3(kApplyThreads), 0, s, t);
+  const bool small = t.tiles_x * t.tiles_y < kGradSmallTiles;
+  if (small) t.tiles_y = (a.n_rows + kGradTileH - 1) / kGradTileH;
+  const dim3 grid(t.tiles_x * t.tiles_y + n_probe);
+  const cudaError_t e = small ? launch_pdl(k_grad_reduce<1, 8>, grid, dim3(kApplyThreads), 0, s, t)
+                              : launch_pdl(k_grad_reduce<2, 4>, grid, dim3(kApplyThreads), 0, s, t);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -219,3 +219,31 @@ def test_gradient_without_room_for_its_chunk_takes_the_minibatch(lib, torch, m, 
     with pytest.raises(lib.EmgError) as e:
         call(case.n_pos, True)
     assert e.value.status == lib.EMG_ENOMEM
+
+
+@pytest.mark.parametrize("n,n_pos,chunk", [(165, 160, 100), (640, 100, 0)])
+def test_gradients_of_small_and_large_objects(lib, torch, n, n_pos, chunk):
+    """m = 128: small objects are summed over smaller tiles.  Repeats bitwise and equals the sum of
+    one-position calls to FP32 rounding."""
+    m = 128
+    rng = np.random.default_rng(n + chunk)
+    pos = rng.integers(-m // 3, n - m // 2, size=(n_pos, 2)).astype(np.int32)
+    z, q = (c64(rng.standard_normal(s) + 1j * rng.standard_normal(s)) for s in ((n, n + 3), (m, m)))
+    d = (rng.uniform(0.5, 2.0, size=(n_pos, m, m)) * 2 * m * m).astype(np.float32)
+
+    def call(sub, chunk):
+        c = lib.Context(pos[sub], d[sub], n, n + 3, lib.emg_default_params(), obj=torch.from_numpy(z),
+                        probe=torch.from_numpy(q))
+        lib.emg_set_gradient_chunk(c.ctx, chunk)
+        out = _gpu_gradient(lib, torch, c, z, q)
+        again = _gpu_gradient(lib, torch, c, z, q)
+        c.close()
+        assert all(np.array_equal(a, b) for a, b in zip(out, again))
+        return out
+
+    phi, gz, gq = call(slice(None), chunk)
+    parts = [call(slice(k, k + 1), 0) for k in range(n_pos)]
+    want = sum(p[0] for p in parts), sum(p[1] for p in parts), sum(p[2] for p in parts)
+    # FP32 sums of at most 160 terms against FP64 sums of the same terms
+    assert abs(phi - want[0]) <= 1e-6 * want[0]
+    assert rel_err(gz, want[1]) <= 2e-6 and rel_err(gq, want[2]) <= 2e-6
