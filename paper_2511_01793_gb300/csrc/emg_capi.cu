@@ -106,6 +106,7 @@ struct emg_ctx {
   int grad_chunk_req = 0;         // positions per gradient launch asked for (0: automatic)
   int grad_chunk = 0;             // positions per gradient launch in use (0: not chosen yet)
   int grad_slots = 0;             // clusters of a launch, each with a probe-gradient sum
+  int grad_wave = 0;              // positions whose clusters are resident at once (0: unknown)
   float2* d_gz = nullptr;         // [grad_chunk][m][m] when it exceeds the minibatch
   float2* d_gq = nullptr;         // [grad_slots][m][m]
   double* h_scalar = nullptr;     // pinned [64]
@@ -1459,6 +1460,7 @@ emg_status emg_misfit_gradient(emg_ctx* c, const float* object, const float* pro
     }
     c->grad_chunk = chunk;
     c->grad_slots = slots;
+    c->grad_wave = pw;
   }
   const int B = c->grad_chunk;
   float2* gz = c->d_gz ? c->d_gz : c->d_zt;
@@ -1482,7 +1484,7 @@ emg_status emg_misfit_gradient(emg_ctx* c, const float* object, const float* pro
     ga.gz = gz;
     ga.gq = gq;
     ga.phi = c->d_phi + first;
-    cudaError_t e = emg::launch_gradient(c->m, std::min(b, c->grad_slots), ga, c->stream);
+    cudaError_t e = emg::launch_gradient(c->m, std::min(b, c->grad_slots), c->grad_wave, ga, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "k_gradc launch");
     c->launches[kKindOther] += 1;
     emg::GradReduceArgs ra{};

@@ -151,8 +151,8 @@ struct GradReduceArgs {
   int tiles_x, tiles_y;         // set by launch_grad_reduce
 };
 
-// `slots` <= a.b clusters, each with its own probe-gradient sum.
-cudaError_t launch_gradient(int m, int slots, const GradArgs& a, cudaStream_t s);
+// `slots` <= a.b clusters, each with its own probe-gradient sum; `wave` as gradient_positions_per_wave gives it.
+cudaError_t launch_gradient(int m, int slots, int wave, const GradArgs& a, cudaStream_t s);
 // Positions whose gradient clusters are resident on the device at once (0 if unknown).
 int gradient_positions_per_wave(int m);
 // Clusters (and probe-gradient slots) of a launch over `chunk` positions, `wave` of them resident at once.

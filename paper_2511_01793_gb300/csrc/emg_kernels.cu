@@ -1014,10 +1014,10 @@ struct StepTile : CTile<M, C> {
 // simulated positions 54 us against 64 with clusters of 2 and 62 with 4.  m = 256:
 // clusters of 8 with two CTAs per SM 383 us for 1024 positions, of 4 with one 422.
 template <int M> struct WaveCluster { static constexpr int value = M == 256 ? 8 : 1; };
-template <int M>
-struct WaveTile : CTile<M, WaveCluster<M>::value> {
-  using B = CTile<M, WaveCluster<M>::value>;
-  static constexpr int SIDE = M, CTAS = WaveCluster<M>::value;
+template <int M, int C = WaveCluster<M>::value>
+struct WaveTile : CTile<M, C> {
+  using B = CTile<M, C>;
+  static constexpr int SIDE = M, CTAS = C;
   static constexpr bool ONE = true;
   static constexpr int S = B::SR;
   static constexpr size_t slab = (size_t)B::H * S;
@@ -1946,10 +1946,10 @@ __global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_forw
 // hardware then fills each SM as it frees up (1600 positions at m = 256: 1.65
 // ms, one wave 1.75).  us per call before -> after, with the sums: 900 positions
 // at m = 128 244 -> 173, 1444 at m = 64 125 -> 68, 4096 at m = 32 133 -> 64.
-template <int M>
-__global__ void __launch_bounds__(WaveTile<M>::NT, WaveTile<M>::MIN_CTAS) k_gradc(const GradArgs a) {
-  using TL = WaveTile<M>;
-  constexpr int NT = TL::NT, H = TL::H, S = TL::S, N1 = TL::N1, C = TL::CTAS, SLOTS = TL::SLOTS, PER = TL::PER;
+template <int M, int C = WaveCluster<M>::value>
+__global__ void __launch_bounds__(WaveTile<M, C>::NT, WaveTile<M, C>::MIN_CTAS) k_gradc(const GradArgs a) {
+  using TL = WaveTile<M, C>;
+  constexpr int NT = TL::NT, H = TL::H, S = TL::S, N1 = TL::N1, SLOTS = TL::SLOTS, PER = TL::PER;
   cg::cluster_group cl = cg::this_cluster();
   const int rank = C == 1 ? 0 : (int)cl.block_rank();
   extern __shared__ __align__(16) float2 sm[];
@@ -2730,17 +2730,17 @@ cudaError_t launch_forward_t(int count, const FwdArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <int M>
+template <int M, int C = WaveCluster<M>::value>
 constexpr size_t gradc_smem_elems() {
-  return WaveTile<M>::slab + (size_t)WaveTile<M>::H * M / 2;
+  return WaveTile<M, C>::slab + (size_t)WaveTile<M, C>::H * M / 2;
 }
 
-template <int M>
+template <int M, int C = WaveCluster<M>::value>
 cudaError_t launch_gradc_t(int slots, const GradArgs& a, cudaStream_t s) {
-  using TL = WaveTile<M>;
-  constexpr size_t bytes = gradc_smem_elems<M>() * sizeof(float2);
+  using TL = WaveTile<M, C>;
+  constexpr size_t bytes = gradc_smem_elems<M, C>() * sizeof(float2);
   const cudaError_t e =
-      launch_cluster_plain(k_gradc<M>, TL::CTAS, dim3(TL::CTAS * slots), dim3(TL::NT), bytes, s, a);
+      launch_cluster_plain(k_gradc<M, C>, TL::CTAS, dim3(TL::CTAS * slots), dim3(TL::NT), bytes, s, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -2763,9 +2763,9 @@ cudaError_t set_forward_attrs() {
   return set_cluster_smem(k_forward<M, 3>, WaveTile<M>::slab);
 }
 
-template <int M>
+template <int M, int C = WaveCluster<M>::value>
 cudaError_t set_grad_attrs() {
-  return set_cluster_smem(k_gradc<M>, gradc_smem_elems<M>());
+  return set_cluster_smem(k_gradc<M, C>, gradc_smem_elems<M, C>());
 }
 
 // Dynamic shared-memory limits of the cluster kernels (once per device).
@@ -2794,6 +2794,7 @@ cudaError_t set_cluster_attrs() {
   if ((e = set_grad_attrs<32>()) != cudaSuccess) return e;
   if ((e = set_grad_attrs<64>()) != cudaSuccess) return e;
   if ((e = set_grad_attrs<128>()) != cudaSuccess) return e;
+  if ((e = set_grad_attrs<128, 2>()) != cudaSuccess) return e;
   if ((e = set_grad_attrs<256>()) != cudaSuccess) return e;
   return cudaSuccess;
 }
@@ -2971,12 +2972,14 @@ int gradient_positions_per_wave(int m) {
   }
 }
 
-cudaError_t launch_gradient(int m, int slots, const GradArgs& a, cudaStream_t s) {
+cudaError_t launch_gradient(int m, int slots, int wave, const GradArgs& a, cudaStream_t s) {
+  // m = 128 with at most half a wave of positions: clusters of 2, so that they spread over the SMs (us per
+  // call without the misfit, one CTA against 2: 1 position 26.6 / 20.5, 38 30.8 / 22.6, 76 32.8 / 24.7)
   switch (m) {
     case 16: return launch_gradc_t<16>(slots, a, s);
     case 32: return launch_gradc_t<32>(slots, a, s);
     case 64: return launch_gradc_t<64>(slots, a, s);
-    case 128: return launch_gradc_t<128>(slots, a, s);
+    case 128: return 2 * slots <= wave ? launch_gradc_t<128, 2>(slots, a, s) : launch_gradc_t<128>(slots, a, s);
     case 256: return launch_gradc_t<256>(slots, a, s);
     default: return cudaErrorInvalidValue;
   }

@@ -221,10 +221,11 @@ def test_gradient_without_room_for_its_chunk_takes_the_minibatch(lib, torch, m, 
     assert e.value.status == lib.EMG_ENOMEM
 
 
-@pytest.mark.parametrize("n,n_pos,chunk", [(165, 160, 100), (640, 100, 0)])
-def test_gradients_of_small_and_large_objects(lib, torch, n, n_pos, chunk):
-    """m = 128: small objects are summed over smaller tiles.  Repeats bitwise and equals the sum of
-    one-position calls to FP32 rounding."""
+@pytest.mark.parametrize("n,n_pos,chunk", [(165, 160, 100), (640, 100, 0), (640, 100, 70)])
+def test_gradients_of_few_positions_and_small_objects(lib, torch, n, n_pos, chunk):
+    """m = 128: chunks of up to half a wave take clusters of 2, larger ones one CTA per position (100 and a
+    remainder of 60 in one call); small objects are summed over smaller tiles.  Repeats bitwise and equals
+    the sum of one-position calls to FP32 rounding."""
     m = 128
     rng = np.random.default_rng(n + chunk)
     pos = rng.integers(-m // 3, n - m // 2, size=(n_pos, 2)).astype(np.int32)
