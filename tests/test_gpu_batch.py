@@ -332,6 +332,25 @@ def test_fused_probe_prep_with_one_level_waits_for_the_gain(lib, torch, m, cl):
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
 
 
+@pytest.mark.parametrize("m,levels,prolong", [(16, 1, "const"), (16, 2, "bilinear"), (32, 1, "const"), (32, 2, "const"),
+                                              (32, 3, "bilinear"), (32, 4, "bilinear")])
+def test_fused_probe_prep_with_one_cta_per_position(lib, torch, m, levels, prolong):
+    """The default tiling of small probes: single-CTA tickets whose counters grow over the minibatches of
+    an epoch, and (several levels) positions that wait for prep CTAs; bitwise the separate kernel's states."""
+    case = Case(n=2 * m + 40, m=m, side=5, seed=125 + m)
+    p = oracle_params(minibatch=3, levels=levels, prolong=prolong)
+    out = []
+    for fuse in (1, 0):
+        c = make_context(lib, case, p, seed=3)
+        lib.emg_set_cluster(c.ctx, 1)
+        lib.emg_set_prep_fusion(c.ctx, fuse)
+        lib.emg_run_epochs(c.ctx, 4)
+        lib.emg_step_minibatch(c.ctx, [1, 4, 7])
+        out.append(state(c))
+        c.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
 @pytest.mark.parametrize("m,side,b", [(128, 10, 90), (256, 7, 45)])
 def test_fused_probe_prep_over_several_waves(lib, torch, m, side, b):
     """More positions than clusters fit at once: the prep still runs inside the launch (its clusters
