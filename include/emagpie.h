@@ -338,8 +338,11 @@ emg_status emg_shard_apply(emg_ctx* ctx, const int32_t* idx, int32_t b, const fl
  *  object, object_ref  device complex64 [n_rows][n_cols]
  *  probe, probe_ref    device complex64 [m][m]
  *  region              device uint8 [n_rows][n_cols], nonzero = inside; NULL = every pixel
- * Sums run in a fixed order, so the result is bitwise repeatable.  Allocates
+ * Sums run in a fixed order, so the result is bitwise repeatable.  Takes
  * a small scratch buffer (EMG_ENOMEM if that fails) and synchronises `stream`.
+ * The scratch of this call and the next comes from a memory pool of the library
+ * that keeps at most 64 MB per device between calls; emg_destroy of any context
+ * on the device gives them back.
  */
 emg_status emg_aligned_errors(const float* object, const float* object_ref, int32_t n_rows,
                               int32_t n_cols, const float* probe, const float* probe_ref, int32_t m,
@@ -354,7 +357,8 @@ emg_status emg_aligned_errors(const float* object, const float* object_ref, int3
  *  probe_ref  device complex64 [m][m]
  *  pos        device int32 [n_pos][2]
  *  region     device uint8 [n_rows][n_cols], written
- * Allocates n_rows n_cols doubles of scratch and synchronises `stream`.
+ * Takes n_rows n_cols + m^2 doubles of scratch (EMG_ENOMEM if that fails) and
+ * synchronises `stream`.
  */
 emg_status emg_illuminated_region(const float* probe_ref, int32_t m, const int32_t* pos,
                                   int32_t n_pos, int32_t n_rows, int32_t n_cols, double frac,
@@ -442,9 +446,9 @@ emg_status emg_set_cluster(emg_ctx* ctx, int32_t cluster);
 
 /*
  * Where the probe prep of a minibatch runs: 1 (the default) inside the step
- * launch of the cluster kernels, beside the gather and transforms, when the
- * launch fits in one wave of resident clusters; 0 always as its own kernel
- * before the step.  Speed only: the results are identical.  Synchronises.
+ * launch, beside the gather and transforms, when the launch fits in one wave of
+ * resident clusters (m >= 128 with two or more levels: in four); 0 always as its
+ * own kernel before the step.  Speed only: the results are identical.  Synchronises.
  * EMG_EINVAL for other values.
  */
 emg_status emg_set_prep_fusion(emg_ctx* ctx, int32_t enable);

@@ -525,7 +525,6 @@ emg_status enqueue_minibatch(emg_ctx* c, const int32_t* d_idx, int b, double* d_
   sa.joint = c->par.joint;
   sa.verify = c->verify;
   sa.cluster = c->cluster;
-  sa.alpha = c->par.alpha;
   sa.lv = c->lv;
   sa.zt = zt_all + (size_t)s0 * mm;
   sa.qt = qt_all + (size_t)s0 * mm;

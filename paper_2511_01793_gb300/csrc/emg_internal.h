@@ -66,8 +66,7 @@ struct StepArgs {
   int n_rows, n_cols;
   int n_pos, b;                 // positions of the problem and of this minibatch (index checks)
   int levels, prolong, joint, verify;
-  int cluster;                  // CTAs per position: 1 (m <= 32 only), 2, 4 or 8 (m = 256)
-  float alpha;                  // rPIE constant (level-0 gain formed in the cluster step)
+  int cluster;                  // CTAs per position: 1, 2 (m <= 32), 2, 4 (m = 64), 2, 4, 8 (m = 128), 8 (m = 256)
   LevelArrays lv;
   float2* zt;                   // [b][m*m] joint-step object patches z~_k
   float2* qt;                   // [b][m*m] joint-step probes Q~_k

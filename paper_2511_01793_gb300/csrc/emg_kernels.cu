@@ -942,7 +942,8 @@ __global__ void __launch_bounds__(StepThreads<M>::value) k_step(const StepArgs a
 }
 
 // ---------------------------------------------------------------------------
-// One scan position per cluster of C CTAs (m = 64, 128: C = 2; m = 256: C = 8).
+// One scan position per cluster of C CTAs (by default C = 1 for m <= 32, 2 for m = 64, 4 for
+// m = 128, 8 for m = 256; also built: 2 for m <= 32, 4 for m = 64, 2 and 8 for m = 128).
 //
 // CTA `rank` owns patch rows [rank m/C, (rank+1) m/C) for the gather, the row
 // FFT passes, the multigrid passes and the update, and storage columns
@@ -950,8 +951,7 @@ __global__ void __launch_bounds__(StepThreads<M>::value) k_step(const StepArgs a
 // replacement.  The two transposes between row and column slabs go through
 // distributed shared memory; the multigrid up-pass reads the coarse rows
 // adjacent to its slab from the neighbouring ranks (bilinear prolongation).
-// Per CTA the shared memory is one row slab, one column slab and the object
-// slab, so a minibatch of B positions occupies C B SMs.
+// The shared memory of a CTA is StepTile's.
 namespace cg = cooperative_groups;
 
 // Pixels per unrolled group in the update pass of the cluster step kernel.
@@ -983,16 +983,19 @@ struct CTile {
 // multigrid and the update need it.  199 KB per CTA with three slabs leave
 // one CTA of 16 warps per SM and at most 15 clusters of 8 on the device (120
 // SMs); 114 KB let two CTAs share an SM and hide each other's barriers.  An
-// epoch of 4096 positions with minibatches of 256: 8.51 -> 6.93 ms (with the
-// transposes taken into the passes, which alone gives 0.428 -> 0.404 ms for
-// 900 positions at m = 128 with minibatches of 64).
+// epoch of 4096 positions with minibatches of 256, when this was measured: 8.51
+// -> 6.93 ms (with the transposes taken into the passes, which alone gave 0.428 ->
+// 0.404 ms for 900 positions at m = 128 with minibatches of 64); 6.37 and 0.378 ms now.
 template <int M, int C>
 struct StepTile : CTile<M, C> {
   using B = CTile<M, C>;
   static constexpr int SIDE = M, CTAS = C;
   static constexpr bool ONE = M == 256;
   static constexpr int S = B::SR;
-  // CTAs per SM the register budget leaves room for (as many as the shared memory does)
+  // CTAs per SM the register budget leaves room for (as many as the shared memory does).  At m = 64
+  // the cap pays where a minibatch fills the SMs several times over and costs where it does not (1444
+  // positions, C = 2, three levels, us per epoch with it / without: minibatches of 1024 146 / 164, of 64
+  // 343 / 332; two levels, of 256 182 / 187, of 64 with misfit 407 / 406).
   static constexpr int MIN_CTAS = ONE ? 2 : M == 128 ? C / 2 : M == 64 ? 3 * C / 2 : 1;
   static constexpr size_t slab = (size_t)B::H * S;
   // multigrid buffers of every level at which each CTA keeps a row
@@ -3197,7 +3200,6 @@ extern "C" emg_status emg_step_minibatch_noalloc(float* object, int32_t n_rows, 
   sa.prolong = p->prolong;
   sa.joint = p->joint;
   sa.verify = 0;
-  sa.alpha = p->alpha;
   sa.mq = d_mq;
   sa.zt = (float2*)(base + L.zt);
   sa.qt = (float2*)(base + L.qt);

@@ -37,9 +37,10 @@ constexpr int kPosChunk = 512;   // positions staged in shared memory at a time
 
 // Scratch of one call, from a stream-ordered pool of this library (one per
 // device): cudaMalloc and cudaFree cost more than the reductions themselves
-// (about 200 us of a call's 2.7 ms went into them and their synchronisation).
-// The driver orders reuse between streams and threads; the pool keeps at most
-// kScratchKeep bytes between calls and gives them back when a context is destroyed.
+// (512^2 pixels, m = 128, us per call with them / from the pool: region 173 / 79,
+// errors 205 / 89).  The driver orders reuse between streams and threads; the pool
+// keeps at most kScratchKeep bytes between calls and gives them back when a
+// context on the device is destroyed.
 constexpr size_t kScratchKeep = (size_t)64 << 20;
 std::mutex g_scratch_mu;
 cudaMemPool_t g_scratch_pool[256] = {nullptr};
@@ -212,7 +213,8 @@ __global__ void __launch_bounds__(kMetThreads) k_probe_intensity(const float2* _
 // order, into a list, so a pixel walks only those instead of every position;
 // |Q|^2 comes from a table, which leaves one FP64 add per covered pixel and
 // position (the FP64 pipe is the bound: 23 us for 14.7 M of them).  512^2 pixels,
-// 900 positions, m = 128: 2210 us with every position tested at every pixel.
+// 900 positions, m = 128, whole call: 79 us, with every position tested at every
+// pixel 2380.
 constexpr int kIllumRows = 8, kIllumCols = 32, kIllumWarps = kMetThreads / 32;
 __global__ void __launch_bounds__(kMetThreads) k_illumination(const double* __restrict__ p2, int m,
                                                               const int32_t* __restrict__ pos, int n_pos,

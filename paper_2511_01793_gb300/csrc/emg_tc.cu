@@ -961,12 +961,12 @@ __global__ void __launch_bounds__(256) k_tc_rows16(const float2* __restrict__ in
 }
 
 // Grid and tiles per block of k_tc_rows16: grouped only while every SM keeps its eight blocks twice over.
-inline int rows16_group(int n_tiles) {
-  const int g = n_tiles * (256 / kR16Rows) / (152 * 16);
+inline int rows16_group(int n_tiles, int sms) {
+  const int g = n_tiles * (256 / kR16Rows) / (sms * 16);
   return g < 1 ? 1 : g > kR16Group ? kR16Group : g;
 }
-inline int rows16_grid(int n_tiles) {
-  const int g = rows16_group(n_tiles);
+inline int rows16_grid(int n_tiles, int sms) {
+  const int g = rows16_group(n_tiles, sms);
   return (n_tiles + g - 1) / g * (256 / kR16Rows);
 }
 
@@ -1340,8 +1340,8 @@ cudaError_t tc_dft2(TcWork* w, const float2* in, float2* out, int count, int inv
   const size_t n = (size_t)count * m * m;
   const bool r16 = tc_radix16(m);
   if (r16)
-    k_tc_rows16<<<rows16_grid(count), 256, 0, s>>>(in, nullptr, nullptr, nullptr, nullptr, 0, 0, count,
-                                                   rows16_group(count), w->buf[0][0], w->buf[0][1]);
+    k_tc_rows16<<<rows16_grid(count, w->sms), 256, 0, s>>>(in, nullptr, nullptr, nullptr, nullptr, 0, 0, count,
+                                                           rows16_group(count, w->sms), w->buf[0][0], w->buf[0][1]);
   else
     k_tc_split<<<grid_for(n), 256, 0, s>>>(in, w->buf[0][0], w->buf[0][1], n);
   cudaError_t e = cudaGetLastError();
@@ -1383,8 +1383,9 @@ cudaError_t tc_exit_waves(TcWork* w, const TcStepArgs& t, cudaStream_t s) {
   const size_t n = (size_t)t.b * m * m;
   const bool r16 = tc_radix16(m);
   if (r16)
-    k_tc_rows16<<<rows16_grid(t.b), 256, 0, s>>>(nullptr, t.object, t.probe, t.pos, t.order, t.n_rows, t.n_cols, t.b,
-                                                 rows16_group(t.b), w->buf[0][0], w->buf[0][1]);
+    k_tc_rows16<<<rows16_grid(t.b, w->sms), 256, 0, s>>>(nullptr, t.object, t.probe, t.pos, t.order, t.n_rows,
+                                                         t.n_cols, t.b, rows16_group(t.b, w->sms), w->buf[0][0],
+                                                         w->buf[0][1]);
   else
     k_tc_psi<<<grid_for(n), 256, 0, s>>>(t.object, t.probe, t.pos, t.order, t.n_rows, t.n_cols, m, t.b,
                                          w->buf[0][0], w->buf[0][1]);

@@ -116,3 +116,30 @@ def test_illuminated_region_on_odd_tiles_and_long_lists(lib, n_rows, n_cols, m, 
         region = torch.full((n_rows, n_cols), 7, dtype=torch.uint8, device="cuda")
         lib.emg_illuminated_region(qt.data_ptr(), m, pt.data_ptr(), n_pos, n_rows, n_cols, frac, region.data_ptr())
         assert np.array_equal(region.cpu().numpy(), (illum >= frac * illum.max()).astype(np.uint8))
+
+
+def test_scratch_between_quality_calls_is_bounded_and_given_back(lib):
+    """The pool behind the quality calls keeps at most 64 MB, whatever a call took (72 MB here), and
+    destroying a context on the device gives that back."""
+    import torch
+
+    n, m = 3000, 16
+    q = torch.ones((m, m), dtype=torch.complex64, device="cuda")
+    pos = torch.randint(0, n - m, (50, 2), dtype=torch.int32, device="cuda")
+    region = torch.zeros((n, n), dtype=torch.uint8, device="cuda")
+    d = torch.ones((1, m, m), device="cuda")
+
+    def call():
+        lib.emg_illuminated_region(q.data_ptr(), m, pos.data_ptr(), 50, n, n, 0.1, region.data_ptr())
+
+    def destroy_a_context():
+        lib.Context(pos[:1], d, m, m, lib.emg_default_params(), obj=q, probe=q).close()
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    call()
+    before = destroy_a_context()
+    call()
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] <= 68 << 20
+    assert before - destroy_a_context() <= 4 << 20
