@@ -277,6 +277,25 @@ __device__ __forceinline__ float block_max(float v, float* sh) {
   return r;
 }
 
+// Sum over the block of per-thread FP32 partials: FP32 warp trees, then the
+// NT/32 warp sums added in FP64 by one thread in a fixed order; the result is
+// broadcast.  Deterministic; avoids FP64 work in every thread.
+template <int NT>
+__device__ __forceinline__ double block_sum_f(float v, float* shf, double* shd) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) shf[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double r = 0.0;
+#pragma unroll
+    for (int i = 0; i < NT / 32; ++i) r += (double)shf[i];
+    shd[0] = r;
+  }
+  __syncthreads();
+  return shd[0];
+}
+
 // FP64 block sum, broadcast: warp trees, then one warp's tree over the NT/32
 // warp sums.  (The FP64 pipe takes two results per SM and clock: every thread
 // adding all warp sums cost 8 us in a block of 1024.)
@@ -1239,6 +1258,7 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   float2* zbuf = sm + 2 * TL::slab;                           // !ONE: H x M, z_k on my rows (gathered once)
   __shared__ float xf[C];
   __shared__ double xd[C], xd2[C];
+  __shared__ double redd[2];
   __shared__ float redf[NT / 32];
   __shared__ int ticket_sh;
   // Phi_k of small probes: the threads' partials are added in FP64 (few warps, so the FP64
@@ -1807,9 +1827,15 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
   }
   }
   if (a.verify) {
-    warp_partial_sum<Part>(acc_after, sums);
-    __syncthreads();
-    if (tid == 0) cluster_publish<C>(cl, rank, xd2, 0.5 * partials_sum<NT>(sums));
+    double part = 0.0;
+    if constexpr (kSum64) {
+      warp_partial_sum<Part>(acc_after, sums);
+      __syncthreads();
+      if (tid == 0) part = 0.5 * partials_sum<NT>(sums);
+    } else {
+      part = 0.5 * block_sum_f<NT>(acc_after, redf, redd);
+    }
+    if (tid == 0) cluster_publish<C>(cl, rank, xd2, part);
   }
   // With halo rows read from the neighbours (bilinear prolongation, other
   // than two or three levels) a neighbour may still read my coarse rows: no CTA leaves
