@@ -1716,8 +1716,8 @@ __global__ void __launch_bounds__(StepTile<M, C>::NT, StepTile<M, C>::MIN_CTAS) 
                        reinterpret_cast<uintptr_t>(zt) | reinterpret_cast<uintptr_t>(qt)) & 15) == 0;
   // Small probes take the accuracy of correctly rounded roots, as the allocation-free step does: no
   // floor under the squares (an object in units of 1e-9 has |z z+|^2 of 1e-36), and at an exact tie the
-  // principal root.  (An epoch of 100 positions at m = 32, minibatches of 10: 85.5 us, with IEEE roots
-  // and division 107, with one Newton step under the floor 83.8.)
+  // principal root.  (An epoch of 100 positions at m = 32, minibatches of 10: 84 us, with IEEE roots and
+  // division 107.)
   constexpr bool kRounded = M <= 32;
   auto update_pairs = [&](auto multigrid, auto joint) {
     constexpr bool kMg = decltype(multigrid)::value, kJoint = decltype(joint)::value;
